@@ -116,6 +116,8 @@ struct pit_problem {
     int device = 0;
     size_t max_smem = 0;
     int n_sm = 0;  // streaming multiprocessors of the device
+    bool direct_ok = false;  // heat operator whose grids all take the direct solve
+    double direct_dt = 0.0;  // largest step it is used for
     int G = 0;
     long long ntot = 0;
     std::vector<int> levels;      // G*d
@@ -295,12 +297,32 @@ size_t grid_smem_bytes(const pit_problem *P, int prec, int g)
     const GridInfo &I = P->info[g];
     int na = 1;
     for (int i = 0; i < P->desc.d; ++i) na = I.N[i] > na ? I.N[i] : na;
-    return phi_smem_bytes(prec, P->desc.op, P->desc.d, I.n, na);
+    if (prec > PAIR) return direct_smem_bytes(prec, I.n, na, false);
+    return phi_smem_bytes(prec, P->desc.op, I.de, I.n, na);
+}
+
+// Kernel form of a call: the refinements' FP32 solves are direct for the heat
+// operator where every grid allows it, unless
+//   - the caller chose a preconditioner (or none), or caps the iterations so low
+//     that a fixed number of them is what is asked for;
+//   - the tolerance is so loose that CG gets there in an iteration or two, for
+//     less than the direct solve's passes (coarse corrections to 1e-2, whose
+//     size MGRIT's cycle counts depend on);
+//   - the step is so large (dt above the squared extent of an axis, ext: twice
+//     dt) that 1 + dt L is nearly singular in FP32.
+int form_of(const pit_problem *P, const pit_solve_opts &o, double dt, bool ext = false)
+{
+    const int f = prec_form(o.prec);
+    if (!P->direct_ok || o.precond != PIT_PRECOND_DEFAULT || o.maxit < 16 || !(o.rtol <= 1e-4) ||
+        !((ext ? 2.0 : 1.0) * dt <= P->direct_dt))
+        return f;
+    return f == MIXED ? MIXED_D : f == PAIR ? PAIR_D : f;
 }
 
 pit_status plan(pit_problem *P, int prec)
 {
     if (P->planned[prec]) return PIT_OK;
+    if (prec > PAIR && !P->direct_ok) return fail(PIT_ERR_UNSUPPORTED, "no direct solve on this problem");
     if (prec == PAIR && (P->desc.op == PIT_OP_OU || P->desc.op == PIT_OP_LSDE || P->desc.op == PIT_OP_CME))
         return fail(PIT_ERR_UNSUPPORTED, "the pair precision form is implemented for the symmetric operators only");
     std::vector<int> order(P->G);
@@ -317,7 +339,10 @@ pit_status plan(pit_problem *P, int prec)
             continue;
         }
         // (class 1 of the FP32 form runs the refinement form's global-state kernel)
-        const size_t bx = phi_smem_bytes_xg(prec, P->desc.op, P->desc.d, n);
+        int na = 1;
+        for (int i = 0; i < P->desc.d; ++i) na = P->info[g].N[i] > na ? P->info[g].N[i] : na;
+        const size_t bx = prec > PAIR ? direct_smem_bytes(prec, n, na, true)
+                                      : phi_smem_bytes_xg(prec, P->desc.op, P->info[g].de, n);
         if (bx > P->max_smem)
             return fail(PIT_ERR_UNSUPPORTED,
                         "grid %d (%d nodes) needs %zu bytes of shared memory for the on-chip solve in this precision "
@@ -434,6 +459,7 @@ StepArgs make_args(pit_problem *P, const pit_solve_opts &o, const StepCall &c, c
     a.faces = P->d_faces;
     a.op = P->op;
     a.rtol = o.rtol;
+    a.rtol2 = (float)(o.rtol * o.rtol);
     a.maxit = o.maxit;
     a.inner_rtol = (float)o.inner_rtol;
     a.ir_maxit = o.ir_maxit;
@@ -444,7 +470,7 @@ StepArgs make_args(pit_problem *P, const pit_solve_opts &o, const StepCall &c, c
     a.ext = c.ext;
     // (the FP32 form's extrapolated steps keep u_n and U2 in a global slab per
     // item; run_steps and lanes_prime size it before any such launch)
-    a.scr = (c.ext && prec_form(o.prec) == SINGLE) ? (float *)P->w_scr.p : nullptr;
+    a.scr = (c.ext && o.prec == PIT_PREC_FP32) ? (float *)P->w_scr.p : nullptr;
     a.stats = P->d_stats;
     return a;
 }
@@ -547,7 +573,7 @@ pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_op
 pit_status run_steps(pit_problem *P, const pit_solve_opts &o, const StepCall &c, const int *active,
                      const pit_lane *L = nullptr)
 {
-    const int prec = prec_form(o.prec);
+    const int prec = form_of(P, o, c.dt, c.ext != 0);
     TRY(plan(P, prec));
     if (c.nb <= 0 || c.nsteps <= 0) return PIT_OK;
     if (L && !L->planned[prec]) return fail(PIT_ERR_INVALID_ARG, "lane without a launch plan");
@@ -565,7 +591,7 @@ pit_status run_steps(pit_problem *P, const pit_solve_opts &o, const StepCall &c,
                                          "solver of this operator", c.nb, P->ntot);
     // (a lane's workspaces and CTA sizes are prepared before its first launch)
     if (v[NBKT].n > 0 && !L)
-        CU(P->w_xg.ensure(sizeof(double) * P->ntot * (size_t)c.nb * xg_slabs(prec, P->desc.op, P->desc.d)));
+        CU(P->w_xg.ensure(sizeof(double) * P->ntot * (size_t)c.nb * xg_slabs(base_form(prec), P->desc.op, P->desc.d)));
     if (c.ext && prec == SINGLE && !L) CU(P->w_scr.ensure(sizeof(float) * P->ntot * (size_t)c.nb));
     if (c.ext && prec == SINGLE && P->w_scr.bytes < sizeof(float) * P->ntot * (size_t)c.nb)
         return fail(PIT_ERR_INVALID_ARG, "extrapolated FP32 steps without their scratch");
@@ -596,7 +622,8 @@ pit_status run_steps(pit_problem *P, const pit_solve_opts &o, const StepCall &c,
             b.bg = b.xg + (long long)c.nb * P->ntot;
         }
         cudaStream_t sq = fork ? st[q] : st[0];
-        CU(launch_steps(prec, b, P->threads[prec][wide ? 1 : 0][q], v[q].smem, sq, v[q].xg));
+        const int nt = P->threads[prec][wide ? 1 : 0][q];  // (0: a lane's form that was not primed)
+        CU(launch_steps(prec, b, nt ? nt : 128, v[q].smem, sq, v[q].xg));
         count_kernels(P, wide ? 0 : 1);
     }
     if (fork) {
@@ -786,6 +813,17 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
             I.S[i] = s;
             s *= I.N[i];
         }
+        for (int i = 0; i < d; ++i)
+            if (I.N[i] > 1) I.ax[I.de++] = i;
+        if (I.de == 0) I.de = 1;  // one node: axis 0 listed
+        for (int i = 0; i < d; ++i) {
+            I.ih2[i] = 1.0 / (I.h[i] * I.h[i]);
+            if (I.h[i] < I.h[I.fine]) I.fine = i;
+        }
+        double h2 = 1e300;
+        for (int i = 0; i < d; ++i)
+            if (i != I.fine && I.h[i] < h2) h2 = I.h[i];
+        I.fine_pc = I.N[I.fine] >= 3 && 2.0 * I.h[I.fine] <= h2 * (1.0 + 1e-12);
         I.n = (int)n;
         I.off = P->off[g];
         P->off[g + 1] = P->off[g] + n;
@@ -793,6 +831,13 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
         P->coef[g] = (w % 2 ? -1.0 : 1.0) * binomial(d - 1, w);
     }
     P->ntot = P->off[P->G];
+    P->direct_ok = desc->op == PIT_OP_HEAT;
+    for (const GridInfo &I : P->info) P->direct_ok = P->direct_ok && direct_grid(I);
+    P->direct_dt = 1e300;
+    for (int i = 0; i < d; ++i) {
+        const double len = desc->hi[i] - desc->lo[i];
+        P->direct_dt = std::min(P->direct_dt, len * len);
+    }
     memset(&P->op, 0, sizeof(P->op));
     P->op.op = desc->op;
     P->op.d = d;
@@ -851,7 +896,7 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
         CUB(cudaMemcpy(P->d_order, order.data(), sizeof(int) * P->G, cudaMemcpyHostToDevice));
     }
     CUB(dev_malloc(&P->d_masks, sizeof(uint16_t) * P->ntot));
-    CUB(launch_masks(P->d_grids, P->G, d, P->d_masks, P->stream));
+    CUB(launch_masks(P->d_grids, P->G, P->d_masks, P->stream));
     if (desc->op == PIT_OP_VARHEAT) {
         CUB(dev_malloc(&P->d_faces, sizeof(double) * P->ntot * 2 * d));
         CUB(launch_faces(P->d_grids, P->G, P->op, P->d_faces, P->stream));
@@ -1683,7 +1728,7 @@ pit_status lanes_prime(Mg &M, int Nc)
                    {&o->crs, Nc / o->m, M.dt * o->m, o->m}};
     const int n_reps = o->levels == 3 ? 3 : 2;
     for (int r = 0; r < n_reps; ++r) {
-        const int prec = prec_form(reps[r].so->prec);
+        const int prec = form_of(P, *reps[r].so, reps[r].dt);
         TRY(plan(P, prec));
         if (reps[r].nb <= 0) continue;
         StepCall c;
@@ -1692,7 +1737,9 @@ pit_status lanes_prime(Mg &M, int Nc)
         c.nsteps = reps[r].nsteps;
         c.in = P->m_U.d();  // u0 at every C-point
         c.is = nt;
-        if (P->n_cls[prec][1] > 0) CU(P->w_xg.ensure(sizeof(double) * nt * (size_t)Nc * xg_slabs(prec, P->desc.op, P->desc.d)));
+        // (the level-2 solves and the extrapolated steps may fall to the other form)
+        if (P->n_cls[prec][1] > 0 || P->n_cls[base_form(prec)][1] > 0)
+            CU(P->w_xg.ensure(sizeof(double) * nt * (size_t)Nc * xg_slabs(base_form(prec), P->desc.op, P->desc.d)));
         // (lane launches of extrapolated FP32 steps: the sweeps (one state per
         // grid) and, with three levels, the level-1 relaxations (Nc / m states)
         if (prec == SINGLE && (o->coarse == PIT_COARSE_EXTRAP || o->init == 2))
@@ -2280,14 +2327,15 @@ extern "C" pit_status pit_phi_batch_inplace_static(pit_problem_t P, double dt, i
         }
         scratch = g_static_ptr[dev];
     }
-    const int prec = prec_form(opts->prec);
+    // (refused as the Krylov form is, whichever form runs)
+    const int prec = form_of(P, *opts, dt);
     // the launch plan was made when the problem was created; planning here
     // would allocate, so a form without a plan is refused
-    if (!P->planned[prec])
+    if (!P->planned[prec] || !P->planned[base_form(prec)])
         return fail(PIT_ERR_UNSUPPORTED, "precision form %d is not supported on this problem (operator or grid "
                                          "sizes); pit_phi_batch gives the reason",
                     opts->prec);
-    if (P->n_cls[prec][1] > 0)
+    if (P->n_cls[prec][1] > 0 || P->n_cls[base_form(prec)][1] > 0)
         return fail(PIT_ERR_UNSUPPORTED, "this problem has grids whose solver state needs global scratch; "
                                          "pit_phi_batch_inplace_static cannot serve it");
     const bool wide = n_batch >= 8;

@@ -14,13 +14,20 @@ namespace pit {
 
 // One component grid Omega_l (Sec. 2.1.1): N_i = 2^{l_i} - 1 interior nodes per
 // axis, C-order strides S_i with the last axis fastest, mesh width h_i.
+// ax[0..de-1] are the axes with more than one node, ascending (a grid of one
+// node lists axis 0): the others have no interior neighbours, so a stencil
+// only visits the listed ones and keeps the others in its diagonal.
 struct GridInfo {
     long long off;      // packed offset of the grid in a state vector
     int n;              // interior nodes
-    int pad;
+    int de;             // listed axes, 1..d
     int N[PIT_D];
     int S[PIT_D];
     double h[PIT_D];
+    double ih2[PIT_D];  // 1 / h_i^2
+    int ax[PIT_D];
+    int fine;           // finest axis (the first of the finest), for the heat line preconditioner
+    int fine_pc;        // it has at least three nodes and is at least twice as fine as every other axis
 };
 
 struct OpParams {
@@ -110,7 +117,7 @@ struct DevStats {
 struct StepArgs {
     int item0;              // first item of this launch (launches may be split in chunks)
     const GridInfo *grids;
-    const uint16_t *masks;  // neighbour mask of every node, packed like a state
+    const uint16_t *masks;  // neighbour mask of every node over its grid's listed axes, packed like a state
     const int *order;       // the launch's grids, by decreasing size
     int n_order;            // grids in order
     int n_grids;            // all grids of the problem (row length of norms)
@@ -141,6 +148,7 @@ struct StepArgs {
     const double *faces;     // variable coefficient at the 2d faces of every node, or NULL
     OpParams op;
     double rtol;
+    float rtol2;             // rtol^2
     int maxit;
     float inner_rtol;
     int ir_maxit;
@@ -157,8 +165,11 @@ struct StepArgs {
 // Krylov in FP64 refinement, SINGLE = FP32 Krylov on a power-of-two-scaled
 // FP32 copy of the state (FP64 input and output), PAIR = FP32 Krylov in a
 // refinement whose state and residual are FP32 pairs (symmetric operators).
-enum Prec { PLAIN = 0, MIXED = 1, SINGLE = 2, PAIR = 3 };
-constexpr int NPREC = 4;
+// The _D forms are the refinements with a direct FP32 solve in place of the
+// Krylov solve (heat operator, pit_direct.cuh).
+enum Prec { PLAIN = 0, MIXED = 1, SINGLE = 2, PAIR = 3, MIXED_D = 4, PAIR_D = 5 };
+constexpr int NPREC = 6;
+inline int base_form(int prec) { return prec == MIXED_D ? MIXED : prec == PAIR_D ? PAIR : prec; }
 // Launch parts of one multi-step call: NBKT shared-memory buckets of the
 // grids whose state fits on chip, then the grids with global-memory state.
 constexpr int NBKT = 4;
@@ -198,9 +209,10 @@ cudaError_t launch_net_adam(const float *grad_rows, int n_rows, float scale, flo
                             float *w_bf16, float lr, float b1, float b2, float eps, int t, float *grad_out,
                             cudaStream_t s);
 
-// Shared-memory bytes a backward-Euler item of n nodes needs.
-// (na: nodes of the grid's longest axis, for the heat line preconditioner)
-size_t phi_smem_bytes(int prec, int op, int d, int n, int na);
+// Shared-memory bytes a backward-Euler item of n nodes on a grid of de listed
+// axes needs (na: nodes of the grid's longest axis, for the heat line
+// preconditioner)
+size_t phi_smem_bytes(int prec, int op, int de, int n, int na);
 // Launch one multi-step batch (grid-per-CTA, every Krylov solve on chip);
 // xg selects the variant whose FP64 state lives in global memory.
 cudaError_t launch_steps(int prec, const StepArgs &a, int threads, size_t smem, cudaStream_t s, bool xg = false);
@@ -208,12 +220,18 @@ cudaError_t launch_steps(int prec, const StepArgs &a, int threads, size_t smem, 
 // the number of n_batch x n_total FP64 slabs of global workspace it uses
 // (x, b and the carried x - A x for MIXED; x and the Krylov vectors for
 // PLAIN).
-size_t phi_smem_bytes_xg(int prec, int op, int d, int n);
+size_t phi_smem_bytes_xg(int prec, int op, int de, int n);
+// The same of the direct forms (na: nodes of the longest axis; xg: the variant
+// whose FP64 state lives in global memory).
+size_t direct_smem_bytes(int prec, int n, int na, bool xg);
+// Whether a grid's axes but the longest are short enough for the direct solve.
+bool direct_grid(const GridInfo &G);
 int xg_slabs(int prec, int op, int d);
 // Raise the dynamic shared-memory limit of every backward-Euler kernel.
 cudaError_t phi_kernels_init(size_t max_smem);
-// Neighbour masks of every node (bit 2i: interior neighbour at -e_i, 2i+1: at +e_i).
-cudaError_t launch_masks(const GridInfo *grids, int G, int d, uint16_t *masks, cudaStream_t s);
+// Neighbour masks of every node (bit 2q: interior neighbour at -e_i, 2q+1: at
+// +e_i, i = ax[q] the grid's listed axes).
+cudaError_t launch_masks(const GridInfo *grids, int G, uint16_t *masks, cudaStream_t s);
 
 cudaError_t launch_apply(const GridInfo *grids, int G, long long ntot, int n_batch, double dt,
                          const double *p, double *q, const double *faces, OpParams op, cudaStream_t s);

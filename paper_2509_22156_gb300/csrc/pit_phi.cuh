@@ -73,25 +73,39 @@ namespace pit {
 //   CME     toggle-switch chemical master equation (Sec. 4.3): the same
 //           flux with face velocity a_i - g_i x_i (production a_i, degradation
 //           g_i x_i) and the second difference of (a_i + g_i x_i) p / 2.
-template <int D>
-__device__ __forceinline__ void op_coef(const OpParams &op, const GridInfo &G, const double *faces, int j,
-                                        double dt, double &diag, double *cm, double *cp)
+// axis(q, i, cm, cp) receives the couplings of the listed axis i = ax[q]; the
+// diagonal, which every axis contributes to, is returned.  (Run once per node
+// and launch, so the axes are a run-time loop.)
+struct NodeCoord {
+    const OpParams &op;
+    const GridInfo &G;
+    int j;
+    __device__ __forceinline__ double operator[](int k) const
+    {
+        return op.lo[k] + (double)((j / G.S[k]) % G.N[k] + 1) * G.h[k];
+    }
+};
+template <int OP, class F>
+__device__ __forceinline__ double op_coef(const OpParams &op, const GridInfo &G, const double *faces, int j, double dt,
+                                          F &&axis)
 {
-    diag = 1.0;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-        const int c = (j / G.S[i]) % G.N[i];
+    const int d = op.d;
+    const NodeCoord xc{op, G, j};
+    double diag = 1.0;
+    int q = 0;
+#pragma unroll 1
+    for (int i = 0; i < d; ++i) {
         const double h = G.h[i];
-        const double ih2 = 1.0 / (h * h);
+        const double ih2 = G.ih2[i];
         double dd, dm, dp;
-        if (op.op == PIT_OP_HEAT) {
+        if constexpr (OP == PIT_OP_HEAT) {
             dd = 2.0 * ih2; dm = -ih2; dp = -ih2;
-        } else if (op.op == PIT_OP_VARHEAT) {
-            const double am = faces[(G.off + j) * (2 * D) + 2 * i];
-            const double ap = faces[(G.off + j) * (2 * D) + 2 * i + 1];
+        } else if constexpr (OP == PIT_OP_VARHEAT) {
+            const double am = faces[(G.off + j) * (2 * d) + 2 * i];
+            const double ap = faces[(G.off + j) * (2 * d) + 2 * i + 1];
             dd = (am + ap) * ih2; dm = -am * ih2; dp = -ap * ih2;
-        } else if (op.op == PIT_OP_OU) {
-            const double x = op.lo[i] + (double)(c + 1) * h;
+        } else if constexpr (OP == PIT_OP_OU) {
+            const double x = xc[i];
             const double vp = -op.theta * (x + 0.5 * h);
             const double vm = -op.theta * (x - 0.5 * h);
             const double s2 = 0.5 * op.sigma * op.sigma * ih2;
@@ -99,32 +113,35 @@ __device__ __forceinline__ void op_coef(const OpParams &op, const GridInfo &G, c
             dd += 2.0 * s2;
             dm -= s2;
             dp -= s2;
-        } else if (op.op == PIT_OP_CME) {
-            double xc[D];
-#pragma unroll
-            for (int k = 0; k < D; ++k) xc[k] = op.lo[k] + (double)((j / G.S[k]) % G.N[k] + 1) * G.h[k];
-            cme_coef(cme_production(op, i, xc, D), op.cg[i], xc[i], h, op.central != 0, dd, dm, dp);
+        } else if constexpr (OP == PIT_OP_CME) {
+            cme_coef(cme_production(op, i, xc, d), op.cg[i], xc[i], h, op.central != 0, dd, dm, dp);
         } else {
             // face velocities (A x)_i at x -+ h/2 e_i
             double ax = 0.0;
-#pragma unroll
-            for (int k = 0; k < D; ++k) ax += op.A[i * D + k] * (op.lo[k] + (double)((j / G.S[k]) % G.N[k] + 1) * G.h[k]);
-            const double vp = ax + 0.5 * h * op.A[i * D + i];
-            const double vm = ax - 0.5 * h * op.A[i * D + i];
-            const double s2 = 0.5 * op.H[i * D + i] * ih2;
+            for (int k = 0; k < d; ++k) ax += op.A[i * d + k] * xc[k];
+            const double vp = ax + 0.5 * h * op.A[i * d + i];
+            const double vm = ax - 0.5 * h * op.A[i * d + i];
+            const double s2 = 0.5 * op.H[i * d + i] * ih2;
             drift_coef(vp, vm, h, op.central != 0, dd, dm, dp);
             dd += 2.0 * s2;
             dm -= s2;
             dp -= s2;
         }
         diag += dt * dd;
-        cm[i] = (c > 0) ? dt * dm : 0.0;
-        cp[i] = (c < G.N[i] - 1) ? dt * dp : 0.0;
+        if (q < G.de && G.ax[q] == i) {
+            const int c = (j / G.S[i]) % G.N[i];
+            axis(q, i, (c > 0) ? dt * dm : 0.0, (c < G.N[i] - 1) ? dt * dp : 0.0);
+            ++q;
+        }
     }
+    return diag;
 }
 
 // Constant-coefficient heat stencil with a per-node neighbour mask
-// (bit 2i: interior neighbour at -e_i, bit 2i+1: at +e_i).
+// (bit 2i: interior neighbour at -e_i, bit 2i+1: at +e_i).  Here and in the
+// other stencils D counts the grid's listed axes (GridInfo::ax), not the
+// problem's: a third of the axes of the d = 6, level-10 grid set have one
+// node, whose neighbours are zeros the FP64 pipe would add and multiply.
 template <typename T, int D>
 struct HeatSt {
     const uint16_t *mask;
@@ -173,6 +190,7 @@ struct TabSt {
     int ld;
     int S[D];
     T cr[NP > 0 ? NP : 1];
+    bool mixed = false;  // some cr is not zero (else the diagonal neighbours are not read)
     bool unit = false;  // Jacobi-scaled table: unit diagonal, the diagonal slot holds D^{-1/2}
     __device__ __forceinline__ T operator()(const T *p, int j) const
     {
@@ -184,7 +202,8 @@ struct TabSt {
             const int jp = ((mk >> (2 * i + 1)) & 1u) ? j + S[i] : j;
             s += tab[(1 + 2 * i) * ld + j] * p[jm] + tab[(2 + 2 * i) * ld + j] * p[jp];
         }
-        if constexpr (CROSS && NP > 0) s += cross(p, j, mk);
+        if constexpr (CROSS && NP > 0)
+            if (mixed) s += cross(p, j, mk);
         return s;
     }
     __device__ __forceinline__ T cross(const T *p, int j, unsigned mk) const
@@ -219,7 +238,8 @@ struct TabSt {
             s = fma(-tab[(1 + 2 * i) * ld + j], p[jm], s);
             s = fma(-tab[(2 + 2 * i) * ld + j], p[jp], s);
         }
-        if constexpr (CROSS && NP > 0) s -= cross(p, j, mk);
+        if constexpr (CROSS && NP > 0)
+            if (mixed) s -= cross(p, j, mk);
         return s;
     }
 };
@@ -402,12 +422,14 @@ __device__ __forceinline__ float2 pair_add(float2 x, float2 y)
 // below about 2^-48 (|x_j| + sum_i c_i (2 |x_j| + |x_m| + |x_p|)) (the FP64
 // residual's bound with 2^-48 for 2^-53): far below the 1e-11 relative
 // residuals the refinement asks for unless dt / h^2 reaches the hundreds.
-// Also yields x_j - b_j rounded to FP32.
+// Also yields x_j - b_j rounded to FP32.  The axes that are not listed have
+// zero neighbours: together they add (sum of 2 c_i) x_j, rh + rl as a pair.
 template <int D>
 struct PairHeat {
     const uint16_t *mask;
     int S[D];
     float ch[D], cl[D];
+    float rh = 0.0f, rl = 0.0f;
     __device__ __forceinline__ float operator()(const float2 *x, const float2 *bv, int j, float &xmb) const
     {
         const unsigned mk = mask[j];
@@ -430,6 +452,13 @@ struct PairHeat {
             two_sum(s, -p, s, e4);
             comp = comp + (e4 - q);
         }
+        if (rh != 0.0f) {
+            float e4;
+            const float p = __fmul_rn(rh, xj.x);
+            const float q = __fmaf_rn(rh, xj.x, -p) + (rh * xj.y + rl * xj.x);
+            two_sum(s, -p, s, e4);
+            comp = comp + (e4 - q);
+        }
         return __fadd_rn(s, comp);
     }
 };
@@ -438,13 +467,15 @@ struct PairHeat {
 // coefficients c = dt a / h_i^2 of every node held as pairs (zero neighbours
 // towards the boundary, whose face coefficient still counts):
 //     A x = x + sum_i c_{j-e_i/2} (x_j - x_{j-e_i}) + c_{j+e_i/2} (x_j - x_{j+e_i}).
-// Table layout: c[(2 i) ld + j] towards -e_i, c[(2 i + 1) ld + j] towards +e_i.
+// Table layout: c[(2 i) ld + j] towards -e_i, c[(2 i + 1) ld + j] towards +e_i;
+// c[2 D ld + j] the sum over the faces of the axes that are not listed (rest).
 template <int D>
 struct PairTab {
     const uint16_t *mask;
     const float2 *c;
     int ld;
     int S[D];
+    bool rest = false;
     __device__ __forceinline__ float operator()(const float2 *x, const float2 *bv, int j, float &xmb) const
     {
         const unsigned mk = mask[j];
@@ -469,9 +500,80 @@ struct PairTab {
                 comp = comp + (e2 - q);
             }
         }
+        if (rest) {
+            const float2 cf = c[2 * D * ld + j];
+            float e2;
+            const float p = __fmul_rn(cf.x, xj.x);
+            const float q = __fmaf_rn(cf.x, xj.x, -p) + (cf.x * xj.y + cf.y * xj.x);
+            two_sum(s, -p, s, e2);
+            comp = comp + (e2 - q);
+        }
         return __fadd_rn(s, comp);
     }
 };
+
+// FP32 value times 2^k (exact unless it leaves the FP32 range)
+__device__ __forceinline__ float scale_f(float v, int k)
+{
+    const int k1 = min(max(k, -252), 252), ka = k1 / 2, kb = k1 - ka;
+    return (v * __uint_as_float((unsigned)(127 + ka) << 23)) * __uint_as_float((unsigned)(127 + kb) << 23);
+}
+// k with v 4^k in [1, 4) for a normal FP32 v > 0 (a sum of squares); 0 for 0,
+// infinity and NaN, 64 for a subnormal v
+__device__ __forceinline__ int scale_exp(float v)
+{
+    const int eb = (int)((__float_as_uint(v) >> 23) & 0xffu);
+    if (eb == 0 || eb == 255) return eb == 0 && v != 0.0f ? 64 : 0;
+    return -((eb - 127) >> 1);  // (arithmetic shift: floor)
+}
+
+// Constants of one item's stencils, worked out by a few lanes of the first
+// warp: an FP64 instruction occupies the SM's FP64 unit for as long as a whole
+// warp of nodes, whichever thread asks for it, so values that are the same for
+// the whole block are computed once.
+struct ItemConst {
+    double diag, off[PIT_D], cr[PIT_D * (PIT_D - 1) / 2];
+    float diag32, off32[PIT_D], cr32[PIT_D * (PIT_D - 1) / 2];
+    float ch[PIT_D], cl[PIT_D], rh, rl;  // dt / h^2 of the listed axes, 2 dt sum 1 / h^2 of the others, as FP32 pairs
+    float offf;                          // coupling along the finest axis
+    int use_pc;                          // the line preconditioner is worth it at this step size
+};
+__device__ __forceinline__ void item_const(const StepArgs &a, const GridInfo &G, ItemConst &C)
+{
+    const int t = threadIdx.x, D = G.de, d = a.op.d;
+    if (t < D) {
+        const double c = a.dt * G.ih2[G.ax[t]];
+        C.off[t] = -c;
+        C.off32[t] = (float)-c;
+        C.ch[t] = to_f32(c, 0);
+        C.cl[t] = to_f32(c - to_f64(C.ch[t], 0), 0);
+    } else if (t == 8) {
+        double diag = 1.0;
+        for (int i = 0; i < d; ++i) diag += 2.0 * a.dt * G.ih2[i];
+        C.diag = diag;
+        C.diag32 = (float)diag;
+    } else if (t == 9) {
+        double rest = 0.0;
+        for (int i = 0; i < d; ++i)
+            if (G.N[i] == 1 && i != G.ax[0]) rest += 2.0 * a.dt * G.ih2[i];
+        C.rh = to_f32(rest, 0);
+        C.rl = to_f32(rest - to_f64(C.rh, 0), 0);
+    } else if (t == 10) {
+        const double c = a.dt * G.ih2[G.fine];
+        C.offf = (float)-c;
+        C.use_pc = G.fine_pc && 4.0 * c >= 2.0;
+    } else if (t >= 16 && t < 16 + D * (D - 1) / 2) {
+        int q = 16, i = 0, k = 1;  // pair (i, k), i < k, number t - 16
+        while (q < t) {
+            if (++k == D) k = ++i + 1;
+            ++q;
+        }
+        const int ai = G.ax[i], ak = G.ax[k];
+        const double c = -a.dt * 0.5 * (a.op.H[ai * d + ak] + a.op.H[ak * d + ai]) / (4.0 * G.h[ai] * G.h[ak]);
+        C.cr[t - 16] = c;
+        C.cr32[t - 16] = (float)c;
+    }
+}
 
 __device__ __forceinline__ bool finite_pos(double v) { return v > 0.0 && v < 1.0e300; }
 __device__ __forceinline__ bool finite_pos(float v) { return v > 0.0f && v < 1.0e37f; }
@@ -481,13 +583,15 @@ __device__ __forceinline__ bool finite_pos(float v) { return v > 0.0f && v < 1.0
 // on entry (own nodes written by the caller), the iterate is accumulated into
 // X (FP64 state or FP32 correction).  Stops when (r,r) <= stop2, tested on
 // the sum of the update pass before the stencil pass of the next iteration.
-template <typename T, typename TX, class ST>
+// ZX: the iterate starts from zero (the first iteration writes X; with no
+// iteration X stays as it was).  r_ready: a barrier since r was written.
+template <bool ZX, typename T, typename TX, class ST>
 __device__ int cg_core(const ST &A, int n, TX *X, T *r, T *p, T *s, T *w, Reducer<T> &R, T stop2, int maxit,
-                       int &status)
+                       int &status, bool r_ready = false)
 {
     const int tid = threadIdx.x, nt = blockDim.x;
     status = PIT_OK;
-    __syncthreads();  // r complete
+    if (!r_ready) __syncthreads();  // r complete
     T v[2] = {T(0), T(0)};
 #pragma unroll 4
     for (int j = tid; j < n; j += nt) {
@@ -521,7 +625,7 @@ __device__ int cg_core(const ST &A, int n, TX *X, T *r, T *p, T *s, T *w, Reduce
             const T sj = first ? w[j] : w[j] + beta * s[j];
             p[j] = pj;
             s[j] = sj;
-            X[j] += (TX)(alpha * pj);
+            X[j] = (ZX && first) ? (TX)(alpha * pj) : X[j] + (TX)(alpha * pj);
             const T rj = r[j] - alpha * sj;
             r[j] = rj;
             rr[0] += rj * rj;
@@ -737,13 +841,13 @@ struct LineM {
 // then M, then the stencil pass sums (r,u) and (Au,u) (second reduction); a
 // converged iteration skips M and the stencil.  Stops when (r,r) <= stop2
 // (unpreconditioned norm, the same test as cg_core).
-template <typename T, typename TX, class ST, class PC>
+template <bool ZX, typename T, typename TX, class ST, class PC>
 __device__ int pcg_core(const ST &A, const PC &M, int n, TX *X, T *r, T *u, T *p, T *s, T *w, Reducer<T> &R,
-                        T stop2, int maxit, int &status)
+                        T stop2, int maxit, int &status, bool r_ready = false)
 {
     const int tid = threadIdx.x, nt = blockDim.x;
     status = PIT_OK;
-    __syncthreads();  // r complete
+    if (!r_ready) __syncthreads();  // r complete
     M(r, u);
     __syncthreads();  // u complete
     T v[3] = {T(0), T(0), T(0)};
@@ -779,7 +883,7 @@ __device__ int pcg_core(const ST &A, const PC &M, int n, TX *X, T *r, T *u, T *p
             const T sj = first ? w[j] : w[j] + beta * s[j];
             p[j] = pj;
             s[j] = sj;
-            X[j] += (TX)(alpha * pj);
+            X[j] = (ZX && first) ? (TX)(alpha * pj) : X[j] + (TX)(alpha * pj);
             const T rj = r[j] - alpha * sj;
             r[j] = rj;
             rr[0] += rj * rj;
@@ -822,7 +926,8 @@ __device__ int pcg_core(const ST &A, const PC &M, int n, TX *X, T *r, T *u, T *p
 // progress is reported.  Strongly non-normal systems (the central drift flux
 // at large dt |v| / h) lose the shadow residual's orthogonality every few
 // tens of iterations and need this.
-template <typename T, typename TX, class ST>
+// (ZX as for cg_core)
+template <bool ZX, typename T, typename TX, class ST>
 __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v, T *t, Reducer<T> &R, T stop2,
                              int maxit, int &status)
 {
@@ -915,7 +1020,8 @@ __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v,
         T rn[1] = {T(0)};
 #pragma unroll 4
         for (int j = tid; j < n; j += nt) {
-            X[j] += (TX)(alpha * p[j] + omega * r[j]);
+            const TX dx = (TX)(alpha * p[j] + omega * r[j]);
+            X[j] = (ZX && k == 0) ? dx : X[j] + dx;
             const T rj = r[j] - omega * t[j];
             r[j] = rj;
             rn[0] += rj * rj;
@@ -957,6 +1063,7 @@ __host__ __device__ inline int line_pc_bytes(int op, int prec, bool xg, int na)
     return line_pc_form(op, prec, xg) ? 4 * (6 * na + 3 * 33 + 8) + 16 : 0;
 }
 
+// (d: the grid's listed axes)
 __host__ __device__ inline int n_tab(int op, int d) { return op == PIT_OP_HEAT ? 0 : 2 * d + 1; }
 // (MIXED keeps a third FP64 array, the carried x - A x of the last step;
 // its global-state variant keeps it in global memory with x and b)
@@ -971,28 +1078,16 @@ __host__ __device__ inline int n_f32(int op, int prec, int d, bool xg = false)
     return krylov_vecs(op, prec, xg) + n_tab(op, d);
 }
 
-template <int OP, int PREC, int D, bool XG = false>
-__global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
+// One item on a grid of D listed axes (all threads of the block).
+template <int OP, int PREC, int D, bool XG>
+__device__ __forceinline__ void steps_item(const StepArgs &a, const GridInfo &GI, const ItemConst &IC, int g, int b,
+                                           double *red64, float *red32)
 {
     typedef typename std::conditional<PREC == PLAIN, double, float>::type T;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ GridInfo GI;
-    __shared__ double red64[2 * 128];
-    __shared__ float red32[2 * 128];
 
-    static_assert(!XG || PREC != SINGLE, "no global-state variant of the FP32 form");
-    static_assert(PREC == PLAIN || PREC == MIXED || PREC == SINGLE || PREC == PAIR, "unknown precision form");
-    static_assert(PREC != PAIR || (OP != PIT_OP_OU && OP != PIT_OP_LSDE && OP != PIT_OP_CME),
-                  "the pair form is for the symmetric operators");
     constexpr bool DRIFT = (OP == PIT_OP_OU || OP == PIT_OP_LSDE || OP == PIT_OP_CME);  // non-symmetric: BiCGStab
     constexpr bool CROSS = (OP == PIT_OP_LSDE);                      // mixed-derivative terms
-    const int item = a.item0 + (int)blockIdx.x;
-    const int g = a.order[item / a.n_batch];
-    const int b = item % a.n_batch;
-    if (a.active && !a.active[g]) return;  // uniform over the block
-    if (threadIdx.x == 0) GI = a.grids[g];
-    __syncthreads();
-
     const int tid = threadIdx.x, nt = blockDim.x;
     const int n = GI.n;
     const int ld = (n + 3) & ~3;
@@ -1057,30 +1152,38 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
     }
     if constexpr (OP != PIT_OP_HEAT) {
         for (int j = tid; j < n; j += nt) {
-            double diag, cm[D], cp[D];
-            op_coef<D>(a.op, GI, a.faces, j, dt, diag, cm, cp);
-            if constexpr (PREC != SINGLE && PREC != PAIR) tab64[j] = diag;
-            if constexpr (PREC != PLAIN) tab32[j] = (float)diag;
-#pragma unroll
-            for (int i = 0; i < D; ++i) {
+            const double diag = op_coef<OP>(a.op, GI, a.faces, j, dt, [&](int q, int i, double cm, double cp) {
                 if constexpr (PREC != SINGLE && PREC != PAIR) {
-                    tab64[(1 + 2 * i) * tld + j] = cm[i];
-                    tab64[(2 + 2 * i) * tld + j] = cp[i];
+                    tab64[(1 + 2 * q) * tld + j] = cm;
+                    tab64[(2 + 2 * q) * tld + j] = cp;
                 }
                 if constexpr (PREC == PAIR) {
                     // face coefficients dt a / h^2 as pairs, in the FP64 table's place
                     float2 *cpair = reinterpret_cast<float2 *>(tab64);
-                    const double ih2 = 1.0 / (GI.h[i] * GI.h[i]);
-                    const double am = a.faces[(GI.off + j) * (2 * D) + 2 * i];
-                    const double ap = a.faces[(GI.off + j) * (2 * D) + 2 * i + 1];
-                    cpair[(2 * i) * ld + j] = split_pair(dt * am * ih2, 0);
-                    cpair[(2 * i + 1) * ld + j] = split_pair(dt * ap * ih2, 0);
+                    const double ih2 = GI.ih2[i];
+                    const double am = a.faces[(GI.off + j) * (2 * a.op.d) + 2 * i];
+                    const double ap = a.faces[(GI.off + j) * (2 * a.op.d) + 2 * i + 1];
+                    cpair[(2 * q) * ld + j] = split_pair(dt * am * ih2, 0);
+                    cpair[(2 * q + 1) * ld + j] = split_pair(dt * ap * ih2, 0);
                 }
                 if constexpr (PREC != PLAIN) {
-                    tab32[(1 + 2 * i) * ld + j] = (float)cm[i];
-                    tab32[(2 + 2 * i) * ld + j] = (float)cp[i];
+                    tab32[(1 + 2 * q) * ld + j] = (float)cm;
+                    tab32[(2 + 2 * q) * ld + j] = (float)cp;
+                }
+            });
+            if constexpr (PREC != SINGLE && PREC != PAIR) tab64[j] = diag;
+            if constexpr (PREC == PAIR) {
+                // faces of the axes that are not listed (on one node, of all but axis 0)
+                if (D < a.op.d) {
+                    double rest = 0.0;
+                    for (int i = 0; i < a.op.d; ++i)
+                        if (GI.N[i] == 1 && i != GI.ax[0])
+                            rest += dt * (a.faces[(GI.off + j) * (2 * a.op.d) + 2 * i] +
+                                          a.faces[(GI.off + j) * (2 * a.op.d) + 2 * i + 1]) * GI.ih2[i];
+                    reinterpret_cast<float2 *>(tab64)[2 * D * ld + j] = split_pair(rest, 0);
                 }
             }
+            if constexpr (PREC != PLAIN) tab32[j] = (float)diag;
         }
     }
     // stencils in FP64 and in the working precision
@@ -1094,29 +1197,25 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
     T64.ld = tld;
     T32.ld = ld;
     if constexpr (CROSS) {
-        int q = 0;
+        bool any = false;
 #pragma unroll
-        for (int i = 0; i < D; ++i)
-#pragma unroll
-            for (int k = i + 1; k < D; ++k, ++q) {
-                const double c = -dt * 0.5 * (a.op.H[i * D + k] + a.op.H[k * D + i]) / (4.0 * GI.h[i] * GI.h[k]);
-                T64.cr[q] = c;
-                T32.cr[q] = (float)c;
-            }
-    }
-    {
-        double diag = 1.0;
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            const double ih2 = 1.0 / (GI.h[i] * GI.h[i]);
-            H64.S[i] = HT.S[i] = T64.S[i] = T32.S[i] = GI.S[i];
-            H64.off[i] = -dt * ih2;
-            HT.off[i] = (T)(-dt * ih2);
-            diag += 2.0 * dt * ih2;
+        for (int q = 0; q < D * (D - 1) / 2; ++q) {
+            T64.cr[q] = IC.cr[q];
+            T32.cr[q] = IC.cr32[q];
+            any = any || IC.cr32[q] != 0.0f || __double2hiint(IC.cr[q]) != 0;
         }
-        H64.diag = diag;
-        HT.diag = (T)diag;
+        T64.mixed = T32.mixed = any;
     }
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        H64.S[i] = HT.S[i] = T64.S[i] = T32.S[i] = GI.S[GI.ax[i]];
+        H64.off[i] = IC.off[i];
+        if constexpr (PREC == PLAIN) HT.off[i] = IC.off[i];
+        else HT.off[i] = IC.off32[i];
+    }
+    H64.diag = IC.diag;
+    if constexpr (PREC == PLAIN) HT.diag = IC.diag;
+    else HT.diag = IC.diag32;
     // Jacobi preconditioning of the FP32 correction solves (table operators
     // without mixed-derivative terms, refinement forms): the FP32 system is
     // scaled symmetrically, D^{-1/2} A D^{-1/2} y = D^{-1/2} r, e = D^{-1/2} y,
@@ -1132,8 +1231,8 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
                 const float dj = tab32[j];
 #pragma unroll
                 for (int i = 0; i < D; ++i) {
-                    if ((mk >> (2 * i)) & 1u) tab32[(1 + 2 * i) * ld + j] *= rsqrtf(dj * tab32[j - GI.S[i]]);
-                    if ((mk >> (2 * i + 1)) & 1u) tab32[(2 + 2 * i) * ld + j] *= rsqrtf(dj * tab32[j + GI.S[i]]);
+                    if ((mk >> (2 * i)) & 1u) tab32[(1 + 2 * i) * ld + j] *= rsqrtf(dj * tab32[j - T32.S[i]]);
+                    if ((mk >> (2 * i + 1)) & 1u) tab32[(2 + 2 * i) * ld + j] *= rsqrtf(dj * tab32[j + T32.S[i]]);
                 }
             }
             __syncthreads();  // every off-diagonal scaled with the old diagonals
@@ -1146,19 +1245,21 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
         PT.mask = mask;
         PT.c = reinterpret_cast<const float2 *>(tab64);
         PT.ld = ld;
+        PT.rest = D < a.op.d;
 #pragma unroll
-        for (int i = 0; i < D; ++i) PT.S[i] = GI.S[i];
+        for (int i = 0; i < D; ++i) PT.S[i] = GI.S[GI.ax[i]];
     }
     PairHeat<D> PH;
     if constexpr (PREC == PAIR && OP == PIT_OP_HEAT) {
         PH.mask = mask;
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            const double c = dt / (GI.h[i] * GI.h[i]);
-            PH.S[i] = GI.S[i];
-            PH.ch[i] = to_f32(c, 0);
-            PH.cl[i] = to_f32(c - to_f64(PH.ch[i], 0), 0);
+            PH.S[i] = GI.S[GI.ax[i]];
+            PH.ch[i] = IC.ch[i];
+            PH.cl[i] = IC.cl[i];
         }
+        PH.rh = IC.rh;
+        PH.rl = IC.rl;
     }
     // Line preconditioner (heat, FP32 Krylov, state on chip) along the finest
     // axis a, used when a is at least twice as fine as every other axis and
@@ -1170,32 +1271,13 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
     bool use_pc = false;
     LineM<float> LM{};
     if constexpr (OP == PIT_OP_HEAT && PREC != PLAIN && !XG) {
-        // (every per-axis value is read with a compile-time index, so that
-        // the grid description and the stencil stay in registers)
-        int ax = 0, Na = 0, Sa = 0;
-        double ha = 1e300;
-        float offa = 0.0f;
-#pragma unroll
-        for (int i = 0; i < D; ++i)
-            if (GI.h[i] < ha) {
-                ax = i;
-                ha = GI.h[i];
-                Na = GI.N[i];
-                Sa = GI.S[i];
-                offa = HT.off[i];
-            }
-        double h2 = 1e300;
-#pragma unroll
-        for (int i = 0; i < D; ++i)
-            if (i != ax && GI.h[i] < h2) h2 = GI.h[i];
-        use_pc = a.precond != PIT_PRECOND_NONE && Na >= 3 && 2.0 * ha <= h2 * (1.0 + 1e-12) &&
-                 4.0 * dt / (ha * ha) >= 2.0;
+        use_pc = a.precond != PIT_PRECOND_NONE && IC.use_pc;
         if (use_pc) {
             float *lf = reinterpret_cast<float *>(mask + ld);
-            LM.layout(Na, Sa, n, nt);
+            LM.layout(GI.N[GI.fine], GI.S[GI.fine], n, nt);
             LM.f = lf;
-            LM.off = offa;
-            if (tid == 0) LM.setup(lf, offa, HT.diag);
+            LM.off = IC.offf;
+            if (tid == 0) LM.setup(lf, IC.offf, HT.diag);
         }
     }
     auto A64 = [&](const double *v, int j) -> double {
@@ -1255,20 +1337,25 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
     // ||b|| (exact, folded into the conversion), so they stay inside the normal
     // FP32 range for states of any magnitude.
     bool have_r0 = false;
-    double rn0_c = 0.0, bb_c = 0.0;
+    double rn0_c = 0.0, bb_c = 0.0;  // (PAIR)
     int kr_c = 0;
     float *rv = f32 + ld, *pv = f32 + 2 * ld, *sv = f32 + 3 * ld, *wv = f32 + 4 * ld, *tv = f32 + 5 * ld;
     // MIXED: c = x_s - A x_s of the last completed step, in FP64 (the next
     // step's initial residual for the guess x_s, and with the one before it
-    // the residual of the extrapolated guess); have_c: c holds c_{s-1} at the
-    // start of step s + 1
+    // the residual of the extrapolated guess)
     double *cvec = XG ? a.xg + ((long long)2 * a.n_batch + b) * a.n_total + GI.off : s64 + 2 * ld;
-    bool have_c = false;
+    // cst: what that array holds, 1: c_{s-1}, 2: qv = (e_{s-1} - r_{s-2}) 2^kq_c in
+    // FP32 (after steps from extrapolated guesses); unchecked: steps in a row
+    // whose residual met the tolerance without an FP64 check
+    float *qv = reinterpret_cast<float *>(cvec);
+    int cst = 0, kq_c = 0, unchecked = 0;
 
     for (int step = 1; step <= a.nsteps; ++step) {
         // forcing of this step: f_div consecutive steps share one forcing vector
         const double *f = f0 ? f0 + (long long)((step - 1) / a.f_div) * a.f_step : nullptr;
-        __syncthreads();  // state complete
+        // (a MIXED step that carries its residual reads only the thread's own
+        // nodes before its first reduction)
+        if (PREC != MIXED || !have_r0) __syncthreads();  // state complete
         if constexpr (PREC == PLAIN) {
             double *r = v64, *q1 = v64 + vs, *q2 = v64 + 2 * vs, *q3 = v64 + 3 * vs, *q4 = v64 + 4 * vs;
             double bb[1] = {0.0};
@@ -1296,9 +1383,9 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
             ++passes;
             const double stop2 = a.rtol * a.rtol * bb[0];
             int st, k;
-            if constexpr (DRIFT) k = bicgstab_core<double, double>(T64, n, x, r, q1, q2, q3, q4, R64, stop2, a.maxit, st);
-            else if constexpr (OP == PIT_OP_HEAT) k = cg_core<double, double>(H64, n, x, r, q1, q2, q3, R64, stop2, a.maxit, st);
-            else k = cg_core<double, double>(T64, n, x, r, q1, q2, q3, R64, stop2, a.maxit, st);
+            if constexpr (DRIFT) k = bicgstab_core<false>(T64, n, x, r, q1, q2, q3, q4, R64, stop2, a.maxit, st);
+            else if constexpr (OP == PIT_OP_HEAT) k = cg_core<false>(H64, n, x, r, q1, q2, q3, R64, stop2, a.maxit, st);
+            else k = cg_core<false>(T64, n, x, r, q1, q2, q3, R64, stop2, a.maxit, st);
             iters += k;
             if (st > status) status = st;
         } else if constexpr (PREC == SINGLE) {
@@ -1403,12 +1490,12 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
             const float rt = (float)a.rtol;
             const float stop2 = rt * rt * bb[0];
             int st, k;
-            if constexpr (DRIFT) k = bicgstab_core<float, float>(T32, n, xs, r, q1, q2, q3, q4, R32, stop2, a.maxit, st);
+            if constexpr (DRIFT) k = bicgstab_core<false>(T32, n, xs, r, q1, q2, q3, q4, R32, stop2, a.maxit, st);
             else if constexpr (OP == PIT_OP_HEAT) {
-                if (use_pc) k = pcg_core<float, float>(HT, LM, n, xs, r, q4, q1, q2, q3, R32, stop2, a.maxit, st);
-                else k = cg_core<float, float>(HT, n, xs, r, q1, q2, q3, R32, stop2, a.maxit, st);
+                if (use_pc) k = pcg_core<false>(HT, LM, n, xs, r, q4, q1, q2, q3, R32, stop2, a.maxit, st);
+                else k = cg_core<false>(HT, n, xs, r, q1, q2, q3, R32, stop2, a.maxit, st);
             }
-            else k = cg_core<float, float>(T32, n, xs, r, q1, q2, q3, R32, stop2, a.maxit, st);
+            else k = cg_core<false>(T32, n, xs, r, q1, q2, q3, R32, stop2, a.maxit, st);
             iters += k;
             if (st > status) status = st;
             __syncthreads();  // xs complete
@@ -1546,18 +1633,17 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
                 const float want = 0.5f * sqrtf(to_f32(stop2, -2 * kn) / R2n);
                 const float tgt = want > a.inner_rtol ? want : (float)a.inner_rtol;
                 const float stop32 = tgt * tgt * R2n;
-                for (int j = tid; j < n; j += nt) {
-                    rv[j] *= jac ? inv * tab32[j] : inv;
-                    e[j] = 0.0f;
-                }
+                for (int j = tid; j < n; j += nt) rv[j] *= jac ? inv * tab32[j] : inv;
                 int st, k;
                 if constexpr (OP == PIT_OP_HEAT) {
-                    if (use_pc) k = pcg_core<float, float>(HT, LM, n, e, rv, f32 + 5 * ld, pv, sv, wv, R32, stop32, a.maxit, st);
-                    else k = cg_core<float, float>(HT, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st);
+                    if (use_pc) k = pcg_core<true>(HT, LM, n, e, rv, f32 + 5 * ld, pv, sv, wv, R32, stop32, a.maxit, st);
+                    else k = cg_core<true>(HT, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st);
                 } else {
-                    k = cg_core<float, float>(T32, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st);
+                    k = cg_core<true>(T32, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st);
                 }
                 iters += k;
+                if (k == 0)
+                    for (int j = tid; j < n; j += nt) e[j] = 0.0f;
                 if (st == PIT_ERR_NONFINITE) { st_step = st; break; }
                 // x += e 2^kn on the pairs (the scaling is exact; Jacobi: e = D^{-1/2} y)
                 const float csf = __uint_as_float((unsigned)(127 + kn) << 23);
@@ -1648,9 +1734,14 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
                     use_pc = false;
                 }
             }
-            double rn2, bb;
-            int kr;  // the stored FP32 residual rv holds r 2^kr
-            if (have_r0) {
+            // Squared norms as FP32 values of scaled vectors: rn = ||r 2^kr||^2
+            // (rv holds r 2^kr), bb = ||b 2^kb||^2.  The stopping test needs no
+            // more (the sums are FP32), and a comparison in FP64 would cost the
+            // FP64 unit as much for every warp as a node's addition.
+            float rn, bb;
+            int kr, kb;
+            const bool carried = have_r0;
+            if (carried) {
                 // Step s + 1 without forcing: b = x_s, and rv holds r_s 2^kr_c,
                 // r_s = x_{s-1} - A x_s, the FP64 residual of the last check of
                 // step s.  With d = x_s - x_{s-1} (FP64), c_s = x_s - A x_s =
@@ -1660,39 +1751,82 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
                 // r0 = x_s - A x_s - A d = c_s - c_{s-1} + r_s, exact up to
                 // rounding without a stencil pass (the residual of the guess is
                 // about (dt lambda)^2 |x| for a smooth mode of decay rate lambda,
-                // against dt lambda |x| for the guess x_s).
+                // against dt lambda |x| for the guess x_s).  Once step s itself
+                // started from its extrapolated guess, c_s - c_{s-1} = r_s -
+                // r_{s-1} + e_s with e_s the sum of its corrections (x_s =
+                // x_{s-1} + d_{s-1} + e_s), so r0 = 2 r_s + (e_s - r_{s-1}): FP32
+                // throughout, from the sum qv that the steps keep, to 2^-24 of
+                // terms no larger than the corrections themselves.
                 const int kq = kr_c;
-                const bool pred = a.predict && have_c;
                 // additive forcing of the previous step (x holds x_s + g_s)
                 const double *gp =
                     a.g ? a.g + (long long)b * a.g_stride + (long long)(step - 2) * a.g_step + GI.off : nullptr;
+                const int from = !a.predict || gp ? 0 : cst == 2 && kq - kq_c <= 60 && kq_c - kq <= 60 ? 2 : cst == 1 ? 1 : 0;
                 float acc[2] = {0.0f, 0.0f};
-#pragma unroll 4
-                for (int j = tid; j < n; j += nt) {
-                    const double xs = x[j], bo = bvec[j];
-                    const float rs = rv[j];
-                    const double d = xs - bo;
-                    const double cn = to_f64(rs, -kq) + d;
-                    float r0;
-                    if (pred) {
-                        r0 = to_f32_rn(cn - cvec[j], kq) + rs;
-                        x[j] = xs + d;
-                    } else {
-                        r0 = to_f32_rn(cn, kq);
-                        if (gp) x[j] = xs - gp[j];
+                if (from == 2) {
+                    const float sc = scale_f(1.0f, kq - kq_c);
+                    // (four nodes loaded before any is stored: in the global-state
+                    // variant possibly aliasing stores would serialise the loads)
+                    for (int j0 = tid; j0 < n; j0 += 4 * nt) {
+                        double xs[4], bo[4];
+                        float rs[4], qo[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int j = j0 + q * nt;
+                            if (j < n) {
+                                xs[q] = x[j];
+                                bo[q] = bvec[j];
+                                rs[q] = rv[j];
+                                qo[q] = qv[j];
+                            }
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int j = j0 + q * nt;
+                            if (j < n) {
+                                const float r0 = fmaf(2.0f, rs[q], qo[q] * sc);
+                                const float xf = to_f32(xs[q], kq);
+                                qv[j] = -rs[q];
+                                x[j] = fma(2.0, xs[q], -bo[q]);
+                                bvec[j] = xs[q];
+                                rv[j] = r0;
+                                acc[0] += r0 * r0;
+                                acc[1] += xf * xf;
+                            }
+                        }
                     }
-                    if (!gp) cvec[j] = cn;
-                    bvec[j] = xs;
-                    rv[j] = r0;
-                    const float xf = to_f32(xs, kq);
-                    acc[0] += r0 * r0;
-                    acc[1] += xf * xf;
+                } else {
+#pragma unroll 4
+                    for (int j = tid; j < n; j += nt) {
+                        const double xs = x[j], bo = bvec[j];
+                        const float rs = rv[j];
+                        const double d = xs - bo;
+                        const double cn = to_f64(rs, -kq) + d;
+                        float r0;
+                        if (from == 1) {
+                            r0 = to_f32_rn(cn - cvec[j], kq) + rs;
+                            x[j] = xs + d;
+                            pv[j] = -rs;
+                        } else {
+                            r0 = to_f32_rn(cn, kq);
+                            if (gp) x[j] = xs - gp[j];
+                            else cvec[j] = cn;
+                        }
+                        bvec[j] = xs;
+                        rv[j] = r0;
+                        const float xf = to_f32(xs, kq);
+                        acc[0] += r0 * r0;
+                        acc[1] += xf * xf;
+                    }
                 }
-                R32.template sum<2>(acc);  // also: x, b and rv complete
-                rn2 = to_f64(acc[0], -2 * kq);
-                bb = to_f64(acc[1], -2 * kq);
-                kr = kq;
-                have_c = (gp == nullptr);
+                R32.template sum<2>(acc);  // also: x, b and rv complete, cvec read
+                if (from == 1)
+                    for (int j = tid; j < n; j += nt) qv[j] = pv[j];
+                cst = gp ? 0 : from == 0 ? 1 : 2;
+                kq_c = kq;
+                rn = acc[0];
+                bb = acc[1];
+                kr = kb = kq;
             } else {
                 // right-hand side b = x_{s-1} + dt f; optional initial guess;
                 // second SDIRK stage: b = (1 - beta) u_n + beta U1 (b holds u_n,
@@ -1729,8 +1863,8 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
                 double acc[1] = {0.0};
                 for (int j = tid; j < n; j += nt) acc[0] += bvec[j] * bvec[j];
                 R64.template sum<1>(acc);  // also: bvec and x complete
-                bb = acc[0];
-                kr = scale_exp(bb);
+                kr = kb = scale_exp(acc[0]);
+                bb = to_f32(acc[0], 2 * kb);
                 float accf[1] = {0.0f};
                 // without forcing x = b here, so r0 is c_{s-1} = x_{s-1} - A x_{s-1}
 #pragma unroll 4
@@ -1743,66 +1877,81 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
                 }
                 R32.template sum<1>(accf);
                 ++passes;
-                rn2 = to_f64(accf[0], -2 * kr);
-                have_c = carry_ok;
+                rn = accf[0];
+                cst = carry_ok ? 1 : 0;
+                unchecked = -1;
             }
             have_r0 = false;
-            const double stop2 = a.rtol * a.rtol * bb;
-            const int ks = scale_exp(bb);  // FP32 copies of this step: value 2^ks, ||b|| 2^ks in [1, 2)
+            const int ks = kb + scale_exp(bb);  // FP32 copies of this step: value 2^ks, ||b|| 2^ks in [1, 2)
+            float stop2 = a.rtol2 * bb;         // rtol^2 ||b||^2 in the scale of rn
             int st_step = PIT_OK;
-            for (int pass = 0;; ++pass) {
-                if (!(rn2 > stop2)) {
-                    if (rn2 != rn2) st_step = PIT_ERR_NONFINITE;
-                    break;
-                }
-                if (pass >= a.ir_maxit) { st_step = PIT_ERR_NOCONV; break; }
-                // Scalars in FP32 on the scaled residual: rv 2^-kn has squared
-                // norm R2n = ||r||^2 4^(kr - kn) in [1, 4); the power of two
-                // makes the rescaling of the correction exact.
-                const int kn = min(max(kr - scale_exp(rn2), -120), 120);
-                const float inv = __uint_as_float((unsigned)(127 - kn) << 23);  // 2^-kn
-                const float R2n = to_f32(rn2, 2 * (kr - kn));
-                const float want = 0.5f * sqrtf(to_f32(stop2, 2 * (kr - kn)) / R2n);
-                const float tgt = want > a.inner_rtol ? want : (float)a.inner_rtol;
-                const float stop32 = tgt * tgt * R2n;
-                for (int j = tid; j < n; j += nt) {
-                    rv[j] *= jac ? inv * tab32[j] : inv;
-                    e[j] = 0.0f;
-                }
-                int st, k;
-                if constexpr (DRIFT) k = bicgstab_core<float, float>(T32, n, e, rv, pv, sv, wv, tv, R32, stop32, a.maxit, st);
-                else if constexpr (OP == PIT_OP_HEAT) {
-                    if (use_pc) k = pcg_core<float, float>(HT, LM, n, e, rv, f32 + 5 * ld, pv, sv, wv, R32, stop32, a.maxit, st);
-                    else k = cg_core<float, float>(HT, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st);
-                }
-                else k = cg_core<float, float>(T32, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st);
-                iters += k;
-                if (st == PIT_ERR_NONFINITE) { st_step = st; break; }
-                // a stalled or broken-down inner solve still gives a usable
-                // correction; the FP64 residual decides.  x += e 2^(kn - kr)
-                // (FP64, exact scaling)
-                const double cs = pow2d(kn - kr);
-                // (four nodes per thread are loaded before any is stored: x may
-                // live in global memory, where the compiler cannot reorder
-                // loads across the possibly aliasing stores)
-                for (int j0 = tid; j0 < n; j0 += 4 * nt) {
-                    double xv[4];
-                    float ev[4];
+            // (a residual that was only carried counts as met for 15 steps in a
+            // row; the next one is checked in FP64)
+            bool accept = !carried || unchecked < 15;
+            for (int pass = 0;;) {
+                if (!(rn > stop2)) {
+                    if (rn != rn) st_step = PIT_ERR_NONFINITE;
+                    if (st_step != PIT_OK || accept) break;
+                } else {
+                    if (pass >= a.ir_maxit) { st_step = PIT_ERR_NOCONV; break; }
+                    // The FP32 solve runs on rv 2^-kn with squared norm R2n; kn is
+                    // zero unless the norm is so small (large) that the squares of
+                    // the solve would leave the FP32 range.  (The power of two
+                    // makes the rescaling of the correction exact.)
+                    const int kn = rn >= 0x1p-64f && rn <= 0x1p64f ? 0 : min(max(-scale_exp(rn), -120), 120);
+                    const float inv = __uint_as_float((unsigned)(127 - kn) << 23);  // 2^-kn
+                    const float R2n = scale_f(rn, -2 * kn);
+                    const float want = 0.5f * sqrtf(scale_f(stop2, -2 * kn) / R2n);
+                    const float tgt = want > a.inner_rtol ? want : (float)a.inner_rtol;
+                    const float stop32 = tgt * tgt * R2n;
+                    const bool scaled = jac || kn != 0;
+                    if (scaled)
+                        for (int j = tid; j < n; j += nt) rv[j] *= jac ? inv * tab32[j] : inv;
+                    int st, k;
+                    if constexpr (DRIFT) k = bicgstab_core<true>(T32, n, e, rv, pv, sv, wv, tv, R32, stop32, a.maxit, st);
+                    else if constexpr (OP == PIT_OP_HEAT) {
+                        if (use_pc) k = pcg_core<true>(HT, LM, n, e, rv, f32 + 5 * ld, pv, sv, wv, R32, stop32, a.maxit, st, !scaled);
+                        else k = cg_core<true>(HT, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st, !scaled);
+                    }
+                    else k = cg_core<true>(T32, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st, !scaled);
+                    if (k == 0)
+                        for (int j = tid; j < n; j += nt) e[j] = 0.0f;
+                    iters += k;
+                    if (st == PIT_ERR_NONFINITE) { st_step = st; break; }
+                    // a stalled or broken-down inner solve still gives a usable
+                    // correction; the FP64 residual decides.  x += e 2^(kn - kr)
+                    // (FP64, exact scaling)
+                    const double cs = pow2d(kn - kr);
+                    const float cq = scale_f(1.0f, kn - kr + kq_c);
+                    // (four nodes per thread are loaded before any is stored: x may
+                    // live in global memory, where the compiler cannot reorder
+                    // loads across the possibly aliasing stores)
+                    for (int j0 = tid; j0 < n; j0 += 4 * nt) {
+                        double xv[4];
+                        float ev[4], qo[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int j = j0 + q * nt;
-                        if (j < n) {
-                            ev[q] = jac ? e[j] * tab32[j] : e[j];  // Jacobi: e = D^{-1/2} y
-                            xv[q] = x[j];
+                        for (int q = 0; q < 4; ++q) {
+                            const int j = j0 + q * nt;
+                            if (j < n) {
+                                ev[q] = jac ? e[j] * tab32[j] : e[j];  // Jacobi: e = D^{-1/2} y
+                                xv[q] = x[j];
+                                if (cst == 2) qo[q] = qv[j];
+                            }
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int j = j0 + q * nt;
+                            if (j < n) {
+                                x[j] = fma(to_f64(ev[q], 0), cs, xv[q]);
+                                if (cst == 2) qv[j] = fmaf(ev[q], cq, qo[q]);
+                            }
                         }
                     }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int j = j0 + q * nt;
-                        if (j < n) x[j] = fma(to_f64(ev[q], 0), cs, xv[q]);
-                    }
+                    ++pass;
+                    __syncthreads();  // x complete
                 }
-                __syncthreads();  // x complete
+                accept = true;
+                unchecked = -1;
                 // FP64 check: r = b - A x; the stopping test works on the FP32
                 // copy (its squared norm accumulated in FP32), which the next
                 // step also reads for its carried initial residual
@@ -1817,9 +1966,11 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
                 }
                 R32.template sum<1>(accf);
                 ++passes;
-                rn2 = to_f64(accf[0], -2 * ks);
+                rn = accf[0];
                 kr = ks;
+                stop2 = a.rtol2 * scale_f(bb, 2 * (ks - kb));
             }
+            ++unchecked;  // 0 after an FP64 check
             if (st_step > status) status = st_step;
             // rv holds the FP64 residual of the final x (from its check, or
             // the unchanged initial residual when pass 0 met the tolerance)
@@ -1895,12 +2046,45 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(StepArgs a)
     }
 }
 
+// One CTA per item.  The problem's dimension is not a template parameter: the
+// item runs the code of its grid's listed axes.
+template <int OP, int PREC, bool XG>
+__global__ void __launch_bounds__(512, 1) steps_kernel(const __grid_constant__ StepArgs a)
+{
+    static_assert(!XG || PREC != SINGLE, "no global-state variant of the FP32 form");
+    static_assert(PREC == PLAIN || PREC == MIXED || PREC == SINGLE || PREC == PAIR, "unknown precision form");
+    static_assert(PREC != PAIR || (OP != PIT_OP_OU && OP != PIT_OP_LSDE && OP != PIT_OP_CME),
+                  "the pair form is for the symmetric operators");
+    __shared__ GridInfo GI;
+    __shared__ ItemConst IC;
+    __shared__ double red64[2 * 128];
+    __shared__ float red32[2 * 128];
+    const int item = a.item0 + (int)blockIdx.x;
+    const int g = a.order[item / a.n_batch];
+    const int b = item % a.n_batch;
+    if (a.active && !a.active[g]) return;  // uniform over the block
+    static_assert(sizeof(GridInfo) % 4 == 0, "copied by words");
+    for (int t = threadIdx.x; t < (int)(sizeof(GridInfo) / 4); t += blockDim.x)
+        reinterpret_cast<int *>(&GI)[t] = reinterpret_cast<const int *>(a.grids + g)[t];
+    __syncthreads();
+    item_const(a, GI, IC);
+    __syncthreads();
+    switch (GI.de) {
+    case 1: steps_item<OP, PREC, 1, XG>(a, GI, IC, g, b, red64, red32); break;
+    case 2: steps_item<OP, PREC, 2, XG>(a, GI, IC, g, b, red64, red32); break;
+    case 3: steps_item<OP, PREC, 3, XG>(a, GI, IC, g, b, red64, red32); break;
+    case 4: steps_item<OP, PREC, 4, XG>(a, GI, IC, g, b, red64, red32); break;
+    case 5: steps_item<OP, PREC, 5, XG>(a, GI, IC, g, b, red64, red32); break;
+    default: steps_item<OP, PREC, 6, XG>(a, GI, IC, g, b, red64, red32); break;
+    }
+}
+
 // Launchers, one translation unit per (operator, precision form): OPN names
 // the operator (heat, varheat, ou), PN the form (fp64, mixed, fp32).
 #define PIT_STEPS_DECL(OPN, PN)                                                                                   \
     cudaError_t steps_init_##OPN##_##PN(int bytes);                                                               \
-    cudaError_t steps_launch_##OPN##_##PN(int d, const StepArgs &a, dim3 grid, dim3 block, size_t smem,           \
-                                          cudaStream_t s, bool xg);
+    cudaError_t steps_launch_##OPN##_##PN(const StepArgs &a, dim3 grid, dim3 block, size_t smem, cudaStream_t s,  \
+                                          bool xg);
 PIT_STEPS_DECL(heat, fp64) PIT_STEPS_DECL(heat, mixed) PIT_STEPS_DECL(heat, fp32)
 PIT_STEPS_DECL(varheat, fp64) PIT_STEPS_DECL(varheat, mixed) PIT_STEPS_DECL(varheat, fp32)
 PIT_STEPS_DECL(ou, fp64) PIT_STEPS_DECL(ou, mixed) PIT_STEPS_DECL(ou, fp32)
@@ -1908,38 +2092,30 @@ PIT_STEPS_DECL(lsde, fp64) PIT_STEPS_DECL(lsde, mixed) PIT_STEPS_DECL(lsde, fp32
 PIT_STEPS_DECL(cme, fp64) PIT_STEPS_DECL(cme, mixed) PIT_STEPS_DECL(cme, fp32)
 PIT_STEPS_DECL(heat, pair) PIT_STEPS_DECL(varheat, pair)
 
-// Instantiates the attribute setter and launcher of one operator and form for
-// D = 1..6 (XGV: whether the form has the global-state variant).
-#define PIT_STEPS_SET1(OPV, PV, XGV, D)                                                                           \
-    set((const void *)steps_kernel<OPV, PV, D>);                                                                  \
-    if constexpr (XGV) set((const void *)steps_kernel<OPV, PV, D, XGV>);
-#define PIT_STEPS_CASE1(OPV, PV, XGV, D)                                                                          \
-    case D:                                                                                                       \
-        if constexpr (XGV) {                                                                                      \
-            if (xg) { steps_kernel<OPV, PV, D, XGV><<<grid, block, smem, s>>>(a); break; }                        \
-        }                                                                                                         \
-        steps_kernel<OPV, PV, D><<<grid, block, smem, s>>>(a);                                                    \
-        break;
+// Instantiates the attribute setter and launcher of one operator and form
+// (XGV: whether the form has the global-state variant).
 #define PIT_STEPS_OP_PREC(OPN, PN, OPV, PV, XGV)                                                                  \
     cudaError_t steps_init_##OPN##_##PN(int bytes)                                                                \
     {                                                                                                             \
-        cudaError_t e = cudaSuccess;                                                                              \
-        auto set = [&](const void *fn) {                                                                          \
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); \
-        };                                                                                                        \
-        PIT_STEPS_SET1(OPV, PV, XGV, 1) PIT_STEPS_SET1(OPV, PV, XGV, 2) PIT_STEPS_SET1(OPV, PV, XGV, 3)           \
-        PIT_STEPS_SET1(OPV, PV, XGV, 4) PIT_STEPS_SET1(OPV, PV, XGV, 5) PIT_STEPS_SET1(OPV, PV, XGV, 6)           \
+        cudaError_t e = cudaFuncSetAttribute((const void *)steps_kernel<OPV, PV, false>,                          \
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);                 \
+        if constexpr (XGV)                                                                                        \
+            if (e == cudaSuccess)                                                                                 \
+                e = cudaFuncSetAttribute((const void *)steps_kernel<OPV, PV, XGV>,                                \
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);                     \
         return e;                                                                                                 \
     }                                                                                                             \
-    cudaError_t steps_launch_##OPN##_##PN(int d, const StepArgs &a, dim3 grid, dim3 block, size_t smem,           \
-                                          cudaStream_t s, bool xg)                                                \
+    cudaError_t steps_launch_##OPN##_##PN(const StepArgs &a, dim3 grid, dim3 block, size_t smem, cudaStream_t s,  \
+                                          bool xg)                                                                \
     {                                                                                                             \
         if (xg && !XGV) return cudaErrorInvalidValue;                                                             \
-        switch (d) {                                                                                              \
-        PIT_STEPS_CASE1(OPV, PV, XGV, 1) PIT_STEPS_CASE1(OPV, PV, XGV, 2) PIT_STEPS_CASE1(OPV, PV, XGV, 3)        \
-        PIT_STEPS_CASE1(OPV, PV, XGV, 4) PIT_STEPS_CASE1(OPV, PV, XGV, 5) PIT_STEPS_CASE1(OPV, PV, XGV, 6)        \
-        default: return cudaErrorInvalidValue;                                                                    \
+        if constexpr (XGV) {                                                                                      \
+            if (xg) {                                                                                             \
+                steps_kernel<OPV, PV, XGV><<<grid, block, smem, s>>>(a);                                          \
+                return cudaGetLastError();                                                                        \
+            }                                                                                                     \
         }                                                                                                         \
+        steps_kernel<OPV, PV, false><<<grid, block, smem, s>>>(a);                                                \
         return cudaGetLastError();                                                                                \
     }
 
