@@ -179,9 +179,13 @@ struct pit_problem {
     // recombination (Sec. 2.2.2): sparse-grid block plan, built on first use
     bool rc_ready = false;
     RecombPlan rc{};
-    int *rc_lam = nullptr, *rc_list_off = nullptr, *rc_list = nullptr, *rc_lookup = nullptr;
-    long long *rc_off = nullptr;
-    DBuf rc_H, rc_S, rc_cur;
+    RecombPiece *rc_pieces = nullptr;
+    RecombTerm *rc_terms = nullptr;
+    RecombEval *rc_eval = nullptr;
+    int *rc_bad = nullptr;  // a surplus of the last combination sum was not finite
+    RecombBlock *rc_blocks = nullptr;
+    long long *rc_grid_blocks = nullptr;
+    DBuf rc_H, rc_S, rc_T, rc_cur;
 };
 
 namespace {
@@ -875,6 +879,8 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
     CUB(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));
     CUB(phi_kernels_init(P->max_smem));
     CUB(net_kernels_init(P->max_smem));
+    CUB(recombine_init(P->max_smem));
+    CUB(combine_init(P->max_smem));
     CUB(dev_malloc(&P->d_grids, sizeof(GridInfo) * P->G));
     CUB(cudaMemcpy(P->d_grids, P->info.data(), sizeof(GridInfo) * P->G, cudaMemcpyHostToDevice));
     CUB(dev_malloc(&P->d_coef, sizeof(double) * P->G));
@@ -948,13 +954,15 @@ pit_status pit_problem_destroy(pit_problem_t P)
         }
     if (P->ev_fork) cudaEventDestroy(P->ev_fork);
     if (P->ev_join) cudaEventDestroy(P->ev_join);
-    cudaFree(P->rc_lam);
-    cudaFree(P->rc_off);
-    cudaFree(P->rc_list_off);
-    cudaFree(P->rc_list);
-    cudaFree(P->rc_lookup);
+    cudaFree(P->rc_pieces);
+    cudaFree(P->rc_terms);
+    cudaFree(P->rc_eval);
+    cudaFree(P->rc_bad);
+    cudaFree(P->rc_blocks);
+    cudaFree(P->rc_grid_blocks);
     P->rc_H.release();
     P->rc_S.release();
+    P->rc_T.release();
     P->rc_cur.release();
     cudaFree(P->d_grids);
     cudaFree(P->d_coef);
@@ -1227,7 +1235,8 @@ pit_status recomb_plan(pit_problem *P)
         }
     };
     for (int g = 0; g < G; ++g) for_box(g, [&](const int *lam) { used[code_of(lam)] = 1; });
-    std::vector<int> lookup(ncell, -1), blk_lam;
+    std::vector<int> lookup(ncell, -1);
+    std::vector<RecombEval> eval;
     std::vector<long long> blk_off(1, 0);
     int n_blk = 0;
     for (int c = 0; c < ncell; ++c) {
@@ -1239,27 +1248,107 @@ pit_status recomb_plan(pit_problem *P)
             e += lam[i] - 1;
         }
         lookup[c] = n_blk++;
-        blk_lam.insert(blk_lam.end(), lam, lam + d);
+        RecombEval ev{blk_off.back(), {}, 0, 0};
+        for (int i = 0; i < d; ++i) ev.lam[i] = (unsigned char)lam[i];
+        if (!eval.empty())
+            while (ev.from < d - 1 && ev.lam[ev.from] == eval.back().lam[ev.from]) ++ev.from;
+        eval.push_back(ev);
         blk_off.push_back(blk_off.back() + (1LL << e));
     }
-    std::vector<std::vector<int>> lists(n_blk);
-    for (int g = 0; g < G; ++g) for_box(g, [&](const int *lam) { lists[lookup[code_of(lam)]].push_back(g); });
-    std::vector<int> list_off(1, 0), list;
-    for (auto &L : lists) {
-        list.insert(list.end(), L.begin(), L.end());
-        list_off.push_back((int)list.size());
+    // terms of every block and blocks of every grid
+    std::vector<int> list_off(n_blk + 1, 0);
+    std::vector<long long> grid_blocks(1, 0);
+    for (int g = 0; g < G; ++g) {
+        long long k = 0;
+        for_box(g, [&](const int *lam) {
+            ++list_off[lookup[code_of(lam)] + 1];
+            ++k;
+        });
+        grid_blocks.push_back(grid_blocks.back() + k);
+    }
+    if (grid_blocks.back() > 0x7fffffffLL)
+        return fail(PIT_ERR_UNSUPPORTED, "recombination: %lld blocks of all grids", grid_blocks.back());
+    for (int q = 0; q < n_blk; ++q) list_off[q + 1] += list_off[q];
+    std::vector<RecombTerm> terms((size_t)grid_blocks.back());
+    std::vector<RecombBlock> blocks((size_t)grid_blocks.back());
+    std::vector<int> fill(list_off.begin(), list_off.end() - 1);
+    for (int g = 0; g < G; ++g) {
+        long long k = grid_blocks[g];
+        int at = 0;
+        for_box(g, [&](const int *lam) {
+            const int q = lookup[code_of(lam)];
+            blocks[k++] = RecombBlock{blk_off[q], at, 0};
+            terms[fill[q]++] = RecombTerm{P->off[g] + at, P->coef[g]};
+            at += (int)(blk_off[q + 1] - blk_off[q]);
+        });
+    }
+    // The coefficients of a block's terms add up to one, but the d = 6, level-10
+    // set has up to 4,921 of them with an absolute sum near 20,000, and the
+    // surpluses they multiply are nearly equal.  Terms are taken so that the
+    // running sum of coefficients stays small: the sum's rounding errors are
+    // then of the size of a term (in grid order they are 1e-11 of it).
+    for (int q = 0; q < n_blk; ++q) {
+        std::vector<RecombTerm> in(terms.begin() + list_off[q], terms.begin() + list_off[q + 1]);
+        size_t pp = 0, pn = 0;
+        double run = 0.0;
+        for (int k = list_off[q]; k < list_off[q + 1]; ++k) {
+            while (pp < in.size() && in[pp].coef < 0.0) ++pp;
+            while (pn < in.size() && in[pn].coef >= 0.0) ++pn;
+            const bool pos = pn == in.size() || (pp < in.size() && run <= 0.0);
+            terms[k] = in[pos ? pp++ : pn++];
+            run += terms[k].coef;
+        }
+    }
+    std::vector<RecombPiece> pieces;
+    for (int q = 0; q < n_blk; ++q) {
+        const long long sz = blk_off[q + 1] - blk_off[q];
+        if (sz > 0x40000000LL) return fail(PIT_ERR_UNSUPPORTED, "recombination: an increment of %lld nodes", sz);
+        for (long long k = 0; k < sz; k += 256)
+            pieces.push_back(RecombPiece{blk_off[q] + k, (int)k, (int)(sz < 256 ? sz : 256), list_off[q], list_off[q + 1]});
+    }
+    // (the pieces with the most terms a thread first)
+    std::stable_sort(pieces.begin(), pieces.end(), [](const RecombPiece &x, const RecombPiece &y) {
+        return (long long)(x.list1 - x.list0) * x.n > (long long)(y.list1 - y.list0) * y.n;
+    });
+    // classes over the grids by decreasing size (P->d_order)
+    RecombPlan rc{};
+    {
+        std::vector<int> order(G);
+        for (int g = 0; g < G; ++g) order[g] = g;
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return P->info[x].n > P->info[y].n; });
+        int most = 0;
+        for (int g = 0; g < G; ++g) most = std::max(most, (int)(grid_blocks[g + 1] - grid_blocks[g]));
+        for (int k = 0; k < G; ++k) {
+            const int g = order[k], n = P->info[g].n, nbk = (int)(grid_blocks[g + 1] - grid_blocks[g]);
+            // (4,300 nodes: 35 KB; 2,100: 17 KB)
+            const int c = recombine_smem_bytes(n, most, true) > P->max_smem ? 0 : n > 4300 ? 1 : n > 2100 ? 2 : 3;
+            if (rc.cls_n[c]++ == 0) rc.cls_first[c] = k;
+            rc.cls_smem[c] = std::max(rc.cls_smem[c], recombine_smem_bytes(n, nbk, c != 0));
+            if (recombine_smem_bytes(n, nbk, c != 0) > P->max_smem)
+                return fail(PIT_ERR_UNSUPPORTED, "recombination: grid %d has %d increments", g, nbk);
+        }
     }
     auto up = [&](auto *&dst, const auto &v) -> cudaError_t {
         cudaError_t e = dev_malloc(&dst, sizeof(v[0]) * v.size());
         if (e != cudaSuccess) return e;
         return cudaMemcpy(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice);
     };
-    CU(up(P->rc_lam, blk_lam));
-    CU(up(P->rc_off, blk_off));
-    CU(up(P->rc_list_off, list_off));
-    CU(up(P->rc_list, list));
-    CU(up(P->rc_lookup, lookup));
-    P->rc = RecombPlan{n_blk, R, blk_off.back(), P->rc_lam, P->rc_off, P->rc_list_off, P->rc_list, P->rc_lookup};
+    CU(up(P->rc_pieces, pieces));
+    CU(up(P->rc_terms, terms));
+    CU(up(P->rc_eval, eval));
+    CU(dev_malloc(&P->rc_bad, sizeof(int)));
+    CU(up(P->rc_blocks, blocks));
+    CU(up(P->rc_grid_blocks, grid_blocks));
+    rc.n_sparse = blk_off.back();
+    rc.n_blk = n_blk;
+    rc.l_max = Lmax;
+    rc.eval = P->rc_eval;
+    rc.n_pieces = (int)pieces.size();
+    rc.pieces = P->rc_pieces;
+    rc.terms = P->rc_terms;
+    rc.blocks = P->rc_blocks;
+    rc.grid_blocks = P->rc_grid_blocks;
+    P->rc = rc;
     P->rc_ready = true;
     return PIT_OK;
 }
@@ -1270,10 +1359,13 @@ pit_status recombine(pit_problem *P, const double *u, double *out, int nb = 1)
     TRY(recomb_plan(P));
     CU(P->rc_H.ensure(sizeof(double) * P->ntot * (size_t)nb));
     CU(P->rc_S.ensure(sizeof(double) * P->rc.n_sparse * (size_t)nb));
+    if (P->rc.cls_n[0] > 0) CU(P->rc_T.ensure(sizeof(double) * P->ntot * (size_t)nb));
     ProfScope ps(P, 3);
-    CU(launch_recombine(P->rc, P->desc.d, P->d_grids, P->d_coef, P->G, P->ntot, nb, u, P->rc_H.d(), P->rc_S.d(), out,
+    CU(launch_recombine(P->rc, P->d_grids, P->d_order, P->ntot, nb, u, P->rc_H.d(), P->rc_S.d(), P->rc_T.d(), out,
                         P->stream));
-    count_kernels(P, 3, 3);
+    int kernels = 1;
+    for (int c = 0; c < RECOMB_CLS; ++c) kernels += P->rc.cls_n[c] > 0 ? 2 : 0;
+    count_kernels(P, 3, kernels);
     return PIT_OK;
 }
 
@@ -2215,6 +2307,24 @@ extern "C" pit_status pit_mgrit_solve(pit_problem_t P, const double *u0, const p
     return PIT_OK;
 }
 
+// Whether the combination sum at n_pts points takes the sparse grid's
+// surpluses: FP64 operations of the sum over grids (2^d corners and the cells
+// of every grid a point) against those of the surpluses (about eight a node
+// with the gather) and of the increments a point, with 20e6 operations (35 us)
+// for the further launches.  The sum over grids is the faster one for few
+// points on large grid sets.  (Builds the block plan on first use.)
+static bool combine_by_surpluses(pit_problem *P, int n_pts)
+{
+    const double direct = (double)n_pts * P->G * (2.0 * (1 << P->desc.d) + 6.0 * P->desc.d);
+    if (direct < 8.0 * (double)P->ntot + 20e6) return false;
+    if (recomb_plan(P) != PIT_OK) {
+        g_err.clear();
+        return false;
+    }
+    if (combine_eval_smem(P->desc.d, P->rc.l_max) > P->max_smem) return false;
+    return direct > 8.0 * (double)P->ntot + 4.0 * (double)n_pts * P->rc.n_blk + 20e6;
+}
+
 extern "C" pit_status pit_combine(pit_problem_t P, const double *u, int n_pts, const double *pts, double *out)
 {
     if (!P || !u || !pts || !out || n_pts < 0) return fail(PIT_ERR_INVALID_ARG, "bad argument");
@@ -2228,9 +2338,32 @@ extern "C" pit_status pit_combine(pit_problem_t P, const double *u, int n_pts, c
         CU(P->w_out.ensure(sizeof(double) * n_pts));
         target = P->w_out.d();
     }
-    const int chunks = combine_chunks(P->G, n_pts, P->n_sm);
-    if (chunks > 1) CU(P->w_part.ensure(sizeof(double) * (size_t)chunks * n_pts));
-    {
+    if (combine_by_surpluses(P, n_pts)) {
+        // surpluses of the sparse grid, then one basis function of every
+        // increment a point; values that are not finite keep to the points
+        // whose cells they touch, so they are left to the sum over grids
+        CU(P->rc_H.ensure(sizeof(double) * P->ntot));
+        CU(P->rc_S.ensure(sizeof(double) * P->rc.n_sparse));
+        if (P->rc.cls_n[0] > 0) CU(P->rc_T.ensure(sizeof(double) * P->ntot));
+        const int blocks = (n_pts + 127) / 128;
+        // (four blocks of 128 points an SM keep the FP64 unit busy)
+        int chunks = (4 * (P->n_sm > 0 ? P->n_sm : 1) + blocks - 1) / blocks;
+        chunks = std::max(1, std::min(chunks, P->rc.n_blk / 32));
+        if (chunks > 1) CU(P->w_part.ensure(sizeof(double) * (size_t)chunks * n_pts));
+        ProfScope ps(P, 2);
+        CU(cudaMemsetAsync(P->rc_bad, 0, sizeof(int), P->stream));
+        CU(launch_surpluses(P->rc, P->d_grids, P->d_order, P->ntot, 1, du, P->rc_H.d(), P->rc_S.d(), P->rc_T.d(),
+                            P->rc_bad, P->stream));
+        CU(launch_combine_eval(P->rc, P->d_grids, P->d_levels, P->op, P->rc_S.d(), n_pts, dp, target, chunks,
+                               chunks > 1 ? P->w_part.d() : nullptr, P->rc_bad, P->stream));
+        CU(launch_combine(P->d_grids, P->d_coef, P->d_levels, P->G, P->op, du, n_pts, dp, target, 1, nullptr,
+                          P->stream, P->rc_bad));
+        int kernels = 3 + (chunks > 1 ? 1 : 0);
+        for (int c = 0; c < RECOMB_CLS; ++c) kernels += P->rc.cls_n[c] > 0 ? 1 : 0;
+        count_kernels(P, 2, kernels);
+    } else {
+        const int chunks = combine_chunks(P->G, n_pts, P->n_sm);
+        if (chunks > 1) CU(P->w_part.ensure(sizeof(double) * (size_t)chunks * n_pts));
         ProfScope ps(P, 2);
         CU(launch_combine(P->d_grids, P->d_coef, P->d_levels, P->G, P->op, du, n_pts, dp, target, chunks,
                           chunks > 1 ? P->w_part.d() : nullptr, P->stream));

@@ -276,8 +276,10 @@ cudaError_t launch_faces(const GridInfo *grids, int G, OpParams op, double *face
 // over all grids would keep only n_pts / 128 SMs busy, 33 of 152 for the
 // 4,100 points of the d = 6 workload, on FP64 interpolation work.)
 __global__ void combine_kernel(const GridInfo *grids, const double *coef, const int *levels, int G, OpParams op,
-                               const double *u, int n_pts, const double *pts, int gchunk, double *dst)
+                               const double *u, int n_pts, const double *pts, int gchunk, double *dst,
+                               const int *run_if)
 {
+    if (run_if && !*run_if) return;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n_pts) return;
     const int g0 = (int)blockIdx.y * gchunk;
@@ -360,14 +362,15 @@ int combine_chunks(int G, int n_pts, int n_sm)
 
 cudaError_t launch_combine(const GridInfo *grids, const double *coef, const int *levels, int G, OpParams op,
                            const double *u, int n_pts, const double *pts, double *out, int n_chunks, double *part,
-                           cudaStream_t s)
+                           cudaStream_t s, const int *run_if)
 {
     if (n_pts == 0 || G == 0) return cudaSuccess;
     if (n_chunks < 1 || (n_chunks > 1 && !part)) return cudaErrorInvalidValue;
     const int gchunk = (G + n_chunks - 1) / n_chunks;
     const int chunks = (G + gchunk - 1) / gchunk;
     const dim3 grid((unsigned)((n_pts + 127) / 128), (unsigned)chunks);
-    combine_kernel<<<grid, 128, 0, s>>>(grids, coef, levels, G, op, u, n_pts, pts, gchunk, chunks > 1 ? part : out);
+    combine_kernel<<<grid, 128, 0, s>>>(grids, coef, levels, G, op, u, n_pts, pts, gchunk,
+                                     chunks > 1 ? part : out, run_if);
     if (chunks > 1) combine_sum_kernel<<<(n_pts + 127) / 128, 128, 0, s>>>(part, chunks, n_pts, out);
     return cudaGetLastError();
 }

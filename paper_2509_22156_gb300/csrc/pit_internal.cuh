@@ -249,9 +249,18 @@ cudaError_t launch_faces(const GridInfo *grids, int G, OpParams op, double *face
 // chunk set, partial sums in part[chunk * n_pts + k], n_chunks x n_pts doubles,
 // then added in chunk order); 1 means a single kernel writing out directly.
 int combine_chunks(int G, int n_pts, int n_sm);
+// (run_if: the kernel does nothing while *run_if is zero; NULL: always runs)
 cudaError_t launch_combine(const GridInfo *grids, const double *coef, const int *levels, int G, OpParams op,
                            const double *u, int n_pts, const double *pts, double *out, int n_chunks, double *part,
-                           cudaStream_t s);
+                           cudaStream_t s, const int *run_if = nullptr);
+// The same sum from the sparse grid's surpluses S (launch_surpluses): nothing
+// is done while *skip_if is not zero.
+struct RecombPlan;
+size_t combine_eval_smem(int d, int l_max);
+cudaError_t combine_init(size_t max_smem);
+cudaError_t launch_combine_eval(const RecombPlan &R, const GridInfo *grids, const int *levels, const OpParams &op,
+                                const double *S, int n_pts, const double *pts, double *out, int n_chunks, double *part,
+                                const int *skip_if, cudaStream_t s);
 // resid[j*G + g] = || a_j - b_j ||_2 on grid g, for active grids; j < nb.
 cudaError_t launch_resid_norms(const GridInfo *grids, int G, long long ntot, int nb, const double *a,
                                long long a_stride, const double *b, long long b_stride, const int *active,
@@ -264,25 +273,55 @@ cudaError_t launch_resid_max(int G, int nb, const double *resid, const int *acti
                              cudaStream_t s);
 
 // Recombination (Sec. 2.2.2): the sparse grid's hierarchical increments lam
-// (level multi-indices contained in some grid), block b holding the
-// 2^{|lam|_1 - d} surpluses of increment blk_lam[b*d .. b*d+d-1] at
-// [blk_off[b], blk_off[b+1]) in C order; list[list_off[b] .. list_off[b+1])
-// are the grids that contain lam, ascending; lookup[code(lam)] = b (-1: none),
-// code(lam) = ((lam_0 radix + lam_1) radix + ...) + lam_{d-1}.  Device pointers.
-struct RecombPlan {
-    int n_blk;
-    int radix;
-    long long n_sparse;
-    const int *blk_lam;
-    const long long *blk_off;
-    const int *list_off;
-    const int *list;
-    const int *lookup;
+// (level multi-indices contained in some grid) are blocks of 2^{|lam|_1 - d}
+// surpluses, C order inside, one after another; a grid's surpluses are stored
+// as its own blocks, lam ascending lexicographically.  Device pointers.
+struct RecombBlock {      // a block of one grid
+    long long in_sparse;  // where the increment's block starts in the sparse grid
+    int in_grid;          // where it starts in the grid's surpluses
+    int pad;
 };
+struct RecombTerm {       // a grid that contains a block
+    long long at;         // where the grid's copy of the block starts in a packed state
+    double coef;          // the grid's combination coefficient
+};
+struct RecombPiece {      // up to 256 nodes of a block of the sparse grid
+    long long at;         // where they start in the sparse grid
+    int first, n;         // first node in the block, nodes (a power of two)
+    int list0, list1;     // the block's terms, ordered so that running sums of coefficients stay small
+};
+struct RecombEval {       // a block of the sparse grid, for evaluation at points
+    long long at;         // where it starts
+    unsigned char lam[PIT_D];
+    unsigned char from;   // first axis whose level differs from the block before
+    unsigned char pad;
+};
+// Classes of grids by where a CTA keeps the values: 0 in global memory, the
+// others on chip, split by size so that more CTAs of the smaller ones share an
+// SM (three, six and eight of 256 threads).
+constexpr int RECOMB_CLS = 4;
+struct RecombPlan {
+    long long n_sparse;
+    int n_blk, l_max;              // blocks of the sparse grid, largest level
+    const RecombEval *eval;        // per block, lam ascending lexicographically
+    int n_pieces;
+    const RecombPiece *pieces;
+    const RecombTerm *terms;
+    const long long *grid_blocks;  // per grid, first of its blocks (G + 1)
+    const RecombBlock *blocks;
+    int cls_first[RECOMB_CLS], cls_n[RECOMB_CLS];  // range of the grids by decreasing size
+    size_t cls_smem[RECOMB_CLS];
+};
+// S = the sparse grid's surpluses of nb states (the first two of launch_recombine's
+// steps); *bad is set when a surplus is not finite (bad may be NULL).
+cudaError_t launch_surpluses(const RecombPlan &R, const GridInfo *grids, const int *order, long long ntot, int nb,
+                             const double *u, double *H, double *S, double *T, int *bad, cudaStream_t s);
+size_t recombine_smem_bytes(int n, int n_blocks, bool onchip);
+cudaError_t recombine_init(size_t max_smem);
 // out_b = Q u_b on every grid for nb consecutive states b (stride ntot; out
-// may alias u); H: nb x n_total, S: nb x n_sparse doubles of scratch.
-cudaError_t launch_recombine(const RecombPlan &R, int d, const GridInfo *grids, const double *coef, int G,
-                             long long ntot, int nb, const double *u, double *H, double *S, double *out,
-                             cudaStream_t s);
+// may alias u); H: nb x n_total, S: nb x n_sparse doubles of scratch, T: nb x
+// n_total doubles when class 0 is not empty; order: the grids by decreasing size.
+cudaError_t launch_recombine(const RecombPlan &R, const GridInfo *grids, const int *order, long long ntot, int nb,
+                             const double *u, double *H, double *S, double *T, double *out, cudaStream_t s);
 
 }  // namespace pit
