@@ -116,6 +116,9 @@ struct pit_problem {
     int device = 0;
     size_t max_smem = 0;
     int n_sm = 0;  // streaming multiprocessors of the device
+    // clusters of 2^(k+1) CTAs for the FP64 form's class-1 grids: how many run at
+    // once (-1: not asked yet, 0: the grids do not fit), shared memory, reach
+    struct Cluster { int cap = -1, reach = 0, de = 1; size_t smem = 0; } cluster[4];
     bool direct_ok = false;  // heat operator whose grids all take the direct solve
     double direct_dt = 0.0;  // largest step it is used for
     int G = 0;
@@ -503,6 +506,42 @@ PartView part_view(const pit_problem *P, const pit_lane *L, int prec, int part)
             P->smem_cls[prec][1], true};
 }
 
+// Cluster size of a launch of the FP64 form's class-1 grids with `items` items
+// (0: the global-state kernel).  A cluster per item pays while it is the number
+// of items that leaves SMs idle: the largest size whose clusters all run at
+// once.  (Oscillator, seven grids: 16; a relaxation of hundreds of intervals:
+// none, its items fill the SMs.)
+int cluster_size(pit_problem *P, long long items)
+{
+    const std::vector<int> &grids = P->h_order_cls[PLAIN][1];
+    for (int k = 3; k >= 0; --k) {
+        const int C = 2 << k;
+        if (items * C > P->n_sm) continue;
+        pit_problem::Cluster &cl = P->cluster[k];
+        if (cl.cap < 0) {
+            cl.cap = 0;
+            bool fits = !grids.empty();
+            for (int g : grids) {
+                const GridInfo &I = P->info[g];
+                cl.reach = std::max(cl.reach, cluster_reach(I, P->desc.op));
+                cl.de = std::max(cl.de, I.de);
+            }
+            for (int g : grids) {
+                const GridInfo &I = P->info[g];
+                GridInfo J = I;
+                J.de = cl.de;
+                cl.smem = std::max(cl.smem, cluster_smem_bytes(J, C, cl.reach));
+                // (a stencil's neighbours are in this run of nodes or the next)
+                fits = fits && cl.reach <= (I.n + C - 1) / C;
+            }
+            if (fits && cluster_kernel_for(P->desc.op, cl.de) && cl.smem <= P->max_smem)
+                cl.cap = cluster_capacity(P->desc.op, cl.de, C, cl.smem);
+        }
+        if (cl.cap >= items) return C;
+    }
+    return 0;
+}
+
 pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_opts &o, const StepCall &c,
                 const int *active)
 {
@@ -510,6 +549,7 @@ pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_op
     if (slot) return PIT_OK;
     const PartView v = part_view(P, nullptr, prec, cls);
     if (v.n <= 0) return PIT_OK;
+    if (v.xg && prec == PLAIN && cluster_size(P, (long long)v.n * c.nb)) return PIT_OK;
     if (P->forced_threads[wide ? 1 : 0]) {
         slot = P->forced_threads[wide ? 1 : 0];
         return PIT_OK;
@@ -626,6 +666,12 @@ pit_status run_steps(pit_problem *P, const pit_solve_opts &o, const StepCall &c,
             b.bg = b.xg + (long long)c.nb * P->ntot;
         }
         cudaStream_t sq = fork ? st[q] : st[0];
+        if (const int C = v[q].xg && prec == PLAIN ? cluster_size(P, (long long)v[q].n * c.nb) : 0) {
+            const pit_problem::Cluster &cl = P->cluster[C == 16 ? 3 : C == 8 ? 2 : C == 4 ? 1 : 0];
+            CU(launch_cluster(b, cl.de, C, cl.reach, cl.smem, sq));
+            count_kernels(P, wide ? 0 : 1);
+            continue;
+        }
         const int nt = P->threads[prec][wide ? 1 : 0][q];  // (0: a lane's form that was not primed)
         CU(launch_steps(prec, b, nt ? nt : 128, v[q].smem, sq, v[q].xg));
         count_kernels(P, wide ? 0 : 1);

@@ -227,6 +227,16 @@ size_t direct_smem_bytes(int prec, int n, int na, bool xg);
 // Whether a grid's axes but the longest are short enough for the direct solve.
 bool direct_grid(const GridInfo &G);
 int xg_slabs(int prec, int op, int d);
+// FP64 form with one cluster of C CTAs per item (pit_cluster.cu; drift
+// operators, narrow batches of large grids): whether there is a kernel for
+// grids of up to de listed axes, how far the stencil reaches in nodes, the
+// shared memory of a CTA, how many clusters the device runs at once, and the
+// launch.
+bool cluster_kernel_for(int op, int de);
+int cluster_reach(const GridInfo &G, int op);
+size_t cluster_smem_bytes(const GridInfo &G, int C, int reach);
+int cluster_capacity(int op, int de, int C, size_t smem);
+cudaError_t launch_cluster(const StepArgs &a, int de, int C, int reach, size_t smem, cudaStream_t s);
 // Raise the dynamic shared-memory limit of every backward-Euler kernel.
 cudaError_t phi_kernels_init(size_t max_smem);
 // Neighbour masks of every node (bit 2q: interior neighbour at -e_i, 2q+1: at
