@@ -1,6 +1,8 @@
 // Host side of the learned coarse propagator (device code in pit_net.cuh,
 // instantiated per dimension in pit_net_d1.cu .. pit_net_d6.cu): shared-memory
 // sizes, kernel set-up, launch dispatch by dimension, and the Adam step.
+#include <algorithm>
+
 #include "pit_net.cuh"
 
 namespace pit {
@@ -46,7 +48,7 @@ size_t net_smem_bytes(int n)
 size_t net_act_floats(int n, bool train)
 {
     const size_t ld = (size_t)((n + 3) & ~3);
-    return train ? 84 * ld : 35 * ld;
+    return train ? (size_t)net_train_words(n) : 35 * ld;
 }
 
 static size_t g_net_max_smem = 0;
@@ -87,14 +89,22 @@ cudaError_t launch_net_train(const GridInfo *grids, const NetTrainItem *items, i
 {
     if (n_items <= 0) return cudaSuccess;
     const NetTrainItem *it = items;
-    const dim3 grid(n_items), block(256);
+    const dim3 grid(n_items);
+    // activations on chip for the items that fit (act_stride holds those of the
+    // problem's largest grid, so small problems take less shared memory)
+    const size_t tile = (size_t)net_tile_words() * 4;
+    size_t room = std::min((size_t)act_stride * 4, (size_t)net_train_words(NET_CHIP) * 4);
+    if (tile + room > g_net_max_smem) room = g_net_max_smem > tile ? g_net_max_smem - tile : 0;
+    int n_chip = 0;
+    while (net_train_words(n_chip + 4) * 4ull <= room) n_chip += 4;
+    const size_t smem = tile + room;
     switch (op.d) {
-    case 1: net_launch_train_d1(grids, it, u, y, dT, w, act, act_stride, grad_rows, loss_items, op, grid, block, s); break;
-    case 2: net_launch_train_d2(grids, it, u, y, dT, w, act, act_stride, grad_rows, loss_items, op, grid, block, s); break;
-    case 3: net_launch_train_d3(grids, it, u, y, dT, w, act, act_stride, grad_rows, loss_items, op, grid, block, s); break;
-    case 4: net_launch_train_d4(grids, it, u, y, dT, w, act, act_stride, grad_rows, loss_items, op, grid, block, s); break;
-    case 5: net_launch_train_d5(grids, it, u, y, dT, w, act, act_stride, grad_rows, loss_items, op, grid, block, s); break;
-    case 6: net_launch_train_d6(grids, it, u, y, dT, w, act, act_stride, grad_rows, loss_items, op, grid, block, s); break;
+    case 1: net_launch_train_d1(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 2: net_launch_train_d2(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 3: net_launch_train_d3(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 4: net_launch_train_d4(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 5: net_launch_train_d5(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 6: net_launch_train_d6(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

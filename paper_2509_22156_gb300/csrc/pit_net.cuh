@@ -32,14 +32,10 @@ __host__ __device__ constexpr int net_wo(int k)
 __host__ __device__ constexpr int net_bo(int k) { return net_wo(k) + net_cout(k) * net_cin(k) * 5; }
 static_assert(net_bo(3) + 1 == PIT_NET_PARAMS, "parameter layout");
 
-// Weight access from the kernel-parameter bank or from global memory.
+// Weight access from the kernel-parameter bank.
 struct WParam {
     const NetWeights &w;
     __device__ __forceinline__ float operator()(int i) const { return w.w[i]; }
-};
-struct WGlobal {
-    const float *w;
-    __device__ __forceinline__ float operator()(int i) const { return __ldg(w + i); }
 };
 
 // Tap validity of node j along axis i for offset t-2 (t = 0..4): bits of the
@@ -130,12 +126,12 @@ __device__ __forceinline__ double block_sum64(double v, double *red)
 
 // Full forward pass of one item on normalised input already in A0 (channel 0:
 // u / sigma, channel 1: a).  Result (layer-4 pre-activation) in O[0..n).
-// H holds 3 x 16 channels when keep is set (training), else 2 x 16 (ping-pong).
+// H holds 2 x 16 channels (ping-pong).
 template <int D, class WA>
 __device__ void net_forward(const WA &W, const float *A0, float *H, float *O, int n, int ld, const uint32_t *mk2,
-                            const int *S, const float *sf, bool keep)
+                            const int *S, const float *sf)
 {
-    float *H1 = H, *H2 = H + 16 * ld, *H3 = keep ? H + 32 * ld : H;
+    float *H1 = H, *H2 = H + 16 * ld, *H3 = H;
     conv_layer<D, 3, 16, true>(W, net_wo(0), net_bo(0), A0, H1, n, ld, mk2, S, sf);
     __syncthreads();
     conv_layer<D, 17, 16, true>(W, net_wo(1), net_bo(1), H1, H2, n, ld, mk2, S, sf);
@@ -191,7 +187,7 @@ __global__ void __launch_bounds__(256) net_steps_kernel(StepArgs a, const __grid
             const double inv = 1.0 / sigma;
             for (int j = tid; j < n; j += nt) A0[j] = (float)(x[j] * inv);
             __syncthreads();
-            net_forward<D>(WParam{W}, A0, H, O, n, ld, mk2, S, sf, false);
+            net_forward<D>(WParam{W}, A0, H, O, n, ld, mk2, S, sf);
             for (int j = tid; j < n; j += nt) x[j] += sigma * (double)O[j];
         }
         const long long sb = (long long)(step - 1);
@@ -223,37 +219,293 @@ __global__ void __launch_bounds__(256) net_steps_kernel(StepArgs a, const __grid
 // activations, relative squared loss ||Phi_hat(u) - y||^2 / ||y||^2, and the
 // gradient with respect to every parameter, written as one row per item
 // (reduced later in a fixed order, so the gradient is deterministic).
+//
+// What bounds it: shared-memory reads beside the FMAs of the three 85 x 16
+// products a node and layer (forward, input gradient, weight gradient; FP32
+// throughout, weights BF16-rounded).  Activations (51 channels, the gradient of
+// a layer's input overwriting that input) and the layer's weights, transposed
+// so that one 16-byte read gives four outputs' weights, are on chip up to 940
+// nodes and in the item's global slab beyond; neighbour indices of a node are
+// worked out once a pass, a missing tap pointing at a zero element of its row;
+// two nodes a thread share every weight read.  The weight gradient takes tiles
+// of 64 nodes: axis sums of every (channel, tap) row and the output gradients
+// in shared memory, then every thread sums eight outputs of one row over half
+// of the tile.  varheat3d level 8 (85 grids of up to 735 nodes), the whole call
+// with its copies: 1,263 us when every FMA read its own weight from global
+// memory and every row's thread formed its own axis sums, 401 us now.
+constexpr int NET_THREADS = 512, NET_TILE = 64, NET_TLD = NET_TILE + 4;
+constexpr int NET_CHIP = 940;  // largest grid whose activations stay on chip
+__host__ __device__ constexpr int net_ld(int n) { return (n + 4) & ~3; }  // one zero element past the nodes
+__host__ __device__ constexpr int net_train_words(int n) { return 52 * net_ld(n); }
+__host__ __device__ constexpr int net_tile_words() { return 85 * 16 + (86 + 16) * NET_TLD; }
+
+// Indices of a node's neighbours at offsets -2, -1, +1, +2 along every axis
+// (zero: the index of the zero element).
 template <int D>
-__global__ void __launch_bounds__(256) net_train_kernel(const GridInfo *grids, const NetTrainItem *items, const double *u,
-                                                        const double *y, double dT, const float *w, float *act,
-                                                        long long act_stride, float *grad_rows, double *loss_items,
-                                                        OpParams op)
+__device__ __forceinline__ void net_neighbours(uint32_t mk, int j, const int *S, int zero, int (&ix)[D][4])
 {
-    __shared__ GridInfo GI;
-    __shared__ double red[32];
-    __shared__ int S[D];
-    __shared__ float sf[D];
-    __shared__ float gacc[3][16 * 17 * 5 + 16];  // per node-group partial weight gradients of one layer
-    const NetTrainItem it = items[blockIdx.x];
-    if (threadIdx.x == 0) GI = grids[it.g];
-    __syncthreads();
-    const int tid = threadIdx.x, nt = blockDim.x, n = GI.n, ld = (n + 3) & ~3;
-    if (tid < D) {
-        S[tid] = GI.S[tid];
-        sf[tid] = (float)(1.0 / (1.0 + 4.0 * dT / (GI.h[tid] * GI.h[tid])));
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        ix[i][0] = (mk >> (4 * i + 2)) & 1u ? j - 2 * S[i] : zero;
+        ix[i][1] = (mk >> (4 * i)) & 1u ? j - S[i] : zero;
+        ix[i][2] = (mk >> (4 * i + 1)) & 1u ? j + S[i] : zero;
+        ix[i][3] = (mk >> (4 * i + 3)) & 1u ? j + 2 * S[i] : zero;
     }
-    float *base = act + (long long)blockIdx.x * act_stride;
-    float *A0 = base, *H = base + 2 * ld, *O = base + 50 * ld, *DA = base + 51 * ld, *DB = base + 67 * ld;
-    uint32_t *mk2 = reinterpret_cast<uint32_t *>(base + 83 * ld);
+}
+// Nodes a thread takes at a time: two share every weight read; with five or six
+// axes the second node's neighbour indices no longer fit in registers.
+template <int D>
+constexpr bool net_two = D <= 4;
+// axis sum z_t = sum_i in(j + (t - 2) e_i)
+template <int D>
+__device__ __forceinline__ float net_axis_sum(const float *in, int j, int t, const int (&ix)[D][4])
+{
+    if (t == 2) return (float)D * in[j];
+    const int q = t < 2 ? t : t - 1;
+    float z = 0.0f;
+#pragma unroll
+    for (int i = 0; i < D; ++i) z += in[ix[i][q]];
+    return z;
+}
+// a[o] += sum over nch channels and taps of wt[(c 5 + t) 16 + o] z_{c,t} for two nodes
+template <int D>
+__device__ __forceinline__ void net_conv16(const float *in, int nch, int ld, const float4 *wt, int j0, int j1,
+                                           const int (&x0)[D][4], const int (&x1)[D][4], float (&a0)[16], float (&a1)[16])
+{
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+        const float *row = in + c * ld;
+#pragma unroll
+        for (int t = 0; t < 5; ++t) {
+            const float z0 = net_axis_sum<D>(row, j0, t, x0);
+            float z1 = 0.0f;
+            if constexpr (net_two<D>) z1 = net_axis_sum<D>(row, j1, t, x1);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 w = wt[(c * 5 + t) * 4 + q];
+                a0[4 * q] = fmaf(w.x, z0, a0[4 * q]);
+                if constexpr (net_two<D>) a1[4 * q] = fmaf(w.x, z1, a1[4 * q]);
+                a0[4 * q + 1] = fmaf(w.y, z0, a0[4 * q + 1]);
+                if constexpr (net_two<D>) a1[4 * q + 1] = fmaf(w.y, z1, a1[4 * q + 1]);
+                a0[4 * q + 2] = fmaf(w.z, z0, a0[4 * q + 2]);
+                if constexpr (net_two<D>) a1[4 * q + 2] = fmaf(w.z, z1, a1[4 * q + 2]);
+                a0[4 * q + 3] = fmaf(w.w, z0, a0[4 * q + 3]);
+                if constexpr (net_two<D>) a1[4 * q + 3] = fmaf(w.w, z1, a1[4 * q + 3]);
+            }
+        }
+    }
+}
+
+template <int D>
+struct NetItem {  // one item's geometry and buffers
+    int n, ld;
+    const int *S;
+    const float *sf;
+    const uint32_t *mk;
+    float *wt, *zt, *dt;  // weights of a layer, tile of axis sums, tile of output gradients
+};
+
+// out[o][j] of one layer: ReLU of 16 channels, or the last layer's single one
+template <int D>
+__device__ __forceinline__ void net_layer(const NetItem<D> &I, int k, const float *w, const float *in, float *out)
+{
+    const int cin = net_cin(k), cout = net_cout(k), wo = net_wo(k), bo = net_bo(k), nt = blockDim.x;
+    __syncthreads();  // in complete, wt free
+    for (int q = threadIdx.x; q < cin * 5 * 16; q += nt) {
+        const int r = q >> 4, o = q & 15;
+        I.wt[q] = o < cout ? __ldg(w + wo + (o * cin + r / 5) * 5 + r % 5) : 0.0f;
+    }
+    __syncthreads();
+    const float4 *wt = reinterpret_cast<const float4 *>(I.wt);
+    for (int j0 = threadIdx.x; j0 < I.n; j0 += (net_two<D> ? 2 : 1) * nt) {
+        const bool two = net_two<D> && j0 + nt < I.n;
+        const int j1 = two ? j0 + nt : I.n;
+        int x0[D][4], x1[D][4];
+        const uint32_t m0 = I.mk[j0], m1 = two ? I.mk[j1] : 0u;
+        net_neighbours<D>(m0, j0, I.S, I.n, x0);
+        net_neighbours<D>(m1, j1, I.S, I.n, x1);
+        float a0[16], a1[16];
+        if (k == 3) {
+            a0[0] = a1[0] = __ldg(w + bo);
+#pragma unroll 1
+            for (int c = 0; c < 16; ++c)
+#pragma unroll
+                for (int t = 0; t < 5; ++t) {
+                    const float wv = I.wt[(c * 5 + t) * 16];
+                    a0[0] = fmaf(wv, net_axis_sum<D>(in + c * I.ld, j0, t, x0), a0[0]);
+                    if constexpr (net_two<D>) a1[0] = fmaf(wv, net_axis_sum<D>(in + c * I.ld, j1, t, x1), a1[0]);
+                }
+        } else {
+#pragma unroll
+            for (int o = 0; o < 16; ++o) a0[o] = a1[o] = __ldg(w + bo + o);
+            net_conv16<D>(in, cin - 1, I.ld, wt, j0, j1, x0, x1, a0, a1);
+        }
+        // the s channel: s_i where the tap exists
+#pragma unroll
+        for (int t = 0; t < 5; ++t) {
+            float z0 = 0.0f, z1 = 0.0f;
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                if (tap_ok(m0, i, t)) z0 += I.sf[i];
+                if (tap_ok(m1, i, t)) z1 += I.sf[i];
+            }
+            const float *ws = I.wt + ((cin - 1) * 5 + t) * 16;
+            if (k == 3) {
+                a0[0] = fmaf(ws[0], z0, a0[0]);
+                a1[0] = fmaf(ws[0], z1, a1[0]);
+            } else {
+#pragma unroll
+                for (int o = 0; o < 16; ++o) {
+                    a0[o] = fmaf(ws[o], z0, a0[o]);
+                    a1[o] = fmaf(ws[o], z1, a1[o]);
+                }
+            }
+        }
+        if (k == 3) {
+            out[j0] = a0[0];
+            if (two) out[j1] = a1[0];
+        } else {
+#pragma unroll
+            for (int o = 0; o < 16; ++o) {
+                out[o * I.ld + j0] = fmaxf(a0[o], 0.0f);
+                if (two) out[o * I.ld + j1] = fmaxf(a1[o], 0.0f);
+            }
+        }
+    }
+}
+
+// Gradient of the layer's weights and biases from its input and the gradient
+// dc of its pre-activations, into grow.
+template <int D>
+__device__ __forceinline__ void net_weight_grad(const NetItem<D> &I, int k, const float *in, const float *dc, float *grow)
+{
+    const int cind = net_cin(k) - 1, cout = net_cout(k), R = (cind + 1) * 5;
+    const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    const int row = tid >> 2, grp = tid & 1, split = (tid >> 1) & 1;  // row R: the bias
+    const bool active = row <= R && grp * 8 < cout;
+    float acc[8];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) acc[o] = 0.0f;
+    for (int j0 = 0; j0 < I.n; j0 += NET_TILE) {
+        __syncthreads();  // tile free (first: dc complete)
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int kk = lane + 32 * half, j = j0 + kk;
+            if (j < I.n) {
+                int ix[D][4];
+                const uint32_t m = I.mk[j];
+                net_neighbours<D>(m, j, I.S, I.n, ix);
+                for (int c = warp; c <= cind; c += NET_THREADS / 32) {
+#pragma unroll
+                    for (int t = 0; t < 5; ++t) {
+                        float z = 0.0f;
+                        if (c < cind) {
+                            z = net_axis_sum<D>(in + c * I.ld, j, t, ix);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < D; ++i)
+                                if (tap_ok(m, i, t)) z += I.sf[i];
+                        }
+                        I.zt[(c * 5 + t) * NET_TLD + kk] = z;
+                    }
+                }
+            } else {
+                for (int c = warp; c <= cind; c += NET_THREADS / 32)
+#pragma unroll
+                    for (int t = 0; t < 5; ++t) I.zt[(c * 5 + t) * NET_TLD + kk] = 0.0f;
+            }
+        }
+        if (tid < NET_TILE) I.zt[R * NET_TLD + tid] = 1.0f;
+        for (int q = tid; q < 16 * NET_TILE; q += nt) {
+            const int o = q / NET_TILE, kk = q % NET_TILE, j = j0 + kk;
+            I.dt[o * NET_TLD + kk] = o < cout && j < I.n ? dc[o * I.ld + j] : 0.0f;
+        }
+        __syncthreads();
+        if (active) {
+            const float4 *z4 = reinterpret_cast<const float4 *>(I.zt + row * NET_TLD + split * (NET_TILE / 2));
+#pragma unroll 2
+            for (int q = 0; q < NET_TILE / 8; ++q) {
+                const float4 z = z4[q];
+#pragma unroll
+                for (int o = 0; o < 8; ++o) {
+                    const float4 d = reinterpret_cast<const float4 *>(I.dt + (grp * 8 + o) * NET_TLD + split * (NET_TILE / 2))[q];
+                    acc[o] = fmaf(d.x, z.x, acc[o]);
+                    acc[o] = fmaf(d.y, z.y, acc[o]);
+                    acc[o] = fmaf(d.z, z.z, acc[o]);
+                    acc[o] = fmaf(d.w, z.w, acc[o]);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (active && split == 1) {
+#pragma unroll
+        for (int o = 0; o < 8; ++o) I.zt[(row * 2 + grp) * 8 + o] = acc[o];
+    }
+    __syncthreads();
+    if (active && split == 0) {
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+            const int oo = grp * 8 + o;
+            if (oo < cout) {
+                const float v = acc[o] + I.zt[(row * 2 + grp) * 8 + o];
+                grow[row == R ? net_bo(k) + oo : net_wo(k) + (oo * (cind + 1) + row / 5) * 5 + row % 5] = v;
+            }
+        }
+    }
+}
+
+// Gradient of the layer's 16 input channels through the ReLU of the layer
+// before, in place of that layer's output h:
+// din[c][j] = sum_t sum_o W[o][c][t] sum_i dc[o][j - (t-2) e_i].
+template <int D>
+__device__ __forceinline__ void net_input_grad(const NetItem<D> &I, int k, const float *w, const float *dc, float *h)
+{
+    const int cout = net_cout(k), wo = net_wo(k), nt = blockDim.x;
+    __syncthreads();  // wt and the tiles free, dc and h read
+    for (int q = threadIdx.x; q < cout * 5 * 16; q += nt) {
+        const int r = q >> 4, c = q & 15;  // row (o, t'), t' = 4 - t
+        I.wt[q] = __ldg(w + wo + ((r / 5) * 17 + c) * 5 + (4 - r % 5));
+    }
+    __syncthreads();
+    const float4 *wt = reinterpret_cast<const float4 *>(I.wt);
+    for (int j0 = threadIdx.x; j0 < I.n; j0 += (net_two<D> ? 2 : 1) * nt) {
+        const bool two = net_two<D> && j0 + nt < I.n;
+        const int j1 = two ? j0 + nt : I.n;
+        int x0[D][4], x1[D][4];
+        net_neighbours<D>(I.mk[j0], j0, I.S, I.n, x0);
+        net_neighbours<D>(two ? I.mk[j1] : 0u, j1, I.S, I.n, x1);
+        float a0[16], a1[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) a0[c] = a1[c] = 0.0f;
+        net_conv16<D>(dc, cout, I.ld, wt, j0, j1, x0, x1, a0, a1);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+            h[c * I.ld + j0] = h[c * I.ld + j0] > 0.0f ? a0[c] : 0.0f;
+            if (two) h[c * I.ld + j1] = h[c * I.ld + j1] > 0.0f ? a1[c] : 0.0f;
+        }
+    }
+}
+
+template <int D>
+__device__ __forceinline__ void net_train_item(const GridInfo &GI, const int *S, const float *sf, double *red, float *tiles,
+                                               float *acts, const NetTrainItem &it, const double *u, const double *y,
+                                               const float *w, float *grow, double *loss, const OpParams &op)
+{
+    const int tid = threadIdx.x, nt = blockDim.x, n = GI.n, ld = net_ld(n);
+    // channels: A0 (2), H1..H3 (16 each), O, then the masks
+    float *A0 = acts, *H1 = acts + 2 * ld, *H2 = H1 + 16 * ld, *H3 = H2 + 16 * ld, *O = H3 + 16 * ld;
+    uint32_t *mk = reinterpret_cast<uint32_t *>(O + ld);
+    NetItem<D> I{n, ld, S, sf, mk, tiles, tiles + 85 * 16, tiles + 85 * 16 + 86 * NET_TLD};
     const double *ui = u + it.off, *yi = y + it.off;
-    float *grow = grad_rows + (long long)blockIdx.x * PIT_NET_PARAMS;
     double ss = 0.0, yy = 0.0;
     for (int j = tid; j < n; j += nt) {
-        mk2[j] = ext_mask<D>(GI, j);
+        mk[j] = ext_mask<D>(GI, j);
         A0[ld + j] = (float)node_coef(op, GI, j, D);
         ss += ui[j] * ui[j];
         yy += yi[j] * yi[j];
     }
+    for (int c = tid; c < 51; c += nt) acts[c * ld + n] = 0.0f;  // the zero element of every row
     ss = block_sum64(ss, red);
     yy = block_sum64(yy, red);
     const double sigma = sqrt(ss / (double)n);
@@ -264,96 +516,62 @@ __global__ void __launch_bounds__(256) net_train_kernel(const GridInfo *grids, c
         for (int j = tid; j < n; j += nt) l += (ui[j] - yi[j]) * (ui[j] - yi[j]);
         l = block_sum64(l, red);
         for (int p = tid; p < PIT_NET_PARAMS; p += nt) grow[p] = 0.0f;
-        if (tid == 0) loss_items[blockIdx.x] = l / yy;
+        if (tid == 0) *loss = l / yy;
         return;
     }
     const double inv = 1.0 / sigma;
     for (int j = tid; j < n; j += nt) A0[j] = (float)(ui[j] * inv);
+    net_layer<D>(I, 0, w, A0, H1);
+    net_layer<D>(I, 1, w, H1, H2);
+    net_layer<D>(I, 2, w, H2, H3);
+    net_layer<D>(I, 3, w, H3, O);
     __syncthreads();
-    WGlobal W{w};
-    net_forward<D>(W, A0, H, O, n, ld, mk2, S, sf, true);
     // loss and dL/d(layer-4 pre-activation) = 2 e sigma / ||y||^2
     double l = 0.0;
     for (int j = tid; j < n; j += nt) {
         const double e = ui[j] + sigma * (double)O[j] - yi[j];
         l += e * e;
-        DA[j] = (float)(2.0 * e * sigma / yy);
+        O[j] = (float)(2.0 * e * sigma / yy);
     }
     l = block_sum64(l, red);
-    if (tid == 0) loss_items[blockIdx.x] = l / yy;
-    __syncthreads();
+    if (tid == 0) *loss = l / yy;
+    net_weight_grad<D>(I, 3, H3, O, grow);
+    net_input_grad<D>(I, 3, w, O, H3);
+    net_weight_grad<D>(I, 2, H2, H3, grow);
+    net_input_grad<D>(I, 2, w, H3, H2);
+    net_weight_grad<D>(I, 1, H1, H2, grow);
+    net_input_grad<D>(I, 1, w, H2, H1);
+    net_weight_grad<D>(I, 0, A0, H1, grow);
+}
 
-    // backward, layer k = 3..0: dpre_k in DCUR (Cout x ld); layer input IN (Cin-1 data channels)
-    float *DCUR = DA, *DNXT = DB;
-    for (int k = 3; k >= 0; --k) {
-        const int cout = net_cout(k);
-        const int cind = net_cin(k) - 1;  // data channels (2 or 16)
-        const float *IN = (k == 0) ? A0 : H + (k - 1) * 16 * ld;
-        const int wo = net_wo(k), bo = net_bo(k);
-        const int nw = cout * (cind + 1) * 5;
-        // weight and bias gradients: 85 (c,t) pairs (35 for layer 0) x 3 node groups
-        const int pairs = (cind + 1) * 5;
-        for (int q = tid; q < 3 * (nw + cout); q += nt) gacc[q / (nw + cout)][q % (nw + cout)] = 0.0f;
-        __syncthreads();
-        for (int q = tid; q < 3 * pairs; q += nt) {
-            const int grp = q / pairs, pc = q % pairs;
-            const int c = pc / 5, t = pc % 5;
-            float accw[16];
-#pragma unroll
-            for (int o = 0; o < 16; ++o) accw[o] = 0.0f;
-            float accb[16];
-#pragma unroll
-            for (int o = 0; o < 16; ++o) accb[o] = 0.0f;
-            for (int j = grp; j < n; j += 3) {
-                const uint32_t mk = mk2[j];
-                float z = 0.0f;
-                for (int i = 0; i < D; ++i)
-                    if (tap_ok(mk, i, t)) z += (c < cind) ? IN[c * ld + j + (t - 2) * S[i]] : sf[i];
-#pragma unroll
-                for (int o = 0; o < 16; ++o) {
-                    if (o < cout) {
-                        const float dp = DCUR[o * ld + j];
-                        accw[o] = fmaf(dp, z, accw[o]);
-                        accb[o] += dp;
-                    }
-                }
-            }
-            for (int o = 0; o < cout; ++o) gacc[grp][(o * (cind + 1) + c) * 5 + t] = accw[o];
-            if (pc == 0)
-                for (int o = 0; o < cout; ++o) gacc[grp][nw + o] = accb[o];
-        }
-        __syncthreads();
-        for (int p = tid; p < nw + cout; p += nt)
-            grow[wo + p] = (gacc[0][p] + gacc[1][p]) + gacc[2][p];  // wo + nw == bo
-        (void)bo;
-        if (k == 0) break;
-        // input gradient of layer k through the ReLU of layer k-1:
-        // din[c][jj] = sum_t sum_o W[o][c][t] sum_i dpre[o][jj - (t-2) e_i]
-        const float *HPREV = H + (k - 1) * 16 * ld;
-        for (int j = tid; j < n; j += nt) {
-            const uint32_t mk = mk2[j];
-            float din[16];
-#pragma unroll
-            for (int c = 0; c < 16; ++c) din[c] = 0.0f;
-#pragma unroll
-            for (int t = 0; t < 5; ++t) {
-                for (int o = 0; o < cout; ++o) {
-                    float qv = 0.0f;
-#pragma unroll
-                    for (int i = 0; i < D; ++i)
-                        if (tap_ok(mk, i, 4 - t)) qv += DCUR[o * ld + j - (t - 2) * S[i]];
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) din[c] = fmaf(W(wo + (o * 17 + c) * 5 + t), qv, din[c]);
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < 16; ++c) DNXT[c * ld + j] = HPREV[c * ld + j] > 0.0f ? din[c] : 0.0f;
-        }
-        __syncthreads();
-        float *tmp = DCUR;
-        DCUR = DNXT;
-        DNXT = tmp;
+template <int D>
+__global__ void __launch_bounds__(NET_THREADS, 1)
+    net_train_kernel(const GridInfo *grids, const NetTrainItem *items, const double *u, const double *y, double dT,
+                     const float *w, float *act, long long act_stride, int n_chip, float *grad_rows, double *loss_items,
+                     OpParams op)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ GridInfo GI;
+    __shared__ double red[32];
+    __shared__ int S[D];
+    __shared__ float sf[D];
+    const NetTrainItem it = items[blockIdx.x];
+    if (threadIdx.x == 0) GI = grids[it.g];
+    __syncthreads();
+    const int tid = threadIdx.x;
+    if (tid < D) {
+        S[tid] = GI.S[tid];
+        sf[tid] = (float)(1.0 / (1.0 + 4.0 * dT / (GI.h[tid] * GI.h[tid])));
     }
+    __syncthreads();
+    float *tiles = reinterpret_cast<float *>(smem);
+    float *grow = grad_rows + (long long)blockIdx.x * PIT_NET_PARAMS;
+    // (two calls, so that the one on chip uses shared-memory instructions)
+    if (GI.n <= n_chip)
+        net_train_item<D>(GI, S, sf, red, tiles, tiles + net_tile_words(), it, u, y, w, grow, loss_items + blockIdx.x, op);
+    else
+        net_train_item<D>(GI, S, sf, red, tiles, act + (long long)blockIdx.x * act_stride, it, u, y, w, grow,
+                          loss_items + blockIdx.x, op);
 }
 
 // Per-dimension launchers (one translation unit per d, pit_net_d<d>.cu).
@@ -362,15 +580,17 @@ __global__ void __launch_bounds__(256) net_train_kernel(const GridInfo *grids, c
     void net_launch_steps_d##D(const StepArgs &a, const NetWeights &W, float *act, long long act_stride,         \
                                dim3 grid, dim3 block, size_t smem, cudaStream_t s);                              \
     void net_launch_train_d##D(const GridInfo *grids, const NetTrainItem *it, const double *u, const double *y,   \
-                               double dT, const float *w, float *act, long long act_stride, float *grad_rows,    \
-                               double *loss_items, OpParams op, dim3 grid, dim3 block, cudaStream_t s);
+                               double dT, const float *w, float *act, long long act_stride, int n_chip,          \
+                               float *grad_rows, double *loss_items, OpParams op, dim3 grid, size_t smem,        \
+                               cudaStream_t s);
 PIT_NET_DECL(1) PIT_NET_DECL(2) PIT_NET_DECL(3) PIT_NET_DECL(4) PIT_NET_DECL(5) PIT_NET_DECL(6)
 
 #define PIT_NET_DIM(D)                                                                                           \
     cudaError_t net_init_d##D(int bytes)                                                                         \
     {                                                                                                            \
-        return cudaFuncSetAttribute((const void *)net_steps_kernel<D>,                                           \
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);                         \
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;                                           \
+        const cudaError_t e = cudaFuncSetAttribute((const void *)net_steps_kernel<D>, attr, bytes);              \
+        return e != cudaSuccess ? e : cudaFuncSetAttribute((const void *)net_train_kernel<D>, attr, bytes);      \
     }                                                                                                            \
     void net_launch_steps_d##D(const StepArgs &a, const NetWeights &W, float *act, long long act_stride,         \
                                dim3 grid, dim3 block, size_t smem, cudaStream_t s)                               \
@@ -378,11 +598,12 @@ PIT_NET_DECL(1) PIT_NET_DECL(2) PIT_NET_DECL(3) PIT_NET_DECL(4) PIT_NET_DECL(5) 
         net_steps_kernel<D><<<grid, block, smem, s>>>(a, W, act, act_stride);                                    \
     }                                                                                                            \
     void net_launch_train_d##D(const GridInfo *grids, const NetTrainItem *it, const double *u, const double *y,   \
-                               double dT, const float *w, float *act, long long act_stride, float *grad_rows,    \
-                               double *loss_items, OpParams op, dim3 grid, dim3 block, cudaStream_t s)           \
+                               double dT, const float *w, float *act, long long act_stride, int n_chip,          \
+                               float *grad_rows, double *loss_items, OpParams op, dim3 grid, size_t smem,        \
+                               cudaStream_t s)                                                                   \
     {                                                                                                            \
-        net_train_kernel<D><<<grid, block, 0, s>>>(grids, it, u, y, dT, w, act, act_stride, grad_rows,           \
-                                                   loss_items, op);                                              \
+        net_train_kernel<D><<<grid, NET_THREADS, smem, s>>>(grids, it, u, y, dT, w, act, act_stride, n_chip,     \
+                                                            grad_rows, loss_items, op);                          \
     }
 
 }  // namespace pit
