@@ -121,6 +121,7 @@ struct pit_problem {
     struct Cluster { int cap = -1, reach = 0, de = 1; size_t smem = 0; } cluster[4];
     bool direct_ok = false;  // heat operator whose grids all take the direct solve
     double direct_dt = 0.0;  // largest step it is used for
+    double fix_n = 0.0, fix_h = 0.0;  // largest n^{1/2}, n^{1/2} sum 1 / h^2 of a grid (error of the integer residual)
     int G = 0;
     long long ntot = 0;
     std::vector<int> levels;      // G*d
@@ -471,6 +472,7 @@ StepArgs make_args(pit_problem *P, const pit_solve_opts &o, const StepCall &c, c
     a.inner_rtol = (float)o.inner_rtol;
     a.ir_maxit = o.ir_maxit;
     a.inexact = c.inexact;
+    a.fixed = 8.0 * 0x1p-53 * std::max(P->fix_n, c.dt * P->fix_h) <= 0.25 * o.rtol;
     a.precond = o.precond;
     a.predict = o.guess != PIT_GUESS_PREVIOUS;
     a.sdirk = c.sdirk;
@@ -882,7 +884,13 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
     }
     P->ntot = P->off[P->G];
     P->direct_ok = desc->op == PIT_OP_HEAT;
-    for (const GridInfo &I : P->info) P->direct_ok = P->direct_ok && direct_grid(I);
+    for (const GridInfo &I : P->info) {
+        P->direct_ok = P->direct_ok && direct_grid(I);
+        double s = 0.0;
+        for (int i = 0; i < d; ++i) s += I.ih2[i];
+        P->fix_n = std::max(P->fix_n, sqrt((double)I.n));
+        P->fix_h = std::max(P->fix_h, sqrt((double)I.n) * s);
+    }
     P->direct_dt = 1e300;
     for (int i = 0; i < d; ++i) {
         const double len = desc->hi[i] - desc->lo[i];

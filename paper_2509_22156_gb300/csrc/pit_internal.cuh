@@ -153,6 +153,7 @@ struct StepArgs {
     float inner_rtol;
     int ir_maxit;
     int inexact;             // 1: a solve stopped by its iteration caps is not a failure
+    int fixed;               // MIXED_D: the tolerance allows the integer state (pit_fixed.cuh)
     int precond;             // pit_precond of the Krylov solves
     int predict;             // MIXED without forcing: extrapolated initial guess 2 x_s - x_{s-1}
     int sdirk;               // MIXED or SINGLE: every step is a two-stage SDIRK step, dt its stage step

@@ -1,7 +1,7 @@
 // Host-side dispatch of the multi-step backward-Euler kernels (pit_phi.cuh):
 // shared-memory sizing, attribute set-up and launch by operator, precision
 // form and dimension.
-#include "pit_direct.cuh"
+#include "pit_fixed.cuh"
 
 namespace pit {
 
@@ -56,7 +56,7 @@ cudaError_t phi_kernels_init(size_t max_smem)
                                    steps_init_lsde_fp64,    steps_init_lsde_mixed,    steps_init_lsde_fp32,
                                    steps_init_cme_fp64,     steps_init_cme_mixed,     steps_init_cme_fp32,
                                    steps_init_heat_pair,    steps_init_varheat_pair, direct_init_mixed,
-                                   direct_init_pair};
+                                   direct_init_pair,        fixed_init};
     for (auto f : inits)
         if (e == cudaSuccess) e = f(bytes);
     if (e == cudaSuccess) g_max_smem = max_smem;
@@ -70,6 +70,10 @@ cudaError_t launch_steps(int prec, const StepArgs &a, int threads, size_t smem, 
     if (blocks > 0x7fffffffLL || smem > g_max_smem || threads < 32 || threads > 512 || (threads & 31))
         return cudaErrorInvalidConfiguration;
     const dim3 grid((unsigned)blocks), block(threads);
+    // (steps without forcing or a caller's guess carry their residual, and may
+    // hold the state as integers)
+    if (prec == MIXED_D && a.fixed && !a.f && !a.g && !a.guess && !a.sdirk && !a.ext)
+        return fixed_launch(a, grid, block, smem, s, xg);
     if (prec == MIXED_D) return direct_launch_mixed(a, grid, block, smem, s, xg);
     if (prec == PAIR_D) return direct_launch_pair(a, grid, block, smem, s, xg);
     if (prec == SINGLE && xg) {

@@ -1,0 +1,98 @@
+"""Integer-state refinement of the heat operator (steps without forcing) against the oracle: long decays (the state is
+rescaled on the way), states of any magnitude, both initial guesses, grids on chip and in global memory, inputs that are
+not finite, and the tolerance at which the FP64 check takes over.
+
+Tolerance: every step's residual is at most rtol ||b|| and the form's own error a quarter of that, ||A^-1|| <= 1: S
+steps are within 1.25 S rtol of the exact propagation relative to the state that decays least, 1e-9 for the S used."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2509_22156_gb300 import binding as B
+from paper_2509_22156_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2509_22156_gb300 import build
+    build.build()
+    B.load()
+    torch.cuda.set_device(0)
+
+
+def opts(rtol=1e-11, guess=B.PIT_GUESS_DEFAULT):
+    return B.solve_opts(B.PIT_PREC_MIXED, rtol=rtol, maxit=4000, inner_rtol=1e-6, ir_maxit=12, guess=guess)
+
+
+def solve(P, u, dt, steps, o):
+    out = torch.empty(P.n_total, dtype=torch.float64, device="cuda")
+    st = P.sequential_solve(torch.from_numpy(u).cuda(), dt, steps, out, o)
+    return out.cpu().numpy(), st
+
+
+def worst(P, a, b):
+    return max(np.linalg.norm(a[P.offsets[g]:P.offsets[g + 1]] - b[P.offsets[g]:P.offsets[g + 1]]) /
+               np.linalg.norm(b[P.offsets[g]:P.offsets[g + 1]]) for g in range(P.G))
+
+
+@pytest.mark.parametrize("guess", [B.PIT_GUESS_PREVIOUS, B.PIT_GUESS_EXTRAPOLATE])
+@pytest.mark.parametrize("d,n,dt,steps", [(1, 5, 0.2, 60), (2, 5, 0.05, 60), (3, 4, 1e-3, 33), (4, 4, 1e-3, 20),
+                                          (6, 3, 1e-3, 20)])
+def test_long_decay_matches_oracle(d, n, dt, steps, guess):
+    P = B.Problem(d, n, 1, W.OP_HEAT)
+    O = oracle.Problem(d, n, 1, W.OP_HEAT)
+    u = O.initial(W.IC_SINES, W.random_sine_modes(d, 4, 2, seed=3)) + 0.3 * O.initial(W.IC_SINES, W.sine_modes(d, [(1.0, [1] * d)]))
+    got, st = solve(P, u, dt, steps, opts(guess=guess))
+    assert st.n_failed == 0
+    ref = O.sequential(u, dt, steps, rtol=1e-15)
+    # (the lowest mode decays least: later residuals are relative to it)
+    assert worst(P, got, ref) < 1e-9
+
+
+def test_states_of_any_magnitude_scale_exactly():
+    # the state is held times a power of two taken from its norm: results scale bit by bit
+    P = B.Problem(3, 5, 1, W.OP_HEAT)
+    u = W.random_vector(9, P.n_total)
+    a, _ = solve(P, u, 1e-3, 12, opts())
+    for e in (-300, -40, 40, 300):
+        b, _ = solve(P, np.ldexp(u, e), 1e-3, 12, opts())
+        np.testing.assert_array_equal(b, np.ldexp(a, e))
+    z, st = solve(P, np.zeros(P.n_total), 1e-3, 12, opts())
+    assert st.n_failed == 0 and not z.any()
+
+
+def test_rough_states_and_global_memory_grids():
+    # a line of 16,383 nodes needs the global-state variant
+    P = B.Problem(1, 14, 1, W.OP_HEAT)
+    O = oracle.Problem(1, 14, 1, W.OP_HEAT)
+    u = W.random_vector(4, P.n_total)
+    dt = 1e-9  # dt / h^2 = 0.27
+    got, st = solve(P, u, dt, 6, opts())
+    assert st.n_failed == 0
+    assert worst(P, got, O.sequential(u, dt, 6, rtol=1e-15)) < 1e-9
+
+
+def test_tight_tolerances_and_bad_inputs():
+    P = B.Problem(2, 6, 1, W.OP_HEAT)
+    O = oracle.Problem(2, 6, 1, W.OP_HEAT)
+    u = O.initial(W.IC_SINES, W.random_sine_modes(2, 4, 3, seed=5))
+    got, st = solve(P, u, 1e-3, 10, opts(rtol=2e-14))  # below what the integer residual is used for
+    assert st.n_failed == 0
+    assert worst(P, got, O.sequential(u, 1e-3, 10, rtol=1e-15)) < 1e-11
+    for bad in (np.nan, np.inf):
+        v = u.copy()
+        v[P.offsets[2] + 1] = bad
+        out = torch.empty(P.n_total, dtype=torch.float64, device="cuda")
+        with pytest.raises(B.PitError) as e:
+            P.sequential_solve(torch.from_numpy(v).cuda(), 1e-3, 3, out, opts())
+        assert e.value.status == B.PIT_ERR_NONFINITE
+        got = out.cpu().numpy()  # the other grids are solved
+        ref = O.sequential(u, 1e-3, 3, rtol=1e-15)
+        for g in range(P.G):
+            sl = slice(P.offsets[g], P.offsets[g + 1])
+            if g != 2:
+                assert np.linalg.norm(got[sl] - ref[sl]) < 1e-9 * np.linalg.norm(ref[sl])
