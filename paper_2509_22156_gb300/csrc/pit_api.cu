@@ -2597,15 +2597,24 @@ struct Rng {
     }
 };
 
-pit_status net_loss_grad_dev(pit_problem *P, double dT, int n_batch, const double *u, const double *y,
-                             const NetTrainItem *items_host, int n_items, const float *w_dev, float *grad_dev,
-                             double *loss_host)
+// Activation offsets of consecutive items in one training launch; returns the
+// floats they take.
+size_t net_place(const pit_problem *P, NetTrainItem *items, int n)
+{
+    long long at = 0;
+    for (int k = 0; k < n; ++k) {
+        items[k].act = at;
+        at += (long long)net_act_floats(P->info[items[k].g].n, true);
+    }
+    return (size_t)at;
+}
+
+pit_status net_loss_grad_dev(pit_problem *P, double dT, const double *u, const double *y, NetTrainItem *items_host,
+                             int n_items, const float *w_dev, float *grad_dev, double *loss_host)
 {
     int nmax = 0;
     for (const GridInfo &I : P->info) nmax = I.n > nmax ? I.n : nmax;
-    (void)n_batch;
-    const long long slab = (long long)net_act_floats(nmax, true);
-    CU(P->n_act.ensure(sizeof(float) * (size_t)(slab * n_items)));
+    CU(P->n_act.ensure(sizeof(float) * net_place(P, items_host, n_items)));
     CU(P->n_rows.ensure(sizeof(float) * (size_t)PIT_NET_PARAMS * n_items));
     CU(P->n_loss.ensure(sizeof(double) * n_items));
     CU(P->n_items.ensure(sizeof(NetTrainItem) * n_items));
@@ -2613,8 +2622,8 @@ pit_status net_loss_grad_dev(pit_problem *P, double dT, int n_batch, const doubl
     {
         ProfScope ps(P, 3);
         CU(launch_net_train(P->d_grids, (const NetTrainItem *)P->n_items.p, n_items, u, y, dT, w_dev,
-                            (float *)P->n_act.p, slab, (float *)P->n_rows.p, P->n_loss.d(), P->op, P->stream));
-        count_kernels(P, 3);
+                            (float *)P->n_act.p, nmax, (float *)P->n_rows.p, P->n_loss.d(), P->op, P->stream));
+        count_kernels(P, 3, 2);
     }
     if (grad_dev)
         CU(launch_net_adam((const float *)P->n_rows.p, n_items, 1.0f, nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 0,
@@ -2686,9 +2695,9 @@ extern "C" pit_status pit_net_loss_grad(pit_problem_t P, double dT, int n_batch,
     if (!ptr_is_device(u) || !ptr_is_device(y)) return fail(PIT_ERR_INVALID_ARG, "u and y must be device memory");
     std::vector<NetTrainItem> items;
     for (int b = 0; b < n_batch; ++b)
-        for (int g = 0; g < P->G; ++g) items.push_back({g, 0, (long long)b * P->ntot + P->off[g]});
+        for (int g = 0; g < P->G; ++g) items.push_back({g, 0, (long long)b * P->ntot + P->off[g], 0});
     CU(P->n_grad.ensure(sizeof(float) * PIT_NET_PARAMS));
-    TRY(net_loss_grad_dev(P, dT, n_batch, u, y, items.data(), (int)items.size(), (const float *)P->n_w.p,
+    TRY(net_loss_grad_dev(P, dT, u, y, items.data(), (int)items.size(), (const float *)P->n_w.p,
                           (float *)P->n_grad.p, loss));
     CU(cudaMemcpyAsync(grad, P->n_grad.p, sizeof(float) * PIT_NET_PARAMS, cudaMemcpyDeviceToHost, P->stream));
     CU(cudaStreamSynchronize(P->stream));
@@ -2756,7 +2765,7 @@ extern "C" pit_status pit_train_coarse(pit_problem_t P, const pit_train_opts *o,
     std::vector<NetTrainItem> train, hold;
     for (int p = 0; p < n_states; ++p)
         for (int g = 0; g < G; ++g) {
-            NetTrainItem it{g, 0, (long long)p * nt + P->off[g]};
+            NetTrainItem it{g, 0, (long long)p * nt + P->off[g], 0};
             if (p < n_train_states) train.push_back(it);
             else hold.push_back(it);
         }
@@ -2801,6 +2810,7 @@ extern "C" pit_status pit_train_coarse(pit_problem_t P, const pit_train_opts *o,
     std::vector<NetTrainItem> order(train);
     for (int ep = 0; ep < o->epochs; ++ep) {
         for (int k = (int)order.size() - 1; k > 0; --k) std::swap(order[k], order[rng.next() % (uint64_t)(k + 1)]);
+        for (int s0 = 0; s0 < (int)order.size(); s0 += B) net_place(P, &order[s0], std::min(B, (int)order.size() - s0));
         CU(cudaMemcpyAsync(P->n_items.p, order.data(), sizeof(NetTrainItem) * order.size(), cudaMemcpyHostToDevice,
                            P->stream));
         int n_loss = 0;
@@ -2809,9 +2819,9 @@ extern "C" pit_status pit_train_coarse(pit_problem_t P, const pit_train_opts *o,
             {
                 ProfScope ps(P, 3);
                 CU(launch_net_train(P->d_grids, (const NetTrainItem *)P->n_items.p + s0, nb, Ud, Yd, dT,
-                                    (const float *)P->n_w.p, (float *)P->n_act.p, slab, (float *)P->n_rows.p,
+                                    (const float *)P->n_w.p, (float *)P->n_act.p, nmax, (float *)P->n_rows.p,
                                     P->n_loss.d() + s0, P->op, P->stream));
-                count_kernels(P, 3);
+                count_kernels(P, 3, 2);
             }
             ++t;
             CU(launch_net_adam((const float *)P->n_rows.p, nb, 1.0f / nb, (float *)P->n_master.p, (float *)P->n_m.p,

@@ -192,6 +192,7 @@ struct NetTrainItem {
     int g;          // grid
     int pad;
     long long off;  // offset of the grid's values in the packed u and y arrays
+    long long act;  // offset of the item's activations in floats (training)
 };
 
 size_t net_smem_bytes(int n);
@@ -200,9 +201,10 @@ cudaError_t net_kernels_init(size_t max_smem);
 // Launches items a.item0 .. a.item0 + n_items - 1.
 cudaError_t launch_net_steps(const StepArgs &a, const NetWeights &W, float *act, long long act_stride, size_t smem,
                              cudaStream_t s, int n_items);
+// n_max: nodes of the largest grid among the items.
 cudaError_t launch_net_train(const GridInfo *grids, const NetTrainItem *items, int n_items, const double *u,
-                             const double *y, double dT, const float *w, float *act, long long act_stride,
-                             float *grad_rows, double *loss_items, OpParams op, cudaStream_t s);
+                             const double *y, double dT, const float *w, float *act, int n_max, float *grad_rows,
+                             double *loss_items, OpParams op, cudaStream_t s);
 // Sums n_rows gradient rows (item order) into grad_out (if non-NULL) and, when
 // master is non-NULL, takes one Adam step on the master weights (gradient
 // scaled by `scale`) and writes their BF16 rounding to w_bf16.

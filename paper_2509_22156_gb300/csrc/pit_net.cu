@@ -84,27 +84,28 @@ cudaError_t launch_net_steps(const StepArgs &a, const NetWeights &W, float *act,
 }
 
 cudaError_t launch_net_train(const GridInfo *grids, const NetTrainItem *items, int n_items, const double *u,
-                             const double *y, double dT, const float *w, float *act, long long act_stride,
-                             float *grad_rows, double *loss_items, OpParams op, cudaStream_t s)
+                             const double *y, double dT, const float *w, float *act, int n_max, float *grad_rows,
+                             double *loss_items, OpParams op, cudaStream_t s)
 {
     if (n_items <= 0) return cudaSuccess;
+    if (n_items > 0x1fffffff) return cudaErrorInvalidConfiguration;
     const NetTrainItem *it = items;
     const dim3 grid(n_items);
-    // activations on chip for the items that fit (act_stride holds those of the
-    // problem's largest grid, so small problems take less shared memory)
-    const size_t tile = (size_t)net_tile_words() * 4;
-    size_t room = std::min((size_t)act_stride * 4, (size_t)net_train_words(NET_CHIP) * 4);
+    // activations on chip for the items that fit (small problems take less shared
+    // memory)
+    const size_t tile = 85 * 16 * 4;
+    size_t room = (size_t)net_chip_words(std::min(n_max, NET_CHIP)) * 4;
     if (tile + room > g_net_max_smem) room = g_net_max_smem > tile ? g_net_max_smem - tile : 0;
     int n_chip = 0;
-    while (net_train_words(n_chip + 4) * 4ull <= room) n_chip += 4;
+    while (net_chip_words(n_chip + 4) * 4ull <= room) n_chip += 4;
     const size_t smem = tile + room;
     switch (op.d) {
-    case 1: net_launch_train_d1(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
-    case 2: net_launch_train_d2(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
-    case 3: net_launch_train_d3(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
-    case 4: net_launch_train_d4(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
-    case 5: net_launch_train_d5(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
-    case 6: net_launch_train_d6(grids, it, u, y, dT, w, act, act_stride, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 1: net_launch_train_d1(grids, it, u, y, dT, w, act, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 2: net_launch_train_d2(grids, it, u, y, dT, w, act, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 3: net_launch_train_d3(grids, it, u, y, dT, w, act, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 4: net_launch_train_d4(grids, it, u, y, dT, w, act, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 5: net_launch_train_d5(grids, it, u, y, dT, w, act, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
+    case 6: net_launch_train_d6(grids, it, u, y, dT, w, act, n_chip, grad_rows, loss_items, op, grid, smem, s); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

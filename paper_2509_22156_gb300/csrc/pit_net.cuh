@@ -222,22 +222,31 @@ __global__ void __launch_bounds__(256) net_steps_kernel(StepArgs a, const __grid
 //
 // What bounds it: shared-memory reads beside the FMAs of the three 85 x 16
 // products a node and layer (forward, input gradient, weight gradient; FP32
-// throughout, weights BF16-rounded).  Activations (51 channels, the gradient of
-// a layer's input overwriting that input) and the layer's weights, transposed
-// so that one 16-byte read gives four outputs' weights, are on chip up to 940
-// nodes and in the item's global slab beyond; neighbour indices of a node are
-// worked out once a pass, a missing tap pointing at a zero element of its row;
-// two nodes a thread share every weight read.  The weight gradient takes tiles
-// of 64 nodes: axis sums of every (channel, tap) row and the output gradients
-// in shared memory, then every thread sums eight outputs of one row over half
-// of the tile.  varheat3d level 8 (85 grids of up to 735 nodes), the whole call
-// with its copies: 1,263 us when every FMA read its own weight from global
-// memory and every row's thread formed its own axis sums, 401 us now.
+// throughout, weights BF16-rounded), and the largest grid, one CTA working on
+// it.  Two kernels: net_train_kernel takes an item forward and back to every
+// layer's output gradient, net_wgrad_kernel one (item, layer) to its weight
+// gradient, so that the layers' sums run on different SMs.  In the first,
+// activations (51 channels, the gradient of a layer's input overwriting that
+// input) and the layer's weights, transposed so that one 16-byte read gives
+// four outputs' weights, are on chip up to 940 nodes and in the item's global
+// slab beyond; neighbour indices of a node are worked out once a pass, a missing
+// tap pointing at a zero element of its row; two nodes a thread share every
+// weight read.  The weight gradient takes tiles of 64 nodes: axis sums of every
+// (channel, tap) row and the output gradients in shared memory, then every
+// thread sums eight outputs of one row over half of the tile.
+// varheat3d level 8 (85 grids of up to 735 nodes), the whole call with its
+// copies: 1,263 us when every FMA read its own weight from global memory and
+// every row's thread formed its own axis sums, 401 us with both parts in one
+// kernel, 286 us now.
 constexpr int NET_THREADS = 512, NET_TILE = 64, NET_TLD = NET_TILE + 4;
 constexpr int NET_CHIP = 940;  // largest grid whose activations stay on chip
 __host__ __device__ constexpr int net_ld(int n) { return (n + 4) & ~3; }  // one zero element past the nodes
-__host__ __device__ constexpr int net_train_words(int n) { return 52 * net_ld(n); }
-__host__ __device__ constexpr int net_tile_words() { return 85 * 16 + (86 + 16) * NET_TLD; }
+__host__ __device__ constexpr int net_chip_words(int n) { return 52 * net_ld(n); }
+// an item's global slab: input (2 channels), H1..H3, the output gradients of
+// the last layer (1) and of layers 0..2 (16 each), tap masks
+__host__ __device__ constexpr int net_train_words(int n) { return 100 * net_ld(n); }
+__host__ __device__ constexpr int net_h_row(int k) { return 2 + 16 * k; }               // output of layer k < 3
+__host__ __device__ constexpr int net_d_row(int k) { return k == 3 ? 50 : 51 + 16 * k; }  // gradient of its pre-activations
 
 // Indices of a node's neighbours at offsets -2, -1, +1, +2 along every axis
 // (zero: the index of the zero element).
@@ -306,8 +315,10 @@ struct NetItem {  // one item's geometry and buffers
 };
 
 // out[o][j] of one layer: ReLU of 16 channels, or the last layer's single one
+// (copy: second place of the output, or NULL)
 template <int D>
-__device__ __forceinline__ void net_layer(const NetItem<D> &I, int k, const float *w, const float *in, float *out)
+__device__ __forceinline__ void net_layer(const NetItem<D> &I, int k, const float *w, const float *in, float *out,
+                                          float *copy)
 {
     const int cin = net_cin(k), cout = net_cout(k), wo = net_wo(k), bo = net_bo(k), nt = blockDim.x;
     __syncthreads();  // in complete, wt free
@@ -367,8 +378,13 @@ __device__ __forceinline__ void net_layer(const NetItem<D> &I, int k, const floa
         } else {
 #pragma unroll
             for (int o = 0; o < 16; ++o) {
-                out[o * I.ld + j0] = fmaxf(a0[o], 0.0f);
-                if (two) out[o * I.ld + j1] = fmaxf(a1[o], 0.0f);
+                const float h0 = fmaxf(a0[o], 0.0f), h1 = fmaxf(a1[o], 0.0f);
+                out[o * I.ld + j0] = h0;
+                if (two) out[o * I.ld + j1] = h1;
+                if (copy) {
+                    copy[o * I.ld + j0] = h0;
+                    if (two) copy[o * I.ld + j1] = h1;
+                }
             }
         }
     }
@@ -456,10 +472,11 @@ __device__ __forceinline__ void net_weight_grad(const NetItem<D> &I, int k, cons
 }
 
 // Gradient of the layer's 16 input channels through the ReLU of the layer
-// before, in place of that layer's output h:
+// before, whose output is h, into out (may be h) and copy (or NULL):
 // din[c][j] = sum_t sum_o W[o][c][t] sum_i dc[o][j - (t-2) e_i].
 template <int D>
-__device__ __forceinline__ void net_input_grad(const NetItem<D> &I, int k, const float *w, const float *dc, float *h)
+__device__ __forceinline__ void net_input_grad(const NetItem<D> &I, int k, const float *w, const float *dc, const float *h,
+                                               float *out, float *copy)
 {
     const int cout = net_cout(k), wo = net_wo(k), nt = blockDim.x;
     __syncthreads();  // wt and the tiles free, dc and h read
@@ -481,31 +498,49 @@ __device__ __forceinline__ void net_input_grad(const NetItem<D> &I, int k, const
         net_conv16<D>(dc, cout, I.ld, wt, j0, j1, x0, x1, a0, a1);
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
-            h[c * I.ld + j0] = h[c * I.ld + j0] > 0.0f ? a0[c] : 0.0f;
-            if (two) h[c * I.ld + j1] = h[c * I.ld + j1] > 0.0f ? a1[c] : 0.0f;
+            const float d0 = h[c * I.ld + j0] > 0.0f ? a0[c] : 0.0f;
+            out[c * I.ld + j0] = d0;
+            if (copy) copy[c * I.ld + j0] = d0;
+            if (two) {
+                const float d1 = h[c * I.ld + j1] > 0.0f ? a1[c] : 0.0f;
+                out[c * I.ld + j1] = d1;
+                if (copy) copy[c * I.ld + j1] = d1;
+            }
         }
     }
 }
 
-template <int D>
+// slab: the item's global slab; chip: on-chip activations, or NULL
+template <int D, bool CHIP>
 __device__ __forceinline__ void net_train_item(const GridInfo &GI, const int *S, const float *sf, double *red, float *tiles,
-                                               float *acts, const NetTrainItem &it, const double *u, const double *y,
-                                               const float *w, float *grow, double *loss, const OpParams &op)
+                                               float *chip, float *slab, const NetTrainItem &it, const double *u,
+                                               const double *y, const float *w, double *loss, const OpParams &op)
 {
     const int tid = threadIdx.x, nt = blockDim.x, n = GI.n, ld = net_ld(n);
-    // channels: A0 (2), H1..H3 (16 each), O, then the masks
-    float *A0 = acts, *H1 = acts + 2 * ld, *H2 = H1 + 16 * ld, *H3 = H2 + 16 * ld, *O = H3 + 16 * ld;
-    uint32_t *mk = reinterpret_cast<uint32_t *>(O + ld);
-    NetItem<D> I{n, ld, S, sf, mk, tiles, tiles + 85 * 16, tiles + 85 * 16 + 86 * NET_TLD};
+    float *acts = CHIP ? chip : slab;
+    float *A0 = acts, *H1 = acts + net_h_row(0) * ld, *H2 = acts + net_h_row(1) * ld, *H3 = acts + net_h_row(2) * ld;
+    float *O = acts + net_d_row(3) * ld;
+    uint32_t *mkg = reinterpret_cast<uint32_t *>(slab + 99 * ld);
+    uint32_t *mk = CHIP ? reinterpret_cast<uint32_t *>(chip + 51 * ld) : mkg;
+    NetItem<D> I{n, ld, S, sf, mk, tiles, nullptr, nullptr};
     const double *ui = u + it.off, *yi = y + it.off;
     double ss = 0.0, yy = 0.0;
     for (int j = tid; j < n; j += nt) {
-        mk[j] = ext_mask<D>(GI, j);
-        A0[ld + j] = (float)node_coef(op, GI, j, D);
+        const uint32_t m = ext_mask<D>(GI, j);
+        const float c = (float)node_coef(op, GI, j, D);
+        mk[j] = m;
+        A0[ld + j] = c;
+        if (CHIP) {
+            mkg[j] = m;
+            slab[ld + j] = c;
+        }
         ss += ui[j] * ui[j];
         yy += yi[j] * yi[j];
     }
-    for (int c = tid; c < 51; c += nt) acts[c * ld + n] = 0.0f;  // the zero element of every row
+    for (int c = tid; c < 99; c += nt) {  // the zero element of every row
+        slab[c * ld + n] = 0.0f;
+        if (CHIP && c < 51) chip[c * ld + n] = 0.0f;
+    }
     ss = block_sum64(ss, red);
     yy = block_sum64(yy, red);
     const double sigma = sqrt(ss / (double)n);
@@ -515,40 +550,44 @@ __device__ __forceinline__ void net_train_item(const GridInfo &GI, const int *S,
         double l = 0.0;
         for (int j = tid; j < n; j += nt) l += (ui[j] - yi[j]) * (ui[j] - yi[j]);
         l = block_sum64(l, red);
-        for (int p = tid; p < PIT_NET_PARAMS; p += nt) grow[p] = 0.0f;
+        for (int q = tid; q < 99 * ld; q += nt) slab[q] = 0.0f;
         if (tid == 0) *loss = l / yy;
         return;
     }
     const double inv = 1.0 / sigma;
-    for (int j = tid; j < n; j += nt) A0[j] = (float)(ui[j] * inv);
-    net_layer<D>(I, 0, w, A0, H1);
-    net_layer<D>(I, 1, w, H1, H2);
-    net_layer<D>(I, 2, w, H2, H3);
-    net_layer<D>(I, 3, w, H3, O);
+    for (int j = tid; j < n; j += nt) {
+        const float v = (float)(ui[j] * inv);
+        A0[j] = v;
+        if (CHIP) slab[j] = v;
+    }
+    auto copy = [&](int row) -> float * { return CHIP ? slab + row * ld : nullptr; };
+    net_layer<D>(I, 0, w, A0, H1, copy(net_h_row(0)));
+    net_layer<D>(I, 1, w, H1, H2, copy(net_h_row(1)));
+    net_layer<D>(I, 2, w, H2, H3, copy(net_h_row(2)));
+    net_layer<D>(I, 3, w, H3, O, nullptr);
     __syncthreads();
     // loss and dL/d(layer-4 pre-activation) = 2 e sigma / ||y||^2
     double l = 0.0;
     for (int j = tid; j < n; j += nt) {
         const double e = ui[j] + sigma * (double)O[j] - yi[j];
         l += e * e;
-        O[j] = (float)(2.0 * e * sigma / yy);
+        const float d = (float)(2.0 * e * sigma / yy);
+        O[j] = d;
+        if (CHIP) slab[net_d_row(3) * ld + j] = d;
     }
     l = block_sum64(l, red);
     if (tid == 0) *loss = l / yy;
-    net_weight_grad<D>(I, 3, H3, O, grow);
-    net_input_grad<D>(I, 3, w, O, H3);
-    net_weight_grad<D>(I, 2, H2, H3, grow);
-    net_input_grad<D>(I, 2, w, H3, H2);
-    net_weight_grad<D>(I, 1, H1, H2, grow);
-    net_input_grad<D>(I, 1, w, H2, H1);
-    net_weight_grad<D>(I, 0, A0, H1, grow);
+    float *D2 = CHIP ? H3 : slab + net_d_row(2) * ld, *D1 = CHIP ? H2 : slab + net_d_row(1) * ld;
+    float *D0 = CHIP ? H1 : slab + net_d_row(0) * ld;
+    net_input_grad<D>(I, 3, w, O, H3, D2, copy(net_d_row(2)));
+    net_input_grad<D>(I, 2, w, D2, H2, D1, copy(net_d_row(1)));
+    net_input_grad<D>(I, 1, w, D1, H1, D0, copy(net_d_row(0)));
 }
 
 template <int D>
 __global__ void __launch_bounds__(NET_THREADS, 1)
     net_train_kernel(const GridInfo *grids, const NetTrainItem *items, const double *u, const double *y, double dT,
-                     const float *w, float *act, long long act_stride, int n_chip, float *grad_rows, double *loss_items,
-                     OpParams op)
+                     const float *w, float *act, int n_chip, double *loss_items, OpParams op)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ GridInfo GI;
@@ -564,14 +603,33 @@ __global__ void __launch_bounds__(NET_THREADS, 1)
         sf[tid] = (float)(1.0 / (1.0 + 4.0 * dT / (GI.h[tid] * GI.h[tid])));
     }
     __syncthreads();
-    float *tiles = reinterpret_cast<float *>(smem);
-    float *grow = grad_rows + (long long)blockIdx.x * PIT_NET_PARAMS;
+    float *tiles = reinterpret_cast<float *>(smem), *slab = act + it.act;
     // (two calls, so that the one on chip uses shared-memory instructions)
     if (GI.n <= n_chip)
-        net_train_item<D>(GI, S, sf, red, tiles, tiles + net_tile_words(), it, u, y, w, grow, loss_items + blockIdx.x, op);
+        net_train_item<D, true>(GI, S, sf, red, tiles, tiles + 85 * 16, slab, it, u, y, w, loss_items + blockIdx.x, op);
     else
-        net_train_item<D>(GI, S, sf, red, tiles, act + (long long)blockIdx.x * act_stride, it, u, y, w, grow,
-                          loss_items + blockIdx.x, op);
+        net_train_item<D, false>(GI, S, sf, red, tiles, nullptr, slab, it, u, y, w, loss_items + blockIdx.x, op);
+}
+
+// One CTA per (item, layer).
+template <int D>
+__global__ void __launch_bounds__(NET_THREADS, 2)
+    net_wgrad_kernel(const GridInfo *grids, const NetTrainItem *items, double dT, const float *act, float *grad_rows)
+{
+    __shared__ __align__(16) float tiles[(86 + 16) * NET_TLD];
+    __shared__ int S[D];
+    __shared__ float sf[D];
+    const int item = blockIdx.x >> 2, k = 3 - (int)(blockIdx.x & 3);
+    const GridInfo &GI = grids[items[item].g];
+    if (threadIdx.x < D) {
+        S[threadIdx.x] = GI.S[threadIdx.x];
+        sf[threadIdx.x] = (float)(1.0 / (1.0 + 4.0 * dT / (GI.h[threadIdx.x] * GI.h[threadIdx.x])));
+    }
+    const int n = GI.n, ld = net_ld(n);
+    const float *slab = act + items[item].act;
+    const NetItem<D> I{n, ld, S, sf, reinterpret_cast<const uint32_t *>(slab + 99 * ld), nullptr, tiles, tiles + 86 * NET_TLD};
+    net_weight_grad<D>(I, k, k == 0 ? slab : slab + net_h_row(k - 1) * ld, slab + net_d_row(k) * ld,
+                       grad_rows + (long long)item * PIT_NET_PARAMS);
 }
 
 // Per-dimension launchers (one translation unit per d, pit_net_d<d>.cu).
@@ -580,9 +638,8 @@ __global__ void __launch_bounds__(NET_THREADS, 1)
     void net_launch_steps_d##D(const StepArgs &a, const NetWeights &W, float *act, long long act_stride,         \
                                dim3 grid, dim3 block, size_t smem, cudaStream_t s);                              \
     void net_launch_train_d##D(const GridInfo *grids, const NetTrainItem *it, const double *u, const double *y,   \
-                               double dT, const float *w, float *act, long long act_stride, int n_chip,          \
-                               float *grad_rows, double *loss_items, OpParams op, dim3 grid, size_t smem,        \
-                               cudaStream_t s);
+                               double dT, const float *w, float *act, int n_chip, float *grad_rows,              \
+                               double *loss_items, OpParams op, dim3 grid, size_t smem, cudaStream_t s);
 PIT_NET_DECL(1) PIT_NET_DECL(2) PIT_NET_DECL(3) PIT_NET_DECL(4) PIT_NET_DECL(5) PIT_NET_DECL(6)
 
 #define PIT_NET_DIM(D)                                                                                           \
@@ -598,12 +655,11 @@ PIT_NET_DECL(1) PIT_NET_DECL(2) PIT_NET_DECL(3) PIT_NET_DECL(4) PIT_NET_DECL(5) 
         net_steps_kernel<D><<<grid, block, smem, s>>>(a, W, act, act_stride);                                    \
     }                                                                                                            \
     void net_launch_train_d##D(const GridInfo *grids, const NetTrainItem *it, const double *u, const double *y,   \
-                               double dT, const float *w, float *act, long long act_stride, int n_chip,          \
-                               float *grad_rows, double *loss_items, OpParams op, dim3 grid, size_t smem,        \
-                               cudaStream_t s)                                                                   \
+                               double dT, const float *w, float *act, int n_chip, float *grad_rows,              \
+                               double *loss_items, OpParams op, dim3 grid, size_t smem, cudaStream_t s)          \
     {                                                                                                            \
-        net_train_kernel<D><<<grid, NET_THREADS, smem, s>>>(grids, it, u, y, dT, w, act, act_stride, n_chip,     \
-                                                            grad_rows, loss_items, op);                          \
+        net_train_kernel<D><<<grid, NET_THREADS, smem, s>>>(grids, it, u, y, dT, w, act, n_chip, loss_items, op); \
+        net_wgrad_kernel<D><<<dim3(grid.x * 4), NET_THREADS, 0, s>>>(grids, it, dT, act, grad_rows); \
     }
 
 }  // namespace pit
