@@ -6,8 +6,9 @@
 // Dirichlet values, so the discrete sine transform (DST-I) along an axis
 // diagonalises that axis' part.  A solve transforms every axis but the longest
 // one, solves the remaining independent systems along the longest axis and
-// transforms back: 2 de - 1 passes over the vector (de the axes with more than
-// one node), each with one barrier and no reduction.  On the component grids
+// transforms back: at most 2 de - 1 passes over the vector (de the axes with
+// more than one node; two short axes share one), each with one barrier and no
+// reduction.  On the component grids
 // of the combination technique the other axes are short (at most 31 nodes up
 // to level 10 in two dimensions, 15 on most grids), so a transform is a few
 // multiplications a node, done line by line in registers.
@@ -104,8 +105,9 @@ __device__ __forceinline__ void dst(float (&v)[N])
 // ----------------------------------------------------------------------------
 // The direct solve of one item, set up once per launch.
 struct Direct {
-    int n, nax;                  // nodes; transformed axes
-    int N[PIT_D], S[PIT_D];      // transformed axes: nodes and strides
+    int n, nax;                  // nodes; transforms
+    int N[PIT_D], S[PIT_D];      // transformed axis: nodes and stride
+    int N2[PIT_D], S2[PIT_D];    // a second, inner one taken by the same pass (N2 = 1: none)
     int Na, Sa, nl;              // longest axis: nodes, stride, lines
     int P, L;                    // long lines (Na > 31): chunks a line, chunk length
     float norm;                  // product of 2 / (N + 1) over the transforms
@@ -145,9 +147,23 @@ __device__ __forceinline__ void direct_setup(const GridInfo &G, const ItemConst 
         float norm = 1.0f;
         for (int q = 0; q < G.de; ++q) {
             if (q == la) continue;
-            D.N[nax] = G.N[G.ax[q]];
-            D.S[nax] = G.S[G.ax[q]];
-            norm *= 2.0f / (float)(D.N[nax] + 1);
+            const int N = G.N[G.ax[q]], S = G.S[G.ax[q]];
+            norm *= 2.0f / (float)(N + 1);
+            // a short axis joins an earlier pass over a short axis: 9 or 21
+            // values a thread, and a barrier and a trip through shared memory
+            // less each way
+            int at = nax;
+            for (int i = 0; i < nax; ++i)
+                if (D.N2[i] == 1 && D.N[i] * N <= 21 && at == nax) at = i;
+            if (at < nax) {
+                D.N2[at] = N;
+                D.S2[at] = S;
+                continue;
+            }
+            D.N[nax] = N;
+            D.S[nax] = S;
+            D.N2[nax] = 1;
+            D.S2[nax] = 0;
             ++nax;
         }
         D.nax = nax;
@@ -205,6 +221,33 @@ __device__ __forceinline__ void dst_lines(const Direct &D, float *v, int S)
         dst<N>(w);
 #pragma unroll
         for (int k = 0; k < N; ++k) p[k * S] = w[k];
+    }
+}
+// two axes at once, S2 < S1 (the inner axis' lines lie inside one step of the
+// outer one)
+template <int N1, int N2>
+__device__ __forceinline__ void dst_slabs(const Direct &D, float *v, int S1, int S2)
+{
+    const int ns = D.n / (N1 * N2);
+    const float inv1 = 1.0f / (float)S1, inv2 = 1.0f / (float)S2;
+    for (int l = threadIdx.x; l < ns; l += blockDim.x) {
+        float *p = v + line_start(line_start(l, N2, S2, inv2), N1, S1, inv1);
+        float w[N1][N2];
+#pragma unroll
+        for (int i = 0; i < N1; ++i) {
+#pragma unroll
+            for (int k = 0; k < N2; ++k) w[i][k] = p[i * S1 + k * S2];
+            dst<N2>(w[i]);
+        }
+#pragma unroll
+        for (int k = 0; k < N2; ++k) {
+            float c[N1];
+#pragma unroll
+            for (int i = 0; i < N1; ++i) c[i] = w[i][k];
+            dst<N1>(c);
+#pragma unroll
+            for (int i = 0; i < N1; ++i) p[i * S1 + k * S2] = c[i];
+        }
     }
 }
 // longest axis of at most 31 nodes: transform, divide by the eigenvalues, back
@@ -345,10 +388,17 @@ __device__ __forceinline__ void direct_solve(float *v, float mul)
             default: wide_pass((int)(v - smem_f()), mul, 0); break;
             }
         } else {
-            const int i = pass < D.nax ? pass : 2 * D.nax - pass, S = D.S[i];
+            const int i = pass < D.nax ? pass : 2 * D.nax - pass, S = D.S[i], N2 = D.N2[i];
             switch (D.N[i]) {
-            case 3: dst_lines<3>(D, v, S); break;
-            case 7: dst_lines<7>(D, v, S); break;
+            case 3:
+                if (N2 == 1) dst_lines<3>(D, v, S);
+                else if (N2 == 3) dst_slabs<3, 3>(D, v, S, D.S2[i]);
+                else dst_slabs<3, 7>(D, v, S, D.S2[i]);
+                break;
+            case 7:
+                if (N2 == 1) dst_lines<7>(D, v, S);
+                else dst_slabs<7, 3>(D, v, S, D.S2[i]);
+                break;
             case 15: dst_lines<15>(D, v, S); break;
             default: wide_pass((int)(v - smem_f()), mul, S); break;
             }
