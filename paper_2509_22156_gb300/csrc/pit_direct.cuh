@@ -463,7 +463,8 @@ __global__ void __launch_bounds__(512, 1) direct_kernel(const __grid_constant__ 
     __shared__ GridInfo GI;
     __shared__ ItemConst IC;
     __shared__ double red64[2 * 128];
-    __shared__ float red32[2 * 128];
+    __shared__ __align__(16) float red32[2 * 128];
+    for (int t = threadIdx.x; t < 256; t += blockDim.x) red32[t] = 0.0f;
     static_assert(PREC == MIXED || PREC == PAIR, "the refinement forms");
     const int item = a.item0 + (int)blockIdx.x;
     const int g = a.order[item / a.n_batch];
@@ -500,7 +501,7 @@ __global__ void __launch_bounds__(512, 1) direct_kernel(const __grid_constant__ 
     const double *f0 = a.f ? a.f + (long long)b * a.f_stride + GI.off : nullptr;
     const uint16_t *gmask = a.masks + GI.off;
     Reducer<double> R64{red64, 0};
-    Reducer<float> R32{red32, 0};
+    Reducer<float, true> R32{red32, 0};
     int ks = 0;  // PAIR: the state is held times 2^ks
     if constexpr (PREC == PAIR) {
         const double *g0 = a.g ? a.g + (long long)b * a.g_stride + GI.off : nullptr;

@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
     __shared__ ItemConst IC;
     FixConst &FC = fix_s;
     __shared__ double red64[2 * 128];
-    __shared__ float red32[2 * 128];
+    __shared__ __align__(16) float red32[2 * 128];
+    for (int t = threadIdx.x; t < 256; t += blockDim.x) red32[t] = 0.0f;
     const int item = a.item0 + (int)blockIdx.x;
     const int g = a.order[item / a.n_batch];
     const int b = item % a.n_batch;
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
     uint16_t *mask = reinterpret_cast<uint16_t *>(rv + ld);
     direct_setup(GI, IC, (int)(reinterpret_cast<float *>(mask + ld) - smem_f()));
     Reducer<double> R64{red64, 0};
-    Reducer<float> R32{red32, 0};
+    Reducer<float, true> R32{red32, 0};
 
     const double *in = a.in + (long long)b * a.in_stride + GI.off;
     const uint16_t *gmask = a.masks + GI.off;

@@ -259,9 +259,9 @@ __device__ __forceinline__ T warp_sum(T v)
     return v;
 }
 
-template <typename T>
+template <typename T, bool ALL = false>
 struct Reducer {
-    T *buf;    // two halves of 4 x 32 slots
+    T *buf;    // two halves of 4 x 32 slots (ALL: zero at the start, 16-byte aligned)
     int slot;
     // first stage: warp sums into the current half; returns that half
     template <int K>
@@ -278,10 +278,29 @@ struct Reducer {
         }
         return red;
     }
-    // second stage, after the barrier: sum of the nw warp partials
+    // second stage, after the barrier: sum of the nw warp partials.  ALL: every
+    // thread reads and adds them all, in a third of the shuffles' latency.  The
+    // kernels with one or two reductions a step gain by it (heat6d_n9 12.2 -> 11.6
+    // ms); the Krylov loops lose more by the longer code (ou4d_n7 4.9 -> 6.0 ms).
     template <int K>
     __device__ __forceinline__ void stage2(const T *red, T *v)
     {
+        if constexpr (ALL) {
+            static_assert(sizeof(T) == 4, "an FP64 addition holds the unit for every warp that makes it");
+            const int nw = blockDim.x >> 5;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const float4 *q = reinterpret_cast<const float4 *>(red + k * 32);
+                const float4 a = q[0];
+                float s = (a.x + a.y) + (a.z + a.w);
+                for (int w = 4; w < nw; w += 4) {
+                    const float4 b = q[w / 4];
+                    s += (b.x + b.y) + (b.z + b.w);
+                }
+                v[k] = s;
+            }
+            return;
+        }
         const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
         const int top = 1 << (32 - __clz(nw - 1));  // nw rounded up to a power of two
 #pragma unroll
