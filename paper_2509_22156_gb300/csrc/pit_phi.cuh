@@ -630,7 +630,10 @@ __device__ int cg_core(const ST &A, int n, TX *X, T *r, T *p, T *s, T *w, Reduce
         status = (v[1] != v[1]) ? PIT_ERR_NONFINITE : PIT_ERR_BREAKDOWN;
         return 0;
     }
-    T alpha = gam / v[1], beta = T(0);
+    // den: the denominator of alpha.  beta rr / alpha = beta^2 den of the last
+    // iteration (alpha = gam / den, beta = rr / gam), so an iteration divides
+    // twice, and beta while the stencil pass runs.
+    T den = v[1], alpha = gam / den, beta = T(0);
     bool first = true;
     int k = 0;
     for (;;) {
@@ -656,6 +659,7 @@ __device__ int cg_core(const ST &A, int n, TX *X, T *r, T *p, T *s, T *w, Reduce
             if (rr[0] != rr[0]) status = PIT_ERR_NONFINITE;
             break;
         }
+        beta = rr[0] / gam;
         T wr[1] = {T(0)};
 #pragma unroll 4
         for (int j = tid; j < n; j += nt) {
@@ -664,8 +668,7 @@ __device__ int cg_core(const ST &A, int n, TX *X, T *r, T *p, T *s, T *w, Reduce
             wr[0] += wj * r[j];
         }
         R.template sum<1>(wr);
-        beta = rr[0] / gam;
-        const T den = wr[0] - beta * rr[0] / alpha;
+        den = wr[0] - beta * beta * den;
         if (!finite_pos(den)) { status = (den != den) ? PIT_ERR_NONFINITE : PIT_ERR_BREAKDOWN; break; }
         alpha = rr[0] / den;
         gam = rr[0];
@@ -888,7 +891,7 @@ __device__ int pcg_core(const ST &A, const PC &M, int n, TX *X, T *r, T *u, T *p
         status = (v[1] != v[1] || v[2] != v[2]) ? PIT_ERR_NONFINITE : PIT_ERR_BREAKDOWN;
         return 0;
     }
-    T gam = v[1], alpha = v[1] / v[2], beta = T(0);
+    T gam = v[1], den = v[2], alpha = gam / den, beta = T(0);  // (den as in cg_core)
     bool first = true;
     int k = 0;
     for (;;) {
@@ -928,7 +931,7 @@ __device__ int pcg_core(const ST &A, const PC &M, int n, TX *X, T *r, T *u, T *p
         R.template sum<2>(q);
         if (!finite_pos(q[0])) { status = (q[0] != q[0]) ? PIT_ERR_NONFINITE : PIT_ERR_BREAKDOWN; break; }
         beta = q[0] / gam;
-        const T den = q[1] - beta * q[0] / alpha;
+        den = q[1] - beta * beta * den;
         if (!finite_pos(den)) { status = (den != den) ? PIT_ERR_NONFINITE : PIT_ERR_BREAKDOWN; break; }
         alpha = q[0] / den;
         gam = q[0];
@@ -948,11 +951,12 @@ __device__ int pcg_core(const ST &A, const PC &M, int n, TX *X, T *r, T *u, T *p
 // (ZX as for cg_core)
 template <bool ZX, typename T, typename TX, class ST>
 __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v, T *t, Reducer<T> &R, T stop2,
-                             int maxit, int &status)
+                             int maxit, int &status, T rr0 = T(-1))
 {
     const int tid = threadIdx.x, nt = blockDim.x;
     // cosine below which (rh, r) counts as a breakdown
     const T near0 = sizeof(T) == 8 ? T(1e-12) : T(1e-6);
+    // (rr0 >= 0: (r, r) as the caller knows it)
     T rr[1] = {T(0)};
 #pragma unroll 4
     for (int j = tid; j < n; j += nt) {
@@ -962,8 +966,10 @@ __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v,
         v[j] = T(0);
         rr[0] += rj * rj;
     }
-    R.template sum<1>(rr);
-    T rho = T(1), alpha = T(1), omega = T(1), rrv = rr[0], rhh = rr[0];
+    if (rr0 >= T(0)) rr[0] = rr0;
+    else R.template sum<1>(rr);
+    // rho_n = (rh, r), summed with (r, r) where r is formed
+    T rho = T(1), alpha = T(1), omega = T(1), rrv = rr[0], rhh = rr[0], rho_n = rr[0];
     int k = 0, k_restart = -1;
     status = PIT_OK;
     // restart from the current residual (every thread reads and writes only
@@ -977,7 +983,7 @@ __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v,
             v[j] = T(0);
         }
         rho = alpha = omega = T(1);
-        rhh = rrv;
+        rhh = rho_n = rrv;
         return true;
     };
     for (;;) {
@@ -986,17 +992,13 @@ __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v,
             break;
         }
         if (k >= maxit) { status = PIT_ERR_NOCONV; break; }
-        T rho_n[1] = {T(0)};
-#pragma unroll 4
-        for (int j = tid; j < n; j += nt) rho_n[0] += rh[j] * r[j];
-        R.template sum<1>(rho_n);
-        if (rho_n[0] != rho_n[0]) { status = PIT_ERR_NONFINITE; break; }
-        if (!(fabs(rho_n[0]) > near0 * sqrt(rrv) * sqrt(rhh))) {
+        if (rho_n != rho_n) { status = PIT_ERR_NONFINITE; break; }
+        if (!(fabs(rho_n) > near0 * sqrt(rrv) * sqrt(rhh))) {
             if (restart()) continue;
             status = PIT_ERR_BREAKDOWN;
             break;
         }
-        const T beta = (rho_n[0] / rho) * (alpha / omega);
+        const T beta = (rho_n / rho) * (alpha / omega);
         if (beta != beta) { status = PIT_ERR_NONFINITE; break; }
         if (!(fabs(beta) < (T)1e30)) {
             if (restart()) continue;
@@ -1015,7 +1017,7 @@ __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v,
         }
         R.template sum<1>(rhv);
         if (rhv[0] != rhv[0]) { status = PIT_ERR_NONFINITE; break; }
-        alpha = rho_n[0] / rhv[0];
+        alpha = rho_n / rhv[0];
         if (!(fabs(alpha) < (T)1e30)) {
             if (restart()) continue;
             status = PIT_ERR_BREAKDOWN;
@@ -1036,7 +1038,7 @@ __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v,
         omega = (tt[0] > T(0)) ? tt[1] / tt[0] : T(0);
         if (omega != omega) { status = PIT_ERR_NONFINITE; break; }
         if (!(fabs(omega) < (T)1e30)) omega = T(0);  // take the BiCG half step only
-        T rn[1] = {T(0)};
+        T rn[2] = {T(0), T(0)};
 #pragma unroll 4
         for (int j = tid; j < n; j += nt) {
             const TX dx = (TX)(alpha * p[j] + omega * r[j]);
@@ -1044,10 +1046,12 @@ __device__ int bicgstab_core(const ST &A, int n, TX *X, T *r, T *rh, T *p, T *v,
             const T rj = r[j] - omega * t[j];
             r[j] = rj;
             rn[0] += rj * rj;
+            rn[1] += rh[j] * rj;
         }
-        R.template sum<1>(rn);
-        rho = rho_n[0];
+        R.template sum<2>(rn);
+        rho = rho_n;
         rrv = rn[0];
+        rho_n = rn[1];
         ++k;
         if (omega == T(0) && rrv > stop2) {
             if (rrv != rrv) { status = PIT_ERR_NONFINITE; break; }
@@ -1927,7 +1931,7 @@ __device__ __forceinline__ void steps_item(const StepArgs &a, const GridInfo &GI
                     if (scaled)
                         for (int j = tid; j < n; j += nt) rv[j] *= jac ? inv * tab32[j] : inv;
                     int st, k;
-                    if constexpr (DRIFT) k = bicgstab_core<true>(T32, n, e, rv, pv, sv, wv, tv, R32, stop32, a.maxit, st);
+                    if constexpr (DRIFT) k = bicgstab_core<true>(T32, n, e, rv, pv, sv, wv, tv, R32, stop32, a.maxit, st, jac ? -1.0f : R2n);
                     else if constexpr (OP == PIT_OP_HEAT) {
                         if (use_pc) k = pcg_core<true>(HT, LM, n, e, rv, f32 + 5 * ld, pv, sv, wv, R32, stop32, a.maxit, st, !scaled);
                         else k = cg_core<true>(HT, n, e, rv, pv, sv, wv, R32, stop32, a.maxit, st, !scaled);
