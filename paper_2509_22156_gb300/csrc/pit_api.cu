@@ -556,7 +556,10 @@ pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_op
         slot = P->forced_threads[wide ? 1 : 0];
         return PIT_OK;
     }
-    const int cand[4] = {64, 128, 256, 512};
+    // (one warp: grids of a few dozen nodes, whose steps are a chain of reductions
+    // that then wait for no other warp; a trial that larger grids need not pay)
+    const int cand[5] = {32, 64, 128, 256, 512};
+    const int first = v.smem < 4096 ? 0 : 1;
     CU(P->w_tune.ensure(sizeof(double) * P->ntot * c.nb));
     // the trial keeps the call's inputs (a correction sweep starts from zero
     // and is driven by its forcing) and writes only scratch; it runs several
@@ -595,7 +598,7 @@ pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_op
     CU(cudaEventCreate(&e1));
     float best = 1e30f;
     int best_t = 128;
-    for (int k = 0; k < 4; ++k) {
+    for (int k = first; k < 5; ++k) {
         for (int rep = 0; rep < 3; ++rep) {  // first repetition warms up; the last is timed
             CU(cudaEventRecord(e0, P->stream));
             CU(launch_steps(prec, a, cand[k], v.smem, P->stream, v.xg));
