@@ -169,14 +169,14 @@ HBM_FALLBACK_GBS = 6800.0
 
 
 def phi_source_hash() -> str:
-    """Hash of the multi-step kernel's code (its header, and the structures of
-    the shared declarations it reads: GridInfo, OpParams, StepArgs) with
+    """Hash of the multi-step kernels' code (their headers, and the structures of
+    the shared declarations they read: GridInfo, OpParams, StepArgs) with
     comments and blank lines removed, so that an edit of a comment or of an
     unrelated declaration keeps a capture valid and any change of the
     kernel's code invalidates it."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2509_22156_gb300", "csrc")
-    kern = open(os.path.join(csrc, "pit_phi.cuh")).read()
+    kern = "".join(open(os.path.join(csrc, f)).read() for f in ("pit_phi.cuh", "pit_direct.cuh", "pit_fixed.cuh"))
     decl = open(os.path.join(csrc, "pit_internal.cuh")).read()
     structs = "".join(re.findall(r"struct (?:GridInfo|OpParams|StepArgs) \{.*?\n\};", decl, flags=re.S))
     for text in (kern, structs):
@@ -191,7 +191,7 @@ def phi_source_hash() -> str:
 # committed ncu summaries of the relaxation kernel per workload: DRAM bytes per
 # node-step of a relaxation launch (captured on a smaller case of the same
 # kernel where the workload is too large to capture)
-NCU_SUMMARY = {5: "steps_kernel_heat_mixed_heat6d.txt", 2: "steps_kernel_heat_mixed_heat3d_n9.txt"}
+NCU_SUMMARY = {5: "fixed_kernel_heat6d.txt", 2: "steps_kernel_heat_mixed_heat3d_n9.txt"}
 
 
 def ncu_traffic(wl_k):
@@ -404,6 +404,8 @@ def roofline_block(B, wl, prof, chosen, k):
                       "frac": (fp64_flops / t / 1e12 / FP64_FMA_TFLOPS) if t else None,
                       "flops_per_node_pass": 3 * d + 4,
                       "op_mix_limit_frac": (3 * d + 4) / (2.0 * (2 * d + 3)),
+                      "note": "checks without forcing run on integer pipes and are counted as the FP64 passes "
+                              "that they replace" if wl.op == B.PIT_OP_HEAT else "",
                       "peak_source": "measured FP64 FMA probe on this pool"},
         "fp32": {"achieved": fp32_flops / t / 1e12 if t else None, "peak": FP32_FMA_TFLOPS, "unit": "TFLOP/s",
                  "frac": (fp32_flops / t / 1e12 / FP32_FMA_TFLOPS) if t else None,
@@ -413,14 +415,21 @@ def roofline_block(B, wl, prof, chosen, k):
                  "frac": (iters * smem_b / t / 1e9 / SMEM_LOAD_GBS) if t else None,
                  "bytes_per_node_iter": smem_b, "peak_source": "measured shared-memory load probe on this pool"},
     }
-    return {"bound": "hbm", "kernel": f"steps_kernel<{opname},{form},{d}> (grid-resident multi-step backward "
-                                      "Euler, FP32 Krylov in iterative refinement)",
+    # heat refinements: direct FP32 solves, and without forcing integer checks;
+    # a solve counts as the iteration and a check as the pass that it replaces
+    direct = wl.op == B.PIT_OP_HEAT and prec != B.PIT_PREC_FP64
+    kern = {B.PIT_PREC_MIXED: "fixed_kernel and direct_kernel", B.PIT_PREC_MIXED_PAIR: "direct_kernel"}.get(prec) \
+        if direct else f"steps_kernel<{opname},{form}>"
+    how = "direct FP32 solves" if direct else "FP32 Krylov" if prec != B.PIT_PREC_FP64 else "FP64 Krylov"
+    return {"bound": "hbm", "kernel": f"{kern} (d = {d}, grid-resident multi-step backward Euler, {how}"
+                                      + (")" if prec == B.PIT_PREC_FP64 else " in iterative refinement)"),
             "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": (achieved / hbm) if achieved else None,
             "traffic": (trf * steps / max(1, int(prof.launches[0]))) if trf is not None else None,
             "traffic_note": "DRAM bytes per relaxation launch: the committed ncu summary's DRAM bytes per "
                             "node-step times the node-steps of an average relaxation launch of the timed "
                             "region; null when the kernel changed since the capture",
-            "algorithmic_bytes": "40 B per node and FP32 CG iteration + 40 B per node and FP64 refinement pass",
+            "algorithmic_bytes": "40 B per node and FP32 CG iteration + 40 B per node and FP64 refinement pass"
+                                 + (" (a direct solve and an integer check count as one of each)" if direct else ""),
             "peak_source": hbm_src,
             "time_basis_ms": relax_ms, "relax_launches": int(prof.launches[0]),
             "relax_kernels": int(prof.kernels[0]), "sweep_ms": prof.ms[1], "sweep_launches": int(prof.launches[1]),

@@ -166,7 +166,11 @@ typedef struct {
  *                          FP32 Krylov on A e = r to relative
  *                          max(inner_rtol, 0.5 rtol ||b|| / ||r||) (at most maxit
  *                          iterations), x += e in FP64; at most ir_maxit
- *                          passes; the same FP64 stopping rule.
+ *                          passes; the same FP64 stopping rule.  (Heat operator
+ *                          without forcing: the state and b - A x as 64-bit
+ *                          integers of the state's scale, where the error of
+ *                          that, about 2^-50 n^{1/2} max(1, sum_i dt / h_i^2),
+ *                          is below a quarter of rtol.)
  *   prec = PIT_PREC_FP32:  Krylov in FP32 on a copy of the state scaled by a
  *                          power of two (inputs and outputs stay FP64) until
  *                          the FP32 recurrence residual meets rtol; for solves
@@ -200,9 +204,14 @@ typedef struct {
 /* Preconditioner of the Krylov solves (the paper preconditions its CG and
  * BiCGStab by domain decomposition, Sec. 2.1.2 and Sec. 4.1; on one GPU the
  * grid-resident solver offers these):
- *   DEFAULT  heat operator: the line preconditioner (tridiagonal along the
- *            finest axis, in the FP32 Krylov forms on anisotropic grids at
- *            stiff steps); other operators: none.
+ *   DEFAULT  heat operator: in the refinement forms (PIT_PREC_MIXED,
+ *            PIT_PREC_MIXED_PAIR) a direct FP32 solve of the correction
+ *            equation (sine transforms of the short axes, counted as one
+ *            Krylov iteration) where rtol <= 1e-4, maxit >= 16, dt is at most
+ *            the smallest squared extent of the box and no grid has two axes
+ *            of more than 31 nodes; else, and in the FP32 form, the line
+ *            preconditioner (tridiagonal along the finest axis, on anisotropic
+ *            grids at stiff steps).  Other operators: none.
  *   NONE     no preconditioner.
  *   JACOBI   diagonal (Jacobi) preconditioning of the FP32 correction solves
  *            of the refinement forms (PIT_PREC_MIXED, PIT_PREC_MIXED_PAIR) for
@@ -484,7 +493,9 @@ pit_status pit_mgrit_solve(pit_problem_t p, const double *u0, const pit_mgrit_op
  * interpolant on grid g with zero boundary values (Sec. 2.2.2).
  * u: host or device, n_total doubles; pts: host or device, n_pts * d doubles
  * (row-major); out: host or device, n_pts doubles.  Points outside the box
- * are clamped to its boundary cell. */
+ * are clamped to its boundary cell.  For many points the sum is taken from the
+ * sparse grid's surpluses (pit_recombine's plan and scratch, built on first
+ * use); values that are not finite affect the points whose cells touch them. */
 pit_status pit_combine(pit_problem_t p, const double *u, int n_pts, const double *pts, double *out);
 
 /* Recombination (Sec. 2.2.2, Eq. "overall_combination_operator"):
