@@ -339,9 +339,12 @@ __device__ __forceinline__ void long_lines(const Direct &D, float *v, float mul)
             z = fmaf(w, y, z);
             w *= rho;
         }
-        zs[t] = z;
+        // (the sum of a line's first chunk is not asked for below: its place
+        // takes z_{N+1}.  fw and bw are still being read by the line's other
+        // threads here.)
+        if (q > 0) zs[t] = z;
         // z_{N+1}: the tail rho^2 / (1 - rho^2) of y beyond the line, and -beta
-        if (q == P - 1) fw[l] = (rho * y) / (1.0f - rho * rho) - beta * c / rho;
+        if (q == P - 1) zs[l] = (rho * y) / (1.0f - rho * rho) - beta * c / rho;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < tasks; t += blockDim.x) {
@@ -350,7 +353,7 @@ __device__ __forceinline__ void long_lines(const Direct &D, float *v, float mul)
         const float b0 = fmaf(mul, smem_f()[D.base + l], 1.0f);
         const float rho = 2.0f * c / (b0 + 2.0f * c + sqrtf(b0 * (b0 + 4.0f * c)));
         const float pl = pow_n(rho, L), pz = pow_n(rho, N - (P - 1) * L), sc = rho / c * D.norm;
-        float z = fw[l];
+        float z = zs[l];
         for (int i = P - 1; i > q; --i) z = fmaf(i == P - 1 ? pz : pl, z, zs[i * nl + l]);
         float *p = v + line_start(l, N, Sa, inv) + k0 * Sa;
         for (int k = m - 1; k >= 0; --k) {

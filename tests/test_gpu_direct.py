@@ -81,3 +81,18 @@ def test_krylov_keeps_the_calls_the_direct_solve_does_not_take():
                      B.solve_opts(B.PIT_PREC_MIXED, rtol=1e-12, maxit=20000, inner_rtol=1e-5, ir_maxit=40))
     assert st.sum_iters / Q.G > 4
     assert per_grid(Q, out.cpu().numpy(), R.phi(1e-3, u, rtol=1e-15)) < 1e-9
+
+
+@pytest.mark.parametrize("prec,forced", [(B.PIT_PREC_MIXED, False), (B.PIT_PREC_MIXED, True), (B.PIT_PREC_MIXED_PAIR, True)])
+@pytest.mark.parametrize("d,n", [(1, 10), (2, 7), (2, 10)])
+def test_chunked_lines_give_the_same_bits_every_time(d, n, prec, forced):
+    # lines of 63 nodes and more are cut into chunks that exchange sums: every call has to see the same ones
+    P = B.Problem(d, n, 1, W.OP_HEAT)
+    u = torch.from_numpy(np.tile(W.random_vector(21, P.n_total), 24)).cuda()
+    f = torch.from_numpy(np.tile(W.random_vector(22, P.n_total), 24)).cuda() if forced else None
+    out = torch.empty_like(u)
+    first = None
+    for _ in range(20):
+        P.phi_batch(1e-3, u, out, B.solve_opts(prec, rtol=1e-9, maxit=4000, inner_rtol=1e-5, ir_maxit=12), f=f, n_batch=24)
+        first = out[:P.n_total].clone() if first is None else first
+        assert bool((out.view(24, -1) == first).all())
