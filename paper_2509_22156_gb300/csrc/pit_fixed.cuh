@@ -26,7 +26,7 @@
 namespace pit {
 
 struct FixConst {
-    int hi[PIT_D + 1], lo[PIT_D + 1];  // c_i 2^{-E-1} = (hi 2^29 + lo) 2^-60 of the listed axes; [D]: 2 sum of the others
+    int hi[PIT_D + 1], lo[PIT_D + 1];  // c_i 2^{-E-1} = (hi 2^29 + lo) 2^-60 of the listed axes; [D]: sum of the others
     int E;
 };
 __device__ __forceinline__ void fix_const(const StepArgs &a, const GridInfo &G, FixConst &F)
@@ -35,8 +35,9 @@ __device__ __forceinline__ void fix_const(const StepArgs &a, const GridInfo &G, 
         double sum = 0.0, rest = 0.0;
         for (int i = 0; i < a.op.d; ++i) {
             sum += a.dt * G.ih2[i];
-            if (G.N[i] == 1 && i != G.ax[0]) rest += 2.0 * a.dt * G.ih2[i];
+            if (G.N[i] == 1 && i != G.ax[0]) rest += a.dt * G.ih2[i];
         }
+        // (every coefficient, and the sum of any of them, is below 2^{e+1}: hi < 2^31)
         const int e = max(0, (int)((__double2hiint(sum) >> 20) & 0x7ff) - 1023);  // sum 2^-e < 2
         const int q = threadIdx.x;
         const double c = q < G.de ? a.dt * G.ih2[G.ax[q]] : q == G.de ? rest : 0.0;
@@ -93,7 +94,8 @@ static __device__ __noinline__ float fix_residual(const long long *xg, const lon
             B += (long long)tl * ch[i];
         }
         if (rh | rl) {
-            const long long t = 4 * xj;
+            // an axis of one node has zero neighbours: its second difference is 2 x_j
+            const long long t = 4 * t0;
             const int th = (int)(t >> 32), tl = (int)((unsigned)t >> 3);
             A += (long long)th * rh;
             B += (long long)th * rl;

@@ -96,3 +96,23 @@ def test_tight_tolerances_and_bad_inputs():
             sl = slice(P.offsets[g], P.offsets[g + 1])
             if g != 2:
                 assert np.linalg.norm(got[sl] - ref[sl]) < 1e-9 * np.linalg.norm(ref[sl])
+
+
+# The axes with one node add 2 dt / h^2 each to the diagonal, more than the listed axes where those are short: steps on
+# both sides of the points where that sum passes a power of two, boxes with extents of their own, a minimum level above 1.
+@pytest.mark.parametrize("d,n,L0,hi,dts", [
+    (3, 2, 1, None, [0.1, 0.12, 0.13, 0.16, 0.2, 0.26, 0.32]),
+    (4, 4, 1, None, [0.05, 0.08, 0.085, 0.12, 0.13, 0.2]),
+    (6, 3, 1, None, [0.04, 0.05, 0.054, 0.06, 0.08, 0.09, 0.11, 0.16, 0.25]),
+    (2, 3, 1, [1.0, 0.1], [0.002, 0.0026, 0.004, 0.0045, 0.006]),
+    (3, 6, 1, [0.2, 1.0, 0.5], [0.005, 0.01, 0.015, 0.02, 0.03, 0.04]),
+    (2, 5, 2, [0.5, 1.0], [0.01, 0.05, 0.2])])
+def test_one_node_axes_at_large_steps(d, n, L0, hi, dts):
+    box = ([0.0] * d, hi or [1.0] * d)
+    P = B.Problem(d, n, L0, W.OP_HEAT, *box)
+    O = oracle.Problem(d, n, L0, W.OP_HEAT, *box)
+    u = W.random_vector(13, P.n_total)
+    for dt in dts:
+        got, st = solve(P, u, dt, 1, opts())
+        assert st.n_failed == 0, dt
+        assert worst(P, got, O.phi(dt, u, rtol=1e-15)) < 1e-9, dt
