@@ -12,13 +12,17 @@
 //
 // Accuracy: ||x||_2 2^k lies in [2^52, 2^57), so a unit is at most 2^-52 of the
 // norm (FP64 holds 2^-53 of every value); |x_j| <= ||x||_2, the extrapolated
-// guess is below 3 ||x||, a second difference below 2^60.6, and with E chosen so
+// guess 2 x_s - x_{s-1} is below 3 2^57 as long as both states are below 2^57, a
+// second difference below 2^60.6, and with E chosen so
 // that sum c_i 2^-E < 2 the sum of products stays below 2^62.  Dropped bits and
 // the final shifts leave the residual off by a few units (at most 12; times 2^E
 // for large steps): 8 n^{1/2} 2^-53 max(1, sum c_i) of the norm, and the host
 // takes this form only where that is below a quarter of the requested
 // tolerance, the FP64 check elsewhere.  A state that has decayed by more than
-// four bits is shifted up again before its next step.
+// four bits is shifted up again before its next step, as far as the state before
+// it, which the extrapolated guess contains, leaves room; where one step has
+// shrunk the state to less than an eighth, that would leave it too few bits, and
+// the step starts from x_s instead.
 #pragma once
 
 #include "pit_direct.cuh"
@@ -185,14 +189,16 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
         return acc[0];
     };
     // The right-hand side's norm has fallen below 2^53 units: shifts the state
-    // back up to 2^56 (v: ||r||^2 and ||b||^2, updated; everything a step keeps
-    // is scaled with it).  Own nodes; a barrier on both sides.
-    auto rescale = [&](float (&v)[2], int cst) {
+    // back up until the norm, or the larger one whose square is top, is at 2^56
+    // (v: ||r||^2 and ||b||^2, updated; everything a step keeps is scaled with
+    // it).  Own nodes; a barrier on both sides.
+    auto rescale = [&](float (&v)[2], int cst, float top) {
         // (below 2^45 the norm's 2^32-unit parts say too little: eight bits at a
         // time, at most the width of the state)
         for (int it = 0; it < 8 && v[1] < 0x1p42f && k < 900 && (v[1] > 0.0f || v[0] > 0.0f); ++it) {
             const bool coarse = v[1] < 0x1p26f;
-            const int up = min(coarse ? 8 : scale_exp(v[1]) + 24, 900 - k);
+            const int up = min(coarse ? 8 : scale_exp(fmaxf(v[1], top)) + 24, 900 - k);
+            if (up <= 0) break;
             const float sc = __uint_as_float((unsigned)(127 + up) << 23);
             float bb[1] = {0.0f};
             __syncthreads();
@@ -209,17 +215,19 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
             R32.template sum<1>(bb);
             v[0] = (v[0] * sc) * sc;
             v[1] = bb[0];
+            top = (top * sc) * sc;
         }
     };
 
     int status = bad ? PIT_ERR_NONFINITE : PIT_OK, iters = 0, passes = 0;
     bool have_r0 = false;
     int cst = 0, unchecked = 0;  // what cw holds: 0 nothing, 1 c, 2 q
+    float b_last = 0.0f;         // ||x_{s-1}||^2 in 2^32 units
     for (int step = 1; step <= a.nsteps; ++step) {
         if (!have_r0) __syncthreads();  // state complete
         if (!bad) {
             float acc[2] = {0.0f, 0.0f};  // ||r||^2 in residual units, ||b||^2 in 2^32 units of x
-            const bool carried = have_r0;
+            bool carried = have_r0;
             if (carried) {
                 const int from = !a.predict ? 0 : cst;
                 if (from == 2) {
@@ -272,8 +280,17 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
                 }
                 R32.template sum<2>(acc);
                 cst = from == 0 ? 0 : 2;
-                if (acc[1] < 0x1p42f) rescale(acc, cst);
-            } else {
+                if (acc[1] < 0x1p42f) {
+                    if (cst == 2 && b_last > 0x1p6f * acc[1]) {  // shrunk to less than an eighth
+                        for (int j = tid; j < n; j += nt) x[j] = bv[j];
+                        carried = false;
+                        acc[1] = 0.0f;
+                    } else {
+                        rescale(acc, cst, cst == 2 ? b_last : 0.0f);
+                    }
+                }
+            }
+            if (!carried) {
                 for (int j = tid; j < n; j += nt) {
                     const long long xo = x[j];
                     bv[j] = xo;
@@ -285,7 +302,7 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
                 acc[0] = 1.0f;
                 acc[1] = bb[0];
                 if (acc[1] < 0x1p42f) {
-                    rescale(acc, 0);  // (rv is scaled too, and overwritten next)
+                    rescale(acc, 0, 0.0f);  // (rv is scaled too, and overwritten next)
                     __syncthreads();
                 }
                 acc[0] = residual(true);
@@ -294,7 +311,7 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
                 unchecked = -1;
             }
             float rn = acc[0];
-            const float bb = acc[1];
+            const float bb = b_last = acc[1];
             have_r0 = false;
             float stop2 = a.rtol2 * bb * b2r;
             int st_step = PIT_OK;

@@ -116,3 +116,39 @@ def test_one_node_axes_at_large_steps(d, n, L0, hi, dts):
         got, st = solve(P, u, dt, 1, opts())
         assert st.n_failed == 0, dt
         assert worst(P, got, O.phi(dt, u, rtol=1e-15)) < 1e-9, dt
+
+
+def states(O, u, dt, steps):
+    out = [u]
+    for _ in range(steps):
+        out.append(O.phi(dt, out[-1], rtol=1e-15))
+    return out
+
+
+# A step that shrinks the state many times over: the extrapolated guess is then about the state before, far larger than
+# the state whose norm the integers are scaled by.  Each step's residual is at most 1.25 rtol ||x_{s-1}|| and
+# ||A^-1|| <= 1, so the state is off by 1.25 rtol times the sum of the earlier states' norms.
+@pytest.mark.parametrize("d,n,dt,steps,kind", [
+    (4, 1, 1.0, 2, "random"), (4, 1, 1.0, 12, "random"), (6, 1, 0.9, 5, "random"), (1, 4, 0.05, 4, "highest"),
+    (1, 4, 0.5, 6, "random"), (1, 4, 0.5, 8, "highest"), (1, 6, 0.02, 6, "spike"), (1, 8, 0.01, 8, "spike"),
+    (2, 5, 0.3, 6, "random"), (3, 5, 0.05, 10, "spike"), (3, 4, 0.9, 6, "random"), (6, 3, 0.5, 6, "random")])
+def test_steps_that_shrink_the_state_many_times_over(d, n, dt, steps, kind):
+    P = B.Problem(d, n, 1, W.OP_HEAT)
+    O = oracle.Problem(d, n, 1, W.OP_HEAT)
+    u = W.random_vector(17, P.n_total)
+    for g in range(P.G):
+        sl = slice(P.offsets[g], P.offsets[g + 1])
+        m = P.offsets[g + 1] - P.offsets[g]
+        if kind == "highest":
+            u[sl] = np.sin(np.pi * m * np.arange(1, m + 1) / (m + 1))
+        elif kind == "spike":
+            u[sl] = 0.0
+            u[sl][m // 2] = 1.0
+    ref = states(O, u, dt, steps)
+    for guess in (B.PIT_GUESS_PREVIOUS, B.PIT_GUESS_EXTRAPOLATE):
+        got, st = solve(P, u, dt, steps, opts(guess=guess))
+        assert st.n_failed == 0
+        for g in range(P.G):
+            sl = slice(P.offsets[g], P.offsets[g + 1])
+            off = np.linalg.norm(got[sl] - ref[-1][sl])
+            assert off <= 1.25e-11 * sum(np.linalg.norm(r[sl]) for r in ref[:-1]), g
