@@ -935,6 +935,7 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
     CUB(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));
     CUB(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));
     CUB(phi_kernels_init(P->max_smem));
+    CUB(cluster_init(P->max_smem));
     CUB(net_kernels_init(P->max_smem));
     CUB(recombine_init(P->max_smem));
     CUB(combine_init(P->max_smem));

@@ -431,8 +431,6 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cluster_kernel(const __grid_con
     cl.sync();  // no CTA leaves while another may still store into its memory
 }
 
-typedef void (*ClusterFn)(const StepArgs, int);
-
 // the kernel of an operator and grid dimension (listed axes), or NULL
 const void *cluster_fn(int op, int de)
 {
@@ -491,15 +489,23 @@ static cudaLaunchConfig_t cluster_config(int items, int C, size_t smem, cudaStre
     return cfg;
 }
 
+// (a kernel's limits hold for every problem of the process: they are set to the
+// most that any of them asks for, and stay)
+cudaError_t cluster_init(size_t max_smem)
+{
+    for (int op : {(int)PIT_OP_OU, (int)PIT_OP_LSDE, (int)PIT_OP_CME})
+        for (int de = 1; const void *fn = cluster_fn(op, de); ++de) {
+            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+}
+
 int cluster_capacity(int op, int de, int C, size_t smem)
 {
     const void *fn = cluster_fn(op, de);
     if (!fn) return 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        (C > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
-        cudaGetLastError();
-        return 0;
-    }
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = cluster_config(1, C, smem, nullptr, &attr);
     int n = 0;

@@ -231,10 +231,11 @@ size_t direct_smem_bytes(int prec, int n, int na, bool xg);
 bool direct_grid(const GridInfo &G);
 int xg_slabs(int prec, int op, int d);
 // FP64 form with one cluster of C CTAs per item (pit_cluster.cu; drift
-// operators, narrow batches of large grids): whether there is a kernel for
-// grids of up to de listed axes, how far the stencil reaches in nodes, the
+// operators, narrow batches of large grids): kernel set-up, whether there is a
+// kernel for grids of up to de listed axes, how far the stencil reaches in nodes, the
 // shared memory of a CTA, how many clusters the device runs at once, and the
 // launch.
+cudaError_t cluster_init(size_t max_smem);
 bool cluster_kernel_for(int op, int de);
 int cluster_reach(const GridInfo &G, int op);
 size_t cluster_smem_bytes(const GridInfo &G, int C, int reach);

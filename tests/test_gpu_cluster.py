@@ -94,3 +94,23 @@ def test_mgrit_with_clusters_matches_sequential():
         P.mgrit_solve(ud, o, uT)
         P.sequential_solve(ud, dt, 32, seq, fine)
         assert torch.linalg.norm(uT - seq) < 1e-8 * torch.linalg.norm(seq)
+
+
+def test_cluster_sizes_and_problems_take_turns():
+    # batches of one and two states take clusters of different sizes, whose CTAs need different shared memory, and so do
+    # problems of different size: every earlier choice still runs after a later one
+    def probs():
+        for n in (12, 13):
+            a = (2, n, 5, B.PIT_OP_OU, [-6.0] * 2, [6.0] * 2)
+            yield B.Problem(*a), oracle.Problem(*a)
+    pairs = list(probs())
+    ref = {}
+    for k, nb in [(1, 2), (1, 1), (1, 2), (0, 1), (1, 1), (0, 2), (1, 2), (0, 3), (0, 1)]:
+        P, O = pairs[k]
+        u = np.abs(W.random_vector(5 + k, P.n_total)) + 0.1
+        out = torch.empty(nb * P.n_total, dtype=torch.float64, device="cuda")
+        P.phi_batch(1e-3, torch.from_numpy(np.tile(u, nb)).cuda(), out, opts(), n_batch=nb)
+        if k not in ref:
+            ref[k] = O.phi(1e-3, u, rtol=1e-15)
+        got = out.cpu().numpy().reshape(nb, -1)
+        assert np.linalg.norm(got - ref[k]) < 1e-10 * np.linalg.norm(ref[k]) * np.sqrt(nb)
