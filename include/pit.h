@@ -493,9 +493,12 @@ pit_status pit_mgrit_solve(pit_problem_t p, const double *u0, const pit_mgrit_op
  * interpolant on grid g with zero boundary values (Sec. 2.2.2).
  * u: host or device, n_total doubles; pts: host or device, n_pts * d doubles
  * (row-major); out: host or device, n_pts doubles.  Points outside the box
- * are clamped to its boundary cell.  For many points the sum is taken from the
- * sparse grid's surpluses (pit_recombine's plan and scratch, built on first
- * use); values that are not finite affect the points whose cells touch them. */
+ * are clamped to its boundary cell.  For many points the grids that differ in
+ * the last axis' level only are added first (arrays of up to about three state
+ * vectors, kept from the first such call on; without memory for them, the sum
+ * is taken grid by grid).  Either way the rounding error at a point x is of the
+ * size of 2^-53 sum_l |c_l| I_l[|u_l|](x), and values that are not finite
+ * affect the points whose cells touch them. */
 pit_status pit_combine(pit_problem_t p, const double *u, int n_pts, const double *pts, double *out);
 
 /* Recombination (Sec. 2.2.2, Eq. "overall_combination_operator"):

@@ -185,11 +185,18 @@ struct pit_problem {
     RecombPlan rc{};
     RecombPiece *rc_pieces = nullptr;
     RecombTerm *rc_terms = nullptr;
-    RecombEval *rc_eval = nullptr;
-    int *rc_bad = nullptr;  // a surplus of the last combination sum was not finite
     RecombBlock *rc_blocks = nullptr;
     long long *rc_grid_blocks = nullptr;
     DBuf rc_H, rc_S, rc_T, rc_cur;
+    // combination sum over groups of grids, built on first use (host part, then
+    // device tables and the groups' arrays)
+    bool cb_grouped = false, cb_ready = false;
+    double cb_ops = 0.0;       // FP64 operations a point
+    long long cb_nodes = 0;    // doubles of the groups' arrays
+    std::vector<CombineGroup> cb_groups;
+    std::vector<CombineTerm> cb_terms;
+    CombinePlan cb{};
+    DBuf cb_tab, cb_M;
 };
 
 namespace {
@@ -1014,14 +1021,14 @@ pit_status pit_problem_destroy(pit_problem_t P)
     if (P->ev_join) cudaEventDestroy(P->ev_join);
     cudaFree(P->rc_pieces);
     cudaFree(P->rc_terms);
-    cudaFree(P->rc_eval);
-    cudaFree(P->rc_bad);
     cudaFree(P->rc_blocks);
     cudaFree(P->rc_grid_blocks);
     P->rc_H.release();
     P->rc_S.release();
     P->rc_T.release();
     P->rc_cur.release();
+    P->cb_tab.release();
+    P->cb_M.release();
     cudaFree(P->d_grids);
     cudaFree(P->d_coef);
     cudaFree(P->d_levels);
@@ -1294,7 +1301,6 @@ pit_status recomb_plan(pit_problem *P)
     };
     for (int g = 0; g < G; ++g) for_box(g, [&](const int *lam) { used[code_of(lam)] = 1; });
     std::vector<int> lookup(ncell, -1);
-    std::vector<RecombEval> eval;
     std::vector<long long> blk_off(1, 0);
     int n_blk = 0;
     for (int c = 0; c < ncell; ++c) {
@@ -1306,11 +1312,6 @@ pit_status recomb_plan(pit_problem *P)
             e += lam[i] - 1;
         }
         lookup[c] = n_blk++;
-        RecombEval ev{blk_off.back(), {}, 0, 0};
-        for (int i = 0; i < d; ++i) ev.lam[i] = (unsigned char)lam[i];
-        if (!eval.empty())
-            while (ev.from < d - 1 && ev.lam[ev.from] == eval.back().lam[ev.from]) ++ev.from;
-        eval.push_back(ev);
         blk_off.push_back(blk_off.back() + (1LL << e));
     }
     // terms of every block and blocks of every grid
@@ -1393,14 +1394,9 @@ pit_status recomb_plan(pit_problem *P)
     };
     CU(up(P->rc_pieces, pieces));
     CU(up(P->rc_terms, terms));
-    CU(up(P->rc_eval, eval));
-    CU(dev_malloc(&P->rc_bad, sizeof(int)));
     CU(up(P->rc_blocks, blocks));
     CU(up(P->rc_grid_blocks, grid_blocks));
     rc.n_sparse = blk_off.back();
-    rc.n_blk = n_blk;
-    rc.l_max = Lmax;
-    rc.eval = P->rc_eval;
     rc.n_pieces = (int)pieces.size();
     rc.pieces = P->rc_pieces;
     rc.terms = P->rc_terms;
@@ -2365,22 +2361,121 @@ extern "C" pit_status pit_mgrit_solve(pit_problem_t P, const double *u0, const p
     return PIT_OK;
 }
 
-// Whether the combination sum at n_pts points takes the sparse grid's
-// surpluses: FP64 operations of the sum over grids (2^d corners and the cells
-// of every grid a point) against those of the surpluses (about eight a node
-// with the gather) and of the increments a point, with 20e6 operations (35 us)
-// for the further launches.  The sum over grids is the faster one for few
-// points on large grid sets.  (Builds the block plan on first use.)
-static bool combine_by_surpluses(pit_problem *P, int n_pts)
+// Groups of the combination sum: the grids that differ in the last axis' level
+// only, finest first, ordered by their listed axes.
+static void combine_groups(pit_problem *P)
+{
+    if (P->cb_grouped) return;
+    const int d = P->desc.d;
+    std::vector<int> order(P->G);
+    for (int g = 0; g < P->G; ++g) order[g] = g;
+    const int *lev = P->levels.data();
+    std::sort(order.begin(), order.end(), [&](int a, int b) {
+        const int *x = lev + (size_t)a * d, *y = lev + (size_t)b * d;
+        for (int i = 0; i < d - 1; ++i)
+            if (x[i] != y[i]) return x[i] < y[i];
+        return x[d - 1] > y[d - 1];
+    });
+    struct Members { CombineGroup G; int first, last; };
+    std::vector<Members> list;
+    for (int k = 0; k < P->G;) {
+        const int *x = lev + (size_t)order[k] * d;
+        int k1 = k + 1;
+        while (k1 < P->G && std::equal(x, x + d - 1, lev + (size_t)order[k1] * d)) ++k1;
+        CombineGroup G{};
+        G.n = P->info[order[k]].n;
+        long long size = 1;
+        int de = 0;
+        for (int i = 0; i < d; ++i) de += x[i] > 1;
+        for (int i = d - 1, q = de - 1; i >= 0; --i)
+            if (x[i] > 1) {
+                G.mask |= 1 << i;
+                G.lev[q] = (unsigned char)x[i];
+                G.stride[q--] = (int)std::min(size, 0x7fffffffLL);
+                size *= (1LL << x[i]) + 1;
+            }
+        if (x[d - 1] > 1) G.mask |= 1 << PIT_D;
+        G.at = size;  // (its size until the groups are in order)
+        P->cb_ops += 2.0 * (1 << de) + de + 1.0;
+        list.push_back({G, k, k1});
+        k = k1;
+    }
+    std::stable_sort(list.begin(), list.end(), [](const Members &a, const Members &b) { return a.G.mask < b.G.mask; });
+    for (Members &m : list) {
+        const long long size = m.G.at;
+        m.G.at = P->cb_nodes;
+        P->cb_nodes += size;
+        m.G.term0 = (int)P->cb_terms.size();
+        for (int k = m.first; k < m.last; ++k) {
+            const int g = order[k];
+            P->cb_terms.push_back({P->off[g], P->coef[g], lev[(size_t)g * d + d - 1], 0});
+        }
+        m.G.term1 = (int)P->cb_terms.size();
+        P->cb_groups.push_back(m.G);
+        if (size > 0x7fffffffLL) P->cb_ops = 1e300;  // (strides are 32-bit: the sum over grids)
+    }
+    P->cb_grouped = true;
+}
+
+static cudaError_t combine_upload(pit_problem *P)
+{
+    if (P->cb_ready) return cudaSuccess;
+    std::vector<CombinePiece> pieces;
+    std::vector<CombineRun> runs;
+    int l_max = 1;
+    for (int l : P->levels) l_max = std::max(l_max, l);
+    for (int k = 0; k < (int)P->cb_groups.size(); ++k) {
+        const CombineGroup &G = P->cb_groups[k];
+        const int mask = G.mask & ((1 << PIT_D) - 1);
+        for (long long j = 0; j < G.n; j += 256) pieces.push_back({k, (int)j});
+        if (runs.empty() || runs.back().mask != mask) runs.push_back({k, k, mask});
+        runs.back().last = k + 1;
+    }
+    const size_t sz[4] = {P->cb_groups.size() * sizeof(CombineGroup), P->cb_terms.size() * sizeof(CombineTerm),
+                          pieces.size() * sizeof(CombinePiece), runs.size() * sizeof(CombineRun)};
+    const void *src[4] = {P->cb_groups.data(), P->cb_terms.data(), pieces.data(), runs.data()};
+    size_t at[5] = {};
+    for (int q = 0; q < 4; ++q) at[q + 1] = at[q] + ((sz[q] + 255) & ~(size_t)255);
+    cudaError_t e = P->cb_M.ensure(sizeof(double) * (size_t)P->cb_nodes);
+    if (e == cudaSuccess) e = P->cb_tab.ensure(at[4]);
+    char *t = (char *)P->cb_tab.p;
+    for (int q = 0; q < 4 && e == cudaSuccess; ++q) e = cudaMemcpy(t + at[q], src[q], sz[q], cudaMemcpyHostToDevice);
+    // (boundary values; the nodes are written by every call)
+    if (e == cudaSuccess) e = cudaMemsetAsync(P->cb_M.p, 0, sizeof(double) * (size_t)P->cb_nodes, P->stream);
+    if (e != cudaSuccess) return e;
+    P->cb = CombinePlan{(int)pieces.size(), (int)runs.size(), l_max, (const CombineGroup *)t,
+                        (const CombineTerm *)(t + at[1]), (const CombinePiece *)(t + at[2]),
+                        (const CombineRun *)(t + at[3])};
+    P->cb_ready = true;
+    return cudaSuccess;
+}
+
+// Whether the combination sum at n_pts points adds the groups first: FP64
+// operations of the sum over grids (2^d corners and the cells of every grid a
+// point) against those of the addition (about four a node) and of the groups a
+// point, with 20e6 operations (35 us) for the further launches.  The sum over
+// grids is the faster one for few points on large grid sets, and the one that
+// runs where the groups' arrays cannot be had: no memory for them, or a first
+// call while the stream is being captured.
+static bool combine_merged(pit_problem *P, int n_pts)
 {
     const double direct = (double)n_pts * P->G * (2.0 * (1 << P->desc.d) + 6.0 * P->desc.d);
-    if (direct < 8.0 * (double)P->ntot + 20e6) return false;
-    if (recomb_plan(P) != PIT_OK) {
-        g_err.clear();
+    const double fixed = 4.0 * (double)P->ntot + 20e6;
+    if (direct < fixed) return false;
+    combine_groups(P);
+    if (!(direct > fixed + (double)n_pts * P->cb_ops)) return false;
+    if (P->cb_ready) return true;
+    int l_max = 1;
+    for (int l : P->levels) l_max = std::max(l_max, l);
+    if (combine_eval_smem(P->desc.d, l_max) > P->max_smem) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(P->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+        combine_upload(P) != cudaSuccess) {
+        cudaGetLastError();
+        P->cb_M.release();
         return false;
     }
-    if (combine_eval_smem(P->desc.d, P->rc.l_max) > P->max_smem) return false;
-    return direct > 8.0 * (double)P->ntot + 4.0 * (double)n_pts * P->rc.n_blk + 20e6;
+    return true;
 }
 
 extern "C" pit_status pit_combine(pit_problem_t P, const double *u, int n_pts, const double *pts, double *out)
@@ -2396,29 +2491,18 @@ extern "C" pit_status pit_combine(pit_problem_t P, const double *u, int n_pts, c
         CU(P->w_out.ensure(sizeof(double) * n_pts));
         target = P->w_out.d();
     }
-    if (combine_by_surpluses(P, n_pts)) {
-        // surpluses of the sparse grid, then one basis function of every
-        // increment a point; values that are not finite keep to the points
-        // whose cells they touch, so they are left to the sum over grids
-        CU(P->rc_H.ensure(sizeof(double) * P->ntot));
-        CU(P->rc_S.ensure(sizeof(double) * P->rc.n_sparse));
-        if (P->rc.cls_n[0] > 0) CU(P->rc_T.ensure(sizeof(double) * P->ntot));
+    if (combine_merged(P, n_pts)) {
         const int blocks = (n_pts + 127) / 128;
-        // (four blocks of 128 points an SM keep the FP64 unit busy)
-        int chunks = (4 * (P->n_sm > 0 ? P->n_sm : 1) + blocks - 1) / blocks;
-        chunks = std::max(1, std::min(chunks, P->rc.n_blk / 32));
-        if (chunks > 1) CU(P->w_part.ensure(sizeof(double) * (size_t)chunks * n_pts));
+        // (up to four blocks of 128 points an SM: a chunk places its points
+        // anew, which costs more than half-filled SMs do.  65,794 points: d = 4,
+        // level 7 245 us with one chunk, 272 with three; d = 3, level 9 122 and 148)
+        const int want = 4 * (P->n_sm > 0 ? P->n_sm : 1);
+        const int chunks = std::max(1, std::min(want / blocks, (int)P->cb_groups.size() / 8));
+        CU(P->w_part.ensure(sizeof(double) * (size_t)chunks * n_pts));
         ProfScope ps(P, 2);
-        CU(cudaMemsetAsync(P->rc_bad, 0, sizeof(int), P->stream));
-        CU(launch_surpluses(P->rc, P->d_grids, P->d_order, P->ntot, 1, du, P->rc_H.d(), P->rc_S.d(), P->rc_T.d(),
-                            P->rc_bad, P->stream));
-        CU(launch_combine_eval(P->rc, P->d_grids, P->d_levels, P->op, P->rc_S.d(), n_pts, dp, target, chunks,
-                               chunks > 1 ? P->w_part.d() : nullptr, P->rc_bad, P->stream));
-        CU(launch_combine(P->d_grids, P->d_coef, P->d_levels, P->G, P->op, du, n_pts, dp, target, 1, nullptr,
-                          P->stream, P->rc_bad));
-        int kernels = 3 + (chunks > 1 ? 1 : 0);
-        for (int c = 0; c < RECOMB_CLS; ++c) kernels += P->rc.cls_n[c] > 0 ? 1 : 0;
-        count_kernels(P, 2, kernels);
+        CU(launch_combine_merged(P->cb, P->d_grids, P->d_levels, P->op, du, P->cb_M.d(), n_pts, dp, target, chunks,
+                                 P->w_part.d(), P->stream));
+        count_kernels(P, 2, 3);
     } else {
         const int chunks = combine_chunks(P->G, n_pts, P->n_sm);
         if (chunks > 1) CU(P->w_part.ensure(sizeof(double) * (size_t)chunks * n_pts));

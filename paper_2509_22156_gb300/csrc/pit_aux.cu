@@ -276,10 +276,8 @@ cudaError_t launch_faces(const GridInfo *grids, int G, OpParams op, double *face
 // over all grids would keep only n_pts / 128 SMs busy, 33 of 152 for the
 // 4,100 points of the d = 6 workload, on FP64 interpolation work.)
 __global__ void combine_kernel(const GridInfo *grids, const double *coef, const int *levels, int G, OpParams op,
-                               const double *u, int n_pts, const double *pts, int gchunk, double *dst,
-                               const int *run_if)
+                               const double *u, int n_pts, const double *pts, int gchunk, double *dst)
 {
-    if (run_if && !*run_if) return;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n_pts) return;
     const int g0 = (int)blockIdx.y * gchunk;
@@ -362,16 +360,190 @@ int combine_chunks(int G, int n_pts, int n_sm)
 
 cudaError_t launch_combine(const GridInfo *grids, const double *coef, const int *levels, int G, OpParams op,
                            const double *u, int n_pts, const double *pts, double *out, int n_chunks, double *part,
-                           cudaStream_t s, const int *run_if)
+                           cudaStream_t s)
 {
     if (n_pts == 0 || G == 0) return cudaSuccess;
     if (n_chunks < 1 || (n_chunks > 1 && !part)) return cudaErrorInvalidValue;
     const int gchunk = (G + n_chunks - 1) / n_chunks;
     const int chunks = (G + gchunk - 1) / gchunk;
     const dim3 grid((unsigned)((n_pts + 127) / 128), (unsigned)chunks);
-    combine_kernel<<<grid, 128, 0, s>>>(grids, coef, levels, G, op, u, n_pts, pts, gchunk,
-                                     chunks > 1 ? part : out, run_if);
+    combine_kernel<<<grid, 128, 0, s>>>(grids, coef, levels, G, op, u, n_pts, pts, gchunk, chunks > 1 ? part : out);
     if (chunks > 1) combine_sum_kernel<<<(n_pts + 127) / 128, 128, 0, s>>>(part, chunks, n_pts, out);
+    return cudaGetLastError();
+}
+
+// The combination sum at many points.  A component grid's interpolant also lies
+// in the space of any grid that is finer along one axis, so the grids that
+// differ in the last axis' level only (at most d) are one function on the
+// finest of them: merge_kernel adds them there, node by node, and a point then
+// reads one cell of every group: 84 groups for the 195 grids of d = 4, level 7,
+// and 2,002 for the 4,921 of d = 6, level 10.
+//
+// Interpolation weights are never negative, so a value's rounding errors keep
+// to the cells that contain it, as in the sum over grids: the error at a point
+// is of the size of 2^-53 sum_l |c_l| I_l[|u_l|](x), the values near that point.
+// (The sum of hierarchical surpluses, with fewer terms yet, does not have this:
+// its terms are of the size of the largest value anywhere, and the tails of a
+// density come out as noise.)
+__global__ void __launch_bounds__(256) merge_kernel(CombinePlan C, const double *u, double *M)
+{
+    const CombinePiece pc = C.pieces[blockIdx.x];
+    const CombineGroup &G = C.groups[pc.group];
+    const int j = pc.first + threadIdx.x;
+    if (j >= G.n) return;
+    const int d1 = G.mask >> PIT_D, de = __popc(G.mask & ((1 << PIT_D) - 1));  // last axis listed; listed axes
+    const int L = d1 ? G.lev[de - 1] : 1, row = j / ((1 << L) - 1), p = j - row * ((1 << L) - 1) + 1;
+    double s = 0.0;
+    for (int k = G.term0; k < G.term1; ++k) {
+        const CombineTerm t = C.terms[k];
+        const int sh = L - t.lev, N = (1 << t.lev) - 1, c = p >> sh, rem = p & ((1 << sh) - 1);
+        const double *r = u + t.off + (long long)row * N;  // r[c - 1]: node c of the member's line
+        double v = 0.0;
+        if (rem == 0) {
+            v = r[c - 1];
+        } else {
+            // (boundary values are not read, nor multiplied with)
+            const double f = (double)rem / (double)(1 << sh);
+            if (c > 0) v = (1.0 - f) * r[c - 1];
+            if (c < N) v = fma(f, r[c], v);
+        }
+        s = fma(t.coef, v, s);
+    }
+    long long at = G.at + (d1 ? p : 0);
+    for (int q = de - 1 - d1, rr = row; q >= 0; --q) {
+        const int N = (1 << G.lev[q]) - 1;
+        at += (long long)(rr % N + 1) * G.stride[q];
+        rr /= N;
+    }
+    M[at] = s;
+}
+
+// multilinear interpolation in the cell at p, weights t and r = 1 - t
+template <int Q, int DE>
+__device__ __forceinline__ double cell_value(const double *p, const int (&S)[DE + 1], const double (&t)[DE + 1],
+                                             const double (&r)[DE + 1])
+{
+    if constexpr (Q == DE) return *p;
+    else return fma(t[Q], cell_value<Q + 1, DE>(p + S[Q], S, t, r), r[Q] * cell_value<Q + 1, DE>(p, S, t, r));
+}
+// sum over the groups of a run that blockIdx.y takes (every gridDim.y-th); place
+// and cell: this thread's columns of the tables
+template <int DE>
+__device__ __forceinline__ double run_value(const CombinePlan &C, const CombineRun &R, const double *M,
+                                            const double *place, const int *cell)
+{
+    int ax[DE + 1], fine[DE + 1];
+#pragma unroll
+    for (int q = 0, m = R.mask; q < DE; ++q, m &= m - 1) {
+        ax[q] = __ffs(m) - 1;
+        fine[q] = cell[ax[q] * 128];
+    }
+    double v = 0.0;
+    for (int g = R.first + blockIdx.y; g < R.last; g += gridDim.y) {
+        const CombineGroup &G = C.groups[g];
+        long long at = G.at;
+        int S[DE + 1];
+        double t[DE + 1], r[DE + 1];
+#pragma unroll
+        for (int q = 0; q < DE; ++q) {
+            const int lam = G.lev[q];
+            S[q] = G.stride[q];
+            t[q] = place[(ax[q] * C.l_max + lam - 1) * 128];
+            r[q] = 1.0 - t[q];
+            at += (long long)(fine[q] >> (C.l_max - lam)) * S[q];
+        }
+        v += cell_value<0, DE>(M + at, S, t, r);
+    }
+    return v;
+}
+// One thread a point.  What bounds it: the loads of the cells' corners, 608 a
+// point for d = 4, level 7, from L1 and L2, beside the FP64 unit (1,500
+// operations a point, 0.17 ms of its time for 65,794 points).  Those points take
+// 245 us with the addition of the groups (2,041 us grid by grid), 65,794 points
+// on d = 3, level 9 122 us (737), 200,000 on d = 2, level 8 71 us (199).  The place in the cell is tabulated per axis and level
+// on chip, once a point; the axes with one node (a grid of few listed axes has
+// few corners) give one factor for a run of groups.
+template <int D>
+__global__ void __launch_bounds__(128) combine_eval_kernel(const __grid_constant__ CombinePlan C, const GridInfo *grids,
+                                                           const int *levels, OpParams op, const double *M, int n_pts,
+                                                           const double *pts, double *dst)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, L = C.l_max;
+    if (k >= n_pts) return;  // (no barrier below: every thread reads its own columns)
+    double *place = reinterpret_cast<double *>(smem) + threadIdx.x;
+    int *cell = reinterpret_cast<int *>(smem + (size_t)D * L * 128 * 8) + threadIdx.x;
+    double one[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        // position in units of the domain (see combine_kernel); the cell of
+        // level lam is that of level L shifted down.  Outside the box the
+        // boundary cell's linear piece is continued.
+        const double xr = (pts[(long long)k * D + i] - op.lo[i]) / ldexp(grids[0].h[i], levels[i]);
+        const double c = floor(ldexp(xr, L));
+        const int top = (1 << L) - 1;
+        const int fine = c < 0.0 ? 0 : c > (double)top ? top : (int)c;
+        cell[i * 128] = fine;
+        double f = xr;  // place in the cell of level lam, from that of the level before
+        for (int lam = 1; lam <= L; ++lam) {
+            const bool right = (fine >> (L - lam)) & 1;
+            f = fma(2.0, f, right ? -1.0 : 0.0);
+            place[(i * L + lam - 1) * 128] = f;
+            if (lam == 1) one[i] = right ? 1.0 - f : f;
+        }
+    }
+    double acc = 0.0;
+    for (int q = 0; q < C.n_runs; ++q) {
+        const CombineRun R = C.runs[q];
+        double w = 1.0, v;
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+            if (!((R.mask >> i) & 1)) w *= one[i];
+        switch (__popc(R.mask)) {
+        case 0: v = run_value<0>(C, R, M, place, cell); break;
+        case 1: v = run_value<1>(C, R, M, place, cell); break;
+        case 2: if constexpr (D >= 2) v = run_value<2>(C, R, M, place, cell); break;
+        case 3: if constexpr (D >= 3) v = run_value<3>(C, R, M, place, cell); break;
+        case 4: if constexpr (D >= 4) v = run_value<4>(C, R, M, place, cell); break;
+        case 5: if constexpr (D >= 5) v = run_value<5>(C, R, M, place, cell); break;
+        default: if constexpr (D >= 6) v = run_value<6>(C, R, M, place, cell); break;
+        }
+        acc = fma(w, v, acc);
+    }
+    dst[(long long)blockIdx.y * n_pts + k] = acc;
+}
+
+size_t combine_eval_smem(int d, int l_max) { return (size_t)d * 128 * (8 * l_max + 4); }
+
+cudaError_t combine_init(size_t max_smem)
+{
+    const void *k[] = {(const void *)combine_eval_kernel<1>, (const void *)combine_eval_kernel<2>,
+                       (const void *)combine_eval_kernel<3>, (const void *)combine_eval_kernel<4>,
+                       (const void *)combine_eval_kernel<5>, (const void *)combine_eval_kernel<6>};
+    for (const void *f : k) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_combine_merged(const CombinePlan &C, const GridInfo *grids, const int *levels, const OpParams &op,
+                                  const double *u, double *M, int n_pts, const double *pts, double *out, int n_chunks,
+                                  double *part, cudaStream_t s)
+{
+    // (the chunks' sums, one or more, are added by a launch of their own)
+    if (n_chunks < 1 || !part) return cudaErrorInvalidValue;
+    merge_kernel<<<(unsigned)C.n_pieces, 256, 0, s>>>(C, u, M);
+    const dim3 grid((unsigned)((n_pts + 127) / 128), (unsigned)n_chunks);
+    const size_t smem = combine_eval_smem(op.d, C.l_max);
+    switch (op.d) {
+#define PIT_EVAL(D) \
+    case D: combine_eval_kernel<D><<<grid, 128, smem, s>>>(C, grids, levels, op, M, n_pts, pts, part); break;
+        PIT_EVAL(1) PIT_EVAL(2) PIT_EVAL(3) PIT_EVAL(4) PIT_EVAL(5) PIT_EVAL(6)
+#undef PIT_EVAL
+    default: return cudaErrorInvalidValue;
+    }
+    combine_sum_kernel<<<(n_pts + 127) / 128, 128, 0, s>>>(part, n_chunks, n_pts, out);
     return cudaGetLastError();
 }
 

@@ -263,18 +263,47 @@ cudaError_t launch_faces(const GridInfo *grids, int G, OpParams op, double *face
 // chunk set, partial sums in part[chunk * n_pts + k], n_chunks x n_pts doubles,
 // then added in chunk order); 1 means a single kernel writing out directly.
 int combine_chunks(int G, int n_pts, int n_sm);
-// (run_if: the kernel does nothing while *run_if is zero; NULL: always runs)
 cudaError_t launch_combine(const GridInfo *grids, const double *coef, const int *levels, int G, OpParams op,
                            const double *u, int n_pts, const double *pts, double *out, int n_chunks, double *part,
-                           cudaStream_t s, const int *run_if = nullptr);
-// The same sum from the sparse grid's surpluses S (launch_surpluses): nothing
-// is done while *skip_if is not zero.
-struct RecombPlan;
+                           cudaStream_t s);
+// The same sum over fewer grids: the grids that differ in the last axis' level
+// only are first added, with their coefficients, as one function on the finest
+// of them (a group), stored with its zero boundary values on the axes that have
+// more than one node.  Device pointers.
+struct CombineGroup {
+    long long at;               // where its array starts
+    int n;                      // nodes
+    int mask;                   // bit i: axis i is listed (has more than one node)
+    int term0, term1;           // its members
+    int stride[PIT_D];          // of the array along the listed axes, ascending
+    unsigned char lev[PIT_D];   // their levels
+    unsigned char pad[2];
+};
+struct CombineTerm {            // a member
+    long long off;              // packed offset of its grid
+    double coef;
+    int lev;                    // its level along the last axis
+    int pad;
+};
+struct CombinePiece {           // 256 nodes of a group
+    int group, first;
+};
+struct CombineRun {             // groups [first, last) with the same listed axes
+    int first, last, mask;
+};
+struct CombinePlan {
+    int n_pieces, n_runs, l_max;
+    const CombineGroup *groups;
+    const CombineTerm *terms;
+    const CombinePiece *pieces;
+    const CombineRun *runs;
+};
 size_t combine_eval_smem(int d, int l_max);
 cudaError_t combine_init(size_t max_smem);
-cudaError_t launch_combine_eval(const RecombPlan &R, const GridInfo *grids, const int *levels, const OpParams &op,
-                                const double *S, int n_pts, const double *pts, double *out, int n_chunks, double *part,
-                                const int *skip_if, cudaStream_t s);
+// M: the groups' arrays, boundary values zero already.
+cudaError_t launch_combine_merged(const CombinePlan &C, const GridInfo *grids, const int *levels, const OpParams &op,
+                                  const double *u, double *M, int n_pts, const double *pts, double *out, int n_chunks,
+                                  double *part, cudaStream_t s);
 // resid[j*G + g] = || a_j - b_j ||_2 on grid g, for active grids; j < nb.
 cudaError_t launch_resid_norms(const GridInfo *grids, int G, long long ntot, int nb, const double *a,
                                long long a_stride, const double *b, long long b_stride, const int *active,
@@ -304,20 +333,12 @@ struct RecombPiece {      // up to 256 nodes of a block of the sparse grid
     int first, n;         // first node in the block, nodes (a power of two)
     int list0, list1;     // the block's terms, ordered so that running sums of coefficients stay small
 };
-struct RecombEval {       // a block of the sparse grid, for evaluation at points
-    long long at;         // where it starts
-    unsigned char lam[PIT_D];
-    unsigned char from;   // first axis whose level differs from the block before
-    unsigned char pad;
-};
 // Classes of grids by where a CTA keeps the values: 0 in global memory, the
 // others on chip, split by size so that more CTAs of the smaller ones share an
 // SM (three, six and eight of 256 threads).
 constexpr int RECOMB_CLS = 4;
 struct RecombPlan {
     long long n_sparse;
-    int n_blk, l_max;              // blocks of the sparse grid, largest level
-    const RecombEval *eval;        // per block, lam ascending lexicographically
     int n_pieces;
     const RecombPiece *pieces;
     const RecombTerm *terms;
@@ -326,10 +347,6 @@ struct RecombPlan {
     int cls_first[RECOMB_CLS], cls_n[RECOMB_CLS];  // range of the grids by decreasing size
     size_t cls_smem[RECOMB_CLS];
 };
-// S = the sparse grid's surpluses of nb states (the first two of launch_recombine's
-// steps); *bad is set when a surplus is not finite (bad may be NULL).
-cudaError_t launch_surpluses(const RecombPlan &R, const GridInfo *grids, const int *order, long long ntot, int nb,
-                             const double *u, double *H, double *S, double *T, int *bad, cudaStream_t s);
 size_t recombine_smem_bytes(int n, int n_blocks, bool onchip);
 cudaError_t recombine_init(size_t max_smem);
 // out_b = Q u_b on every grid for nb consecutive states b (stride ntot; out

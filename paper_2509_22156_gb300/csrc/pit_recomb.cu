@@ -159,7 +159,7 @@ __device__ __forceinline__ void block_of(const Axes &A, int j, bool small, int &
 // One CTA per (grid, state).  T: natural-order scratch of a state for grids
 // whose values do not fit on chip (NULL: on chip, dynamic shared memory).
 __global__ void __launch_bounds__(256, 4) hier_kernel(RecombPlan R, const GridInfo *grids, const int *order, int n_order,
-                                                   long long ntot, const double *u, double *H, double *T, int *bad)
+                                                   long long ntot, const double *u, double *H, double *T)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ GridInfo G;
@@ -182,15 +182,11 @@ __global__ void __launch_bounds__(256, 4) hier_kernel(RecombPlan R, const GridIn
     __syncthreads();
     all_axes<false>(v, G);
     double *dst = H + b * ntot + G.off;
-    bool fin = true;
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         int blk, pos;
         block_of(A, j, small, blk, pos);
-        const double x = v[j];
-        fin = fin && (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
-        dst[tab[blk] + pos] = x;
+        dst[tab[blk] + pos] = v[j];
     }
-    if (bad && !fin) *bad = 1;
 }
 
 // One CTA of 256 threads per piece of a block (256 nodes at most) and state.
@@ -275,8 +271,8 @@ cudaError_t recombine_init(size_t max_smem)
                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
 }
 
-cudaError_t launch_surpluses(const RecombPlan &R, const GridInfo *grids, const int *order, long long ntot, int nb,
-                             const double *u, double *H, double *S, double *T, int *bad, cudaStream_t s)
+cudaError_t launch_recombine(const RecombPlan &R, const GridInfo *grids, const int *order, long long ntot, int nb,
+                             const double *u, double *H, double *S, double *T, double *out, cudaStream_t s)
 {
     if (nb <= 0) return cudaSuccess;
     if ((long long)R.n_pieces * nb > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -285,140 +281,12 @@ cudaError_t launch_surpluses(const RecombPlan &R, const GridInfo *grids, const i
     for (int c = 0; c < RECOMB_CLS; ++c)
         if (R.cls_n[c] > 0)
             hier_kernel<<<(unsigned)(R.cls_n[c] * nb), 256, R.cls_smem[c], s>>>(
-                R, grids, order + R.cls_first[c], R.cls_n[c], ntot, u, H, c == 0 ? T : nullptr, bad);
+                R, grids, order + R.cls_first[c], R.cls_n[c], ntot, u, H, c == 0 ? T : nullptr);
     gather_kernel<<<(unsigned)(R.n_pieces * nb), 256, 0, s>>>(R, ntot, H, S);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_recombine(const RecombPlan &R, const GridInfo *grids, const int *order, long long ntot, int nb,
-                             const double *u, double *H, double *S, double *T, double *out, cudaStream_t s)
-{
-    if (nb <= 0) return cudaSuccess;
-    const cudaError_t e = launch_surpluses(R, grids, order, ntot, nb, u, H, S, T, nullptr, s);
-    if (e != cudaSuccess) return e;
     for (int c = 0; c < RECOMB_CLS; ++c)
         if (R.cls_n[c] > 0)
             dehier_kernel<<<(unsigned)(R.cls_n[c] * nb), 256, R.cls_smem[c], s>>>(
                 R, grids, order + R.cls_first[c], R.cls_n[c], ntot, S, out, c != 0);
-    return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------
-// Combination sum at points from the sparse grid's surpluses.  The combined
-// solution is sum_lam S_{lam,p} prod_i phi(x_i), one basis function of every
-// increment being nonzero at a point: as many terms as there are increments
-// (210 for d = 4, level 7; 5,005 for d = 6, level 10) where the sum over grids
-// has 2^d corners of every grid (3,120 and 315,000).  A block's products of hat
-// values share those of the block before up to the first axis that differs, so
-// a term mostly costs one multiplication, one load and one FMA; the hat values
-// of every level are tabulated per point on chip.  ou4d level 7, 65,794 points:
-// 2,041 us as a sum over grids (FP64 unit 82 % busy), 139 us with the
-// surpluses' computation included.
-template <int D>
-__global__ void __launch_bounds__(128) combine_eval_kernel(RecombPlan R, const GridInfo *grids, const int *levels,
-                                                           OpParams op, const double *S, int n_pts, const double *pts,
-                                                           int bchunk, double *dst, const int *skip_if)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    if (*skip_if) return;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x, tid = threadIdx.x;
-    const int L = R.l_max;
-    double *phi = reinterpret_cast<double *>(smem);
-    if (k >= n_pts) return;  // (no barrier below: every thread reads its own table)
-    int P[D];
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-        // position in units of the domain (see combine_kernel); the cell of
-        // level lam is that of level L shifted down.  Outside the box the
-        // boundary cell's linear piece is continued.
-        const double xr = (pts[(long long)k * D + i] - op.lo[i]) / ldexp(grids[0].h[i], levels[i]);
-        const double c = floor(ldexp(xr, L));
-        const int top = (1 << L) - 1;
-        const int fine = c < 0.0 ? 0 : c > (double)top ? top : (int)c;
-        P[i] = fine >> 1;
-        // level by level: f in [0, 1) is the place in the cell, and the next
-        // level's bit of the cell number tells its half (two FP64 operations)
-        double f = xr;
-        for (int lam = 1; lam <= L; ++lam) {
-            const bool right = (fine >> (L - lam)) & 1;
-            phi[(i * L + lam - 1) * 128 + tid] = fma(right ? -2.0 : 2.0, f, right ? 2.0 : 0.0);
-            f = fma(2.0, f, right ? -1.0 : 0.0);
-        }
-    }
-    const int b0 = (int)blockIdx.y * bchunk, b1 = min(R.n_blk, b0 + bchunk);
-    double pr[D], acc = 0.0;
-    int ps[D];
-    // (eight terms at a time: their table entries and surpluses are loaded
-    // before the first sum)
-    constexpr int U = 8;
-    for (int b = b0; b < b1; b += U) {
-        RecombEval e[U];
-        double w[U], v[U];
-#pragma unroll
-        for (int q = 0; q < U; ++q) e[q] = R.eval[min(b + q, b1 - 1)];
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            const int from = b + q == b0 ? 0 : e[q].from;
-#pragma unroll
-            for (int i = 0; i < D; ++i)
-                if (i >= from) {
-                    const int lam = e[q].lam[i];
-                    const double f = phi[(i * L + lam - 1) * 128 + tid];
-                    pr[i] = i > 0 ? pr[i > 0 ? i - 1 : 0] * f : f;
-                    ps[i] = ((i > 0 ? ps[i > 0 ? i - 1 : 0] : 0) << (lam - 1)) + (P[i] >> (L - lam));
-                }
-            w[q] = pr[D - 1];
-            v[q] = S[e[q].at + ps[D - 1]];
-        }
-#pragma unroll
-        for (int q = 0; q < U; ++q)
-            if (b + q < b1) acc = fma(w[q], v[q], acc);
-    }
-    dst[(long long)blockIdx.y * n_pts + k] = acc;
-}
-
-__global__ void combine_eval_sum_kernel(const double *part, int n_chunks, int n_pts, double *out, const int *skip_if)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n_pts || *skip_if) return;
-    double s = 0.0;
-    for (int c = 0; c < n_chunks; ++c) s += part[(long long)c * n_pts + k];
-    out[k] = s;
-}
-
-size_t combine_eval_smem(int d, int l_max) { return (size_t)d * l_max * 128 * sizeof(double); }
-
-cudaError_t combine_init(size_t max_smem)
-{
-    const void *k[] = {(const void *)combine_eval_kernel<1>, (const void *)combine_eval_kernel<2>,
-                       (const void *)combine_eval_kernel<3>, (const void *)combine_eval_kernel<4>,
-                       (const void *)combine_eval_kernel<5>, (const void *)combine_eval_kernel<6>};
-    for (const void *f : k) {
-        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
-cudaError_t launch_combine_eval(const RecombPlan &R, const GridInfo *grids, const int *levels, const OpParams &op,
-                                const double *S, int n_pts, const double *pts, double *out, int n_chunks, double *part,
-                                const int *skip_if, cudaStream_t s)
-{
-    const int bchunk = (R.n_blk + n_chunks - 1) / n_chunks, chunks = (R.n_blk + bchunk - 1) / bchunk;
-    const dim3 grid((unsigned)((n_pts + 127) / 128), (unsigned)chunks);
-    const size_t smem = combine_eval_smem(op.d, R.l_max);
-    double *dst = chunks > 1 ? part : out;
-    switch (op.d) {
-#define PIT_EVAL(D)                                                                                              \
-    case D:                                                                                                      \
-        combine_eval_kernel<D><<<grid, 128, smem, s>>>(R, grids, levels, op, S, n_pts, pts, bchunk, dst, skip_if); \
-        break;
-        PIT_EVAL(1) PIT_EVAL(2) PIT_EVAL(3) PIT_EVAL(4) PIT_EVAL(5) PIT_EVAL(6)
-#undef PIT_EVAL
-    default: return cudaErrorInvalidValue;
-    }
-    if (chunks > 1)
-        combine_eval_sum_kernel<<<(n_pts + 127) / 128, 128, 0, s>>>(part, chunks, n_pts, out, skip_if);
     return cudaGetLastError();
 }
 
