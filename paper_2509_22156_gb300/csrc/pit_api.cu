@@ -882,6 +882,10 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
             I.ih2[i] = 1.0 / (I.h[i] * I.h[i]);
             if (I.h[i] < I.h[I.fine]) I.fine = i;
         }
+        for (int i = 0; i < d; ++i) {
+            I.sum2 += I.ih2[i];
+            if (I.N[i] == 1 && i != I.ax[0]) I.rest2 += I.ih2[i];
+        }
         double h2 = 1e300;
         for (int i = 0; i < d; ++i)
             if (i != I.fine && I.h[i] < h2) h2 = I.h[i];
@@ -896,10 +900,8 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
     P->direct_ok = desc->op == PIT_OP_HEAT;
     for (const GridInfo &I : P->info) {
         P->direct_ok = P->direct_ok && direct_grid(I);
-        double s = 0.0;
-        for (int i = 0; i < d; ++i) s += I.ih2[i];
         P->fix_n = std::max(P->fix_n, sqrt((double)I.n));
-        P->fix_h = std::max(P->fix_h, sqrt((double)I.n) * s);
+        P->fix_h = std::max(P->fix_h, sqrt((double)I.n) * I.sum2);
     }
     P->direct_dt = 1e300;
     for (int i = 0; i < d; ++i) {

@@ -36,11 +36,7 @@ struct FixConst {
 __device__ __forceinline__ void fix_const(const StepArgs &a, const GridInfo &G, FixConst &F)
 {
     if (threadIdx.x < 7) {
-        double sum = 0.0, rest = 0.0;
-        for (int i = 0; i < a.op.d; ++i) {
-            sum += a.dt * G.ih2[i];
-            if (G.N[i] == 1 && i != G.ax[0]) rest += a.dt * G.ih2[i];
-        }
+        const double sum = a.dt * G.sum2, rest = a.dt * G.rest2;
         // (every coefficient, and the sum of any of them, is below 2^{e+1}: hi < 2^31)
         const int e = max(0, (int)((__double2hiint(sum) >> 20) & 0x7ff) - 1023);  // sum 2^-e < 2
         const int q = threadIdx.x;

@@ -25,6 +25,7 @@ struct GridInfo {
     int S[PIT_D];
     double h[PIT_D];
     double ih2[PIT_D];  // 1 / h_i^2
+    double sum2, rest2; // sums of 1 / h_i^2 over every axis and over those not listed
     int ax[PIT_D];
     int fine;           // finest axis (the first of the finest), for the heat line preconditioner
     int fine_pc;        // it has at least three nodes and is at least twice as fine as every other axis

@@ -560,28 +560,28 @@ struct ItemConst {
 __device__ __forceinline__ void item_const(const StepArgs &a, const GridInfo &G, ItemConst &C)
 {
     const int t = threadIdx.x, D = G.de, d = a.op.d;
-    if (t < D) {
-        const double c = a.dt * G.ih2[G.ax[t]];
-        C.off[t] = -c;
-        C.off32[t] = (float)-c;
-        C.ch[t] = to_f32(c, 0);
-        C.cl[t] = to_f32(c - to_f64(C.ch[t], 0), 0);
-    } else if (t == 8) {
-        double diag = 1.0;
-        for (int i = 0; i < d; ++i) diag += 2.0 * a.dt * G.ih2[i];
-        C.diag = diag;
-        C.diag32 = (float)diag;
-    } else if (t == 9) {
-        double rest = 0.0;
-        for (int i = 0; i < d; ++i)
-            if (G.N[i] == 1 && i != G.ax[0]) rest += 2.0 * a.dt * G.ih2[i];
-        C.rh = to_f32(rest, 0);
-        C.rl = to_f32(rest - to_f64(C.rh, 0), 0);
-    } else if (t == 10) {
-        const double c = a.dt * G.ih2[G.fine];
-        C.offf = (float)-c;
-        C.use_pc = G.fine_pc && 4.0 * c >= 2.0;
-    } else if (t >= 16 && t < 16 + D * (D - 1) / 2) {
+    if (t < 16) {
+        // (one FP64 product for all: lanes that take different branches wait for
+        // one another)
+        const double c = a.dt * (t < D ? G.ih2[G.ax[t]] : t == 8 ? G.sum2 : t == 9 ? 2.0 * G.rest2 : G.ih2[G.fine]);
+        const float f = (float)c, hi = to_f32(c, 0), lo = to_f32(c - to_f64(hi, 0), 0);
+        if (t < D) {
+            C.off[t] = -c;
+            C.off32[t] = -f;
+            C.ch[t] = hi;
+            C.cl[t] = lo;
+        } else if (t == 8) {
+            const double diag = fma(2.0, c, 1.0);
+            C.diag = diag;
+            C.diag32 = (float)diag;
+        } else if (t == 9) {
+            C.rh = hi;
+            C.rl = lo;
+        } else if (t == 10) {
+            C.offf = -f;
+            C.use_pc = G.fine_pc && 4.0f * f >= 2.0f;
+        }
+    } else if (a.op.op == PIT_OP_LSDE && t < 16 + D * (D - 1) / 2) {  // mixed derivatives
         int q = 16, i = 0, k = 1;  // pair (i, k), i < k, number t - 16
         while (q < t) {
             if (++k == D) k = ++i + 1;
