@@ -121,6 +121,7 @@ struct pit_problem {
     struct Cluster { int cap = -1, reach = 0, de = 1; size_t smem = 0; } cluster[4];
     bool direct_ok = false;  // heat operator whose grids all take the direct solve
     double direct_dt = 0.0;  // largest step it is used for
+    int de_max = 1;            // most listed axes of a grid
     double fix_n = 0.0, fix_h = 0.0;  // largest n^{1/2}, n^{1/2} sum 1 / h^2 of a grid (error of the integer residual)
     int G = 0;
     long long ntot = 0;
@@ -307,13 +308,19 @@ pit_status check_solve_opts(const pit_solve_opts *o)
 // (class 1: the state x and b in the mixed form, x and the Krylov vectors in
 // the FP64 form; the FP32 form has no class 1).  Class 0 lists its grids by
 // decreasing shared-memory need, class 1 by decreasing size.
+// Axes of steps_kernel's body for a grid.  (The tables' length decides nothing
+// for grids of fewer axes: a set that has them has larger grids with more.)
+int body_axes(const pit_problem *P, int prec, const GridInfo &I)
+{
+    return own_body(P->desc.op, prec) ? I.de : P->de_max;
+}
 size_t grid_smem_bytes(const pit_problem *P, int prec, int g)
 {
     const GridInfo &I = P->info[g];
     int na = 1;
     for (int i = 0; i < P->desc.d; ++i) na = I.N[i] > na ? I.N[i] : na;
     if (prec > PAIR) return direct_smem_bytes(prec, I.n, na, false);
-    return phi_smem_bytes(prec, P->desc.op, I.de, I.n, na);
+    return phi_smem_bytes(prec, P->desc.op, body_axes(P, prec, I), I.n, na);
 }
 
 // Kernel form of a call: the refinements' FP32 solves are direct for the heat
@@ -357,7 +364,7 @@ pit_status plan(pit_problem *P, int prec)
         int na = 1;
         for (int i = 0; i < P->desc.d; ++i) na = P->info[g].N[i] > na ? P->info[g].N[i] : na;
         const size_t bx = prec > PAIR ? direct_smem_bytes(prec, n, na, true)
-                                      : phi_smem_bytes_xg(prec, P->desc.op, P->info[g].de, n);
+                                      : phi_smem_bytes_xg(prec, P->desc.op, body_axes(P, prec, P->info[g]), n);
         if (bx > P->max_smem)
             return fail(PIT_ERR_UNSUPPORTED,
                         "grid %d (%d nodes) needs %zu bytes of shared memory for the on-chip solve in this precision "
@@ -436,6 +443,7 @@ StepArgs make_args(pit_problem *P, const pit_solve_opts &o, const StepCall &c, c
     a.masks = P->d_masks;
     a.order = P->d_order;
     a.n_order = P->G;
+    a.de = P->de_max;
     a.n_grids = P->G;
     a.n_total = P->ntot;
     a.xg = nullptr;
@@ -900,6 +908,7 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
     P->direct_ok = desc->op == PIT_OP_HEAT;
     for (const GridInfo &I : P->info) {
         P->direct_ok = P->direct_ok && direct_grid(I);
+        P->de_max = std::max(P->de_max, I.de);
         P->fix_n = std::max(P->fix_n, sqrt((double)I.n));
         P->fix_h = std::max(P->fix_h, sqrt((double)I.n) * I.sum2);
     }

@@ -121,6 +121,7 @@ struct StepArgs {
     const uint16_t *masks;  // neighbour mask of every node over its grid's listed axes, packed like a state
     const int *order;       // the launch's grids, by decreasing size
     int n_order;            // grids in order
+    int de;                 // most listed axes of any grid of the problem
     int n_grids;            // all grids of the problem (row length of norms)
     int n_batch;
     int nsteps;
@@ -172,6 +173,14 @@ struct StepArgs {
 enum Prec { PLAIN = 0, MIXED = 1, SINGLE = 2, PAIR = 3, MIXED_D = 4, PAIR_D = 5 };
 constexpr int NPREC = 6;
 inline int base_form(int prec) { return prec == MIXED_D ? MIXED : prec == PAIR_D ? PAIR : prec; }
+// Whether steps_kernel runs a body of the grid's own listed axes: the FP64 form
+// (every coefficient that is left out saves the FP64 unit), and the variable-
+// coefficient operator (whose tables are the longer for it) and the
+// mixed-derivative one (whose pairs of axes are counted by it) in any form.
+__host__ __device__ constexpr bool own_body(int op, int prec)
+{
+    return prec == PLAIN || op == PIT_OP_VARHEAT || op == PIT_OP_LSDE;
+}
 // Launch parts of one multi-step call: NBKT shared-memory buckets of the
 // grids whose state fits on chip, then the grids with global-memory state.
 constexpr int NBKT = 4;
