@@ -207,9 +207,12 @@ typedef struct {
  *   DEFAULT  heat operator: in the refinement forms (PIT_PREC_MIXED,
  *            PIT_PREC_MIXED_PAIR) a direct FP32 solve of the correction
  *            equation (sine transforms of the short axes, counted as one
- *            Krylov iteration) where rtol <= 1e-4, maxit >= 16, dt is at most
- *            the smallest squared extent of the box and no grid has two axes
- *            of more than 31 nodes; else, and in the FP32 form, the line
+ *            Krylov iteration, inner_rtol not used) where rtol <= 1e-4, maxit
+ *            >= 16, dt is at most the smallest squared extent of the box, no
+ *            grid has two axes of more than 31 nodes and dt / h^2 of the finest
+ *            axis is so large that CG would take longer (1.5 for one step; 0.5
+ *            for several with forcing, 5 on pairs; several without forcing in
+ *            PIT_PREC_MIXED always); else, and in the FP32 form, the line
  *            preconditioner (tridiagonal along the finest axis, on anisotropic
  *            grids at stiff steps).  Other operators: none.
  *   NONE     no preconditioner.

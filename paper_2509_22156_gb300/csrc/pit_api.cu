@@ -121,6 +121,7 @@ struct pit_problem {
     struct Cluster { int cap = -1, reach = 0, de = 1; size_t smem = 0; } cluster[4];
     bool direct_ok = false;  // heat operator whose grids all take the direct solve
     double direct_dt = 0.0;  // largest step it is used for
+    double finest = 0.0;     // largest 1 / h^2
     int de_max = 1;            // most listed axes of a grid
     double fix_n = 0.0, fix_h = 0.0;  // largest n^{1/2}, n^{1/2} sum 1 / h^2 of a grid (error of the integer residual)
     int G = 0;
@@ -303,17 +304,18 @@ pit_status check_solve_opts(const pit_solve_opts *o)
     return PIT_OK;
 }
 
-// Launch plan of a precision form: grids whose on-chip state fits in shared
-// memory form class 0; the others keep their FP64 vectors in global memory
-// (class 1: the state x and b in the mixed form, x and the Krylov vectors in
-// the FP64 form; the FP32 form has no class 1).  Class 0 lists its grids by
-// decreasing shared-memory need, class 1 by decreasing size.
 // Axes of steps_kernel's body for a grid.  (The tables' length decides nothing
 // for grids of fewer axes: a set that has them has larger grids with more.)
 int body_axes(const pit_problem *P, int prec, const GridInfo &I)
 {
     return own_body(P->desc.op, prec) ? I.de : P->de_max;
 }
+
+// Launch plan of a precision form: grids whose on-chip state fits in shared
+// memory form class 0; the others keep their FP64 vectors in global memory
+// (class 1: the state x and b in the mixed form, x and the Krylov vectors in
+// the FP64 form; the FP32 form has no class 1).  Class 0 lists its grids by
+// decreasing shared-memory need, class 1 by decreasing size.
 size_t grid_smem_bytes(const pit_problem *P, int prec, int g)
 {
     const GridInfo &I = P->info[g];
@@ -321,24 +323,6 @@ size_t grid_smem_bytes(const pit_problem *P, int prec, int g)
     for (int i = 0; i < P->desc.d; ++i) na = I.N[i] > na ? I.N[i] : na;
     if (prec > PAIR) return direct_smem_bytes(prec, I.n, na, false);
     return phi_smem_bytes(prec, P->desc.op, body_axes(P, prec, I), I.n, na);
-}
-
-// Kernel form of a call: the refinements' FP32 solves are direct for the heat
-// operator where every grid allows it, unless
-//   - the caller chose a preconditioner (or none), or caps the iterations so low
-//     that a fixed number of them is what is asked for;
-//   - the tolerance is so loose that CG gets there in an iteration or two, for
-//     less than the direct solve's passes (coarse corrections to 1e-2, whose
-//     size MGRIT's cycle counts depend on);
-//   - the step is so large (dt above the squared extent of an axis, ext: twice
-//     dt) that 1 + dt L is nearly singular in FP32.
-int form_of(const pit_problem *P, const pit_solve_opts &o, double dt, bool ext = false)
-{
-    const int f = prec_form(o.prec);
-    if (!P->direct_ok || o.precond != PIT_PRECOND_DEFAULT || o.maxit < 16 || !(o.rtol <= 1e-4) ||
-        !((ext ? 2.0 : 1.0) * dt <= P->direct_dt))
-        return f;
-    return f == MIXED ? MIXED_D : f == PAIR ? PAIR_D : f;
 }
 
 pit_status plan(pit_problem *P, int prec)
@@ -434,6 +418,36 @@ struct StepCall {
     int sdirk = 0;    // two-stage SDIRK steps with stage step dt (coarse propagator PIT_COARSE_SDIRK2)
     int ext = 0;      // extrapolated backward-Euler steps with half step dt (PIT_COARSE_EXTRAP)
 };
+
+// Kernel form of a call: the refinements' FP32 solves are direct for the heat
+// operator where every grid allows it, unless
+//   - the caller chose a preconditioner (or none), or caps the iterations so low
+//     that a fixed number of them is what is asked for;
+//   - the tolerance is so loose that CG gets there in an iteration or two, for
+//     less than the direct solve's passes (coarse corrections to 1e-2, whose
+//     size MGRIT's cycle counts depend on);
+//   - the step is so large (dt above the squared extent of an axis, ext: twice
+//     dt) that 1 + dt L is nearly singular in FP32;
+//   - the step is so mild that CG needs one to three iterations, less than the
+//     direct solve's tables and 2 nax + 1 passes.  x = dt / h^2 of the finest
+//     axis is the measure: a call of one step from 1.5 on (us, CG and direct:
+//     x = 0.2, d = 2, level 6, 64 states 25 and 36; x = 0.8, d = 3, level 7, six
+//     states on pairs 34 and 46; x = 3.2, d = 2, level 8, one state 37 and 30);
+//     several steps on FP32 pairs from 5 on (40 steps, d = 5: x = 2.6 857 and
+//     1,172; d = 3, 100 steps, x = 10 1,873 and 1,562), with forcing from 0.5 on;
+//     several steps without forcing always, whose integer residual (pit_fixed.cuh)
+//     pays for the tables (d = 4, level 5, x = 0.04, 100 steps 554 and 473).
+int form_of(const pit_problem *P, const pit_solve_opts &o, const StepCall &c)
+{
+    const int f = prec_form(o.prec);
+    if (!P->direct_ok || o.precond != PIT_PRECOND_DEFAULT || o.maxit < 16 || !(o.rtol <= 1e-4) ||
+        !((c.ext ? 2.0 : 1.0) * c.dt <= P->direct_dt))
+        return f;
+    const bool carries = !c.f && !c.g && !c.guess && !c.sdirk && !c.ext;
+    const double from = c.nsteps == 1 ? 1.5 : f == PAIR ? 5.0 : carries ? 0.0 : 0.5;
+    if (c.dt * P->finest < from) return f;
+    return f == MIXED ? MIXED_D : f == PAIR ? PAIR_D : f;
+}
 
 StepArgs make_args(pit_problem *P, const pit_solve_opts &o, const StepCall &c, const int *active)
 {
@@ -637,7 +651,7 @@ pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_op
 pit_status run_steps(pit_problem *P, const pit_solve_opts &o, const StepCall &c, const int *active,
                      const pit_lane *L = nullptr)
 {
-    const int prec = form_of(P, o, c.dt, c.ext != 0);
+    const int prec = form_of(P, o, c);
     TRY(plan(P, prec));
     if (c.nb <= 0 || c.nsteps <= 0) return PIT_OK;
     if (L && !L->planned[prec]) return fail(PIT_ERR_INVALID_ARG, "lane without a launch plan");
@@ -909,6 +923,7 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
     for (const GridInfo &I : P->info) {
         P->direct_ok = P->direct_ok && direct_grid(I);
         P->de_max = std::max(P->de_max, I.de);
+        for (int i = 0; i < d; ++i) P->finest = std::max(P->finest, I.ih2[i]);
         P->fix_n = std::max(P->fix_n, sqrt((double)I.n));
         P->fix_h = std::max(P->fix_h, sqrt((double)I.n) * I.sum2);
     }
@@ -1885,8 +1900,6 @@ pit_status lanes_prime(Mg &M, int Nc)
                    {&o->crs, Nc / o->m, M.dt * o->m, o->m}};
     const int n_reps = o->levels == 3 ? 3 : 2;
     for (int r = 0; r < n_reps; ++r) {
-        const int prec = form_of(P, *reps[r].so, reps[r].dt);
-        TRY(plan(P, prec));
         if (reps[r].nb <= 0) continue;
         StepCall c;
         c.dt = reps[r].dt;
@@ -1894,7 +1907,9 @@ pit_status lanes_prime(Mg &M, int Nc)
         c.nsteps = reps[r].nsteps;
         c.in = P->m_U.d();  // u0 at every C-point
         c.is = nt;
-        // (the level-2 solves and the extrapolated steps may fall to the other form)
+        const int prec = form_of(P, *reps[r].so, c);
+        TRY(plan(P, prec));
+        // (the level-2 solves, the extrapolated and the forced steps may fall to the other form)
         if (P->n_cls[prec][1] > 0 || P->n_cls[base_form(prec)][1] > 0)
             CU(P->w_xg.ensure(sizeof(double) * nt * (size_t)Nc * xg_slabs(base_form(prec), P->desc.op, P->desc.d)));
         // (lane launches of extrapolated FP32 steps: the sweeps (one state per
@@ -1902,6 +1917,14 @@ pit_status lanes_prime(Mg &M, int Nc)
         if (prec == SINGLE && (o->coarse == PIT_COARSE_EXTRAP || o->init == 2))
             CU(P->w_scr.ensure(sizeof(float) * nt * (size_t)(o->levels == 3 && Nc / o->m > 1 ? Nc / o->m : 1)));
         for (int part = 0; part < NPART; ++part) TRY(tune(P, prec, c.nb >= 8, part, *reps[r].so, c, M.active));
+        // (mild steps with forcing run CG: their CTA sizes are chosen on the same states)
+        if (prec == MIXED_D && (r > 0 || M.F)) {
+            StepCall t = c;
+            t.g = P->m_Z.d();
+            const int form = form_of(P, *reps[r].so, t);
+            for (int part = 0; form != prec && part < NPART; ++part)
+                TRY(tune(P, form, c.nb >= 8, part, *reps[r].so, c, M.active));
+        }
     }
     return PIT_OK;
 }
@@ -2613,8 +2636,18 @@ extern "C" pit_status pit_phi_batch_inplace_static(pit_problem_t P, double dt, i
         }
         scratch = g_static_ptr[dev];
     }
+    StepCall c;
+    c.dt = dt;
+    c.nb = n_batch;
+    c.nsteps = 1;
+    c.in = u;
+    c.is = P->ntot;
+    c.f = f;
+    c.fs = P->ntot;
+    c.out_last = scratch;  // every node of every item is written: nothing needs clearing
+    c.ols = P->ntot;
     // (refused as the Krylov form is, whichever form runs)
-    const int prec = form_of(P, *opts, dt);
+    const int prec = form_of(P, *opts, c);
     // the launch plan was made when the problem was created; planning here
     // would allocate, so a form without a plan is refused
     if (!P->planned[prec] || !P->planned[base_form(prec)])
@@ -2627,16 +2660,6 @@ extern "C" pit_status pit_phi_batch_inplace_static(pit_problem_t P, double dt, i
     const bool wide = n_batch >= 8;
     const int family = wide ? 0 : 1;
     const int threads = P->threads[prec][family == 0 ? 1 : 0][0] ? P->threads[prec][family == 0 ? 1 : 0][0] : 128;
-    StepCall c;
-    c.dt = dt;
-    c.nb = n_batch;
-    c.nsteps = 1;
-    c.in = u;
-    c.is = P->ntot;
-    c.f = f;
-    c.fs = P->ntot;
-    c.out_last = scratch;  // every node of every item is written: nothing needs clearing
-    c.ols = P->ntot;
     StepArgs a = make_args(P, *opts, c, nullptr);
     a.order = P->d_order_cls[prec][0];
     a.n_order = P->n_cls[prec][0];
