@@ -154,7 +154,8 @@ struct pit_problem {
     // the CTAs of smaller grids pack more densely on an SM
     int split[NPREC][NBKT + 1] = {};
     size_t smem_bkt[NPREC][NBKT] = {};
-    int threads[NPREC][2][NPART] = {};  // [prec][wide batch][part: buckets, then global state]; 0 = not tuned
+    // [prec, or NPREC: MIXED_D with the integer state][wide batch][part: buckets, then global state]; 0 = not tuned
+    int threads[NPREC + 1][2][NPART] = {};
     int forced_threads[2] = {0, 0};  // override [wide batch]
     cudaStream_t sides[NPART - 1] = {};  // streams of the launch parts beside the first
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -576,7 +577,7 @@ int cluster_size(pit_problem *P, long long items)
 pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_opts &o, const StepCall &c,
                 const int *active)
 {
-    int &slot = P->threads[prec][wide ? 1 : 0][cls];
+    int &slot = P->threads[takes_fixed(prec, make_args(P, o, c, active)) ? NPREC : prec][wide ? 1 : 0][cls];
     if (slot) return PIT_OK;
     const PartView v = part_view(P, nullptr, prec, cls);
     if (v.n <= 0) return PIT_OK;
@@ -645,6 +646,16 @@ pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_op
     return PIT_OK;
 }
 
+// CTA size of a launch part.  A lane's launch may come before its own kernel was
+// tuned: the other one of the same state then gives the size, or 128.
+int cta_threads(const pit_problem *P, int prec, const StepArgs &a, bool wide, int part)
+{
+    const int own = takes_fixed(prec, a) ? NPREC : prec;
+    int t = P->threads[own][wide ? 1 : 0][part];
+    if (!t && prec == MIXED_D) t = P->threads[own == NPREC ? prec : NPREC][wide ? 1 : 0][part];
+    return t ? t : 128;
+}
+
 // One multi-step launch of every grid (of a lane, when given): class 0 on the
 // problem's (lane's) stream and, when present, class 1 (state in global
 // memory) concurrently on the side stream, joined before returning.
@@ -706,8 +717,7 @@ pit_status run_steps(pit_problem *P, const pit_solve_opts &o, const StepCall &c,
             count_kernels(P, wide ? 0 : 1);
             continue;
         }
-        const int nt = P->threads[prec][wide ? 1 : 0][q];  // (0: a lane's form that was not primed)
-        CU(launch_steps(prec, b, nt ? nt : 128, v[q].smem, sq, v[q].xg));
+        CU(launch_steps(prec, b, cta_threads(P, prec, b, wide, q), v[q].smem, sq, v[q].xg));
         count_kernels(P, wide ? 0 : 1);
     }
     if (fork) {
@@ -2659,7 +2669,6 @@ extern "C" pit_status pit_phi_batch_inplace_static(pit_problem_t P, double dt, i
                                          "pit_phi_batch_inplace_static cannot serve it");
     const bool wide = n_batch >= 8;
     const int family = wide ? 0 : 1;
-    const int threads = P->threads[prec][family == 0 ? 1 : 0][0] ? P->threads[prec][family == 0 ? 1 : 0][0] : 128;
     StepArgs a = make_args(P, *opts, c, nullptr);
     a.order = P->d_order_cls[prec][0];
     a.n_order = P->n_cls[prec][0];
@@ -2669,7 +2678,7 @@ extern "C" pit_status pit_phi_batch_inplace_static(pit_problem_t P, double dt, i
     a.stats = want ? P->d_stats + family : nullptr;
     {
         ProfScope ps(P, family);
-        CU(launch_steps(prec, a, threads, P->smem_need[prec], P->stream));
+        CU(launch_steps(prec, a, cta_threads(P, prec, a, wide, 0), P->smem_need[prec], P->stream));
         count_kernels(P, family);
     }
     CU(cudaMemcpyAsync(u, scratch, sizeof(double) * count, cudaMemcpyDeviceToDevice, P->stream));

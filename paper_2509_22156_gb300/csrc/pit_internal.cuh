@@ -173,6 +173,9 @@ struct StepArgs {
 enum Prec { PLAIN = 0, MIXED = 1, SINGLE = 2, PAIR = 3, MIXED_D = 4, PAIR_D = 5 };
 constexpr int NPREC = 6;
 inline int base_form(int prec) { return prec == MIXED_D ? MIXED : prec == PAIR_D ? PAIR : prec; }
+// Whether a launch of form prec runs the integer-state kernel (pit_fixed.cuh):
+// steps without forcing or a caller's guess carry their residual.
+bool takes_fixed(int prec, const StepArgs &a);
 // Whether steps_kernel runs a body of the grid's own listed axes: the FP64 form
 // (every coefficient that is left out saves the FP64 unit), and the variable-
 // coefficient operator (whose tables are the longer for it) and the

@@ -63,6 +63,11 @@ cudaError_t phi_kernels_init(size_t max_smem)
     return e;
 }
 
+bool takes_fixed(int prec, const StepArgs &a)
+{
+    return prec == MIXED_D && a.fixed && !a.f && !a.g && !a.guess && !a.sdirk && !a.ext;
+}
+
 cudaError_t launch_steps(int prec, const StepArgs &a, int threads, size_t smem, cudaStream_t s, bool xg)
 {
     const long long blocks = (long long)a.n_batch * a.n_order;
@@ -70,10 +75,7 @@ cudaError_t launch_steps(int prec, const StepArgs &a, int threads, size_t smem, 
     if (blocks > 0x7fffffffLL || smem > g_max_smem || threads < 32 || threads > 512 || (threads & 31))
         return cudaErrorInvalidConfiguration;
     const dim3 grid((unsigned)blocks), block(threads);
-    // (steps without forcing or a caller's guess carry their residual, and may
-    // hold the state as integers)
-    if (prec == MIXED_D && a.fixed && !a.f && !a.g && !a.guess && !a.sdirk && !a.ext)
-        return fixed_launch(a, grid, block, smem, s, xg);
+    if (takes_fixed(prec, a)) return fixed_launch(a, grid, block, smem, s, xg);
     if (prec == MIXED_D) return direct_launch_mixed(a, grid, block, smem, s, xg);
     if (prec == PAIR_D) return direct_launch_pair(a, grid, block, smem, s, xg);
     if (prec == SINGLE && xg) {
