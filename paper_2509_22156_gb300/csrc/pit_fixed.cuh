@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
         mask[j] = gmask[j];
     }
     R64.template sum<1>(ss);
-    const bool bad = !(ss[0] < 1e300);
+    const bool bad = !(ss[0] <= 1.7976931348623157e308);  // (infinite or NaN)
     const int E = FC.E;
     int k = min(max(scale_exp(ss[0]) + 56, -900), 900);  // the state is held times 2^k
     {

@@ -152,3 +152,19 @@ def test_steps_that_shrink_the_state_many_times_over(d, n, dt, steps, kind):
             sl = slice(P.offsets[g], P.offsets[g + 1])
             off = np.linalg.norm(got[sl] - ref[-1][sl])
             assert off <= 1.25e-11 * sum(np.linalg.norm(r[sl]) for r in ref[:-1]), g
+
+
+def test_states_near_the_end_of_the_double_range():
+    # a squared norm of up to 1.8e308 is finite, as in the form with the FP64 check
+    P = B.Problem(3, 5, 1, W.OP_HEAT)
+    u = W.random_vector(9, P.n_total)
+    most = max(float(np.sum(u[P.offsets[g]:P.offsets[g + 1]] ** 2)) for g in range(P.G))
+    e = (1023 - int(np.ceil(np.log2(most)))) // 2  # the largest norm squared times 4^e is below 2^1023
+    assert np.ldexp(most, 2 * e) > 1e304
+    a, _ = solve(P, u, 1e-3, 12, opts())
+    b, st = solve(P, np.ldexp(u, e), 1e-3, 12, opts())
+    assert st.n_failed == 0
+    np.testing.assert_array_equal(b, np.ldexp(a, e))
+    with pytest.raises(B.PitError) as err:
+        solve(P, np.ldexp(u, e + 3), 1e-3, 12, opts())
+    assert err.value.status == B.PIT_ERR_NONFINITE
