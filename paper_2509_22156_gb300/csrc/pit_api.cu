@@ -190,7 +190,7 @@ struct pit_problem {
     RecombTerm *rc_terms = nullptr;
     RecombBlock *rc_blocks = nullptr;
     long long *rc_grid_blocks = nullptr;
-    DBuf rc_H, rc_S, rc_T, rc_cur;
+    DBuf rc_H, rc_S, rc_cur;
     // combination sum over groups of grids, built on first use (host part, then
     // device tables and the groups' arrays)
     bool cb_grouped = false, cb_ready = false;
@@ -1061,7 +1061,6 @@ pit_status pit_problem_destroy(pit_problem_t P)
     cudaFree(P->rc_grid_blocks);
     P->rc_H.release();
     P->rc_S.release();
-    P->rc_T.release();
     P->rc_cur.release();
     P->cb_tab.release();
     P->cb_M.release();
@@ -1449,10 +1448,8 @@ pit_status recombine(pit_problem *P, const double *u, double *out, int nb = 1)
     TRY(recomb_plan(P));
     CU(P->rc_H.ensure(sizeof(double) * P->ntot * (size_t)nb));
     CU(P->rc_S.ensure(sizeof(double) * P->rc.n_sparse * (size_t)nb));
-    if (P->rc.cls_n[0] > 0) CU(P->rc_T.ensure(sizeof(double) * P->ntot * (size_t)nb));
     ProfScope ps(P, 3);
-    CU(launch_recombine(P->rc, P->d_grids, P->d_order, P->ntot, nb, u, P->rc_H.d(), P->rc_S.d(), P->rc_T.d(), out,
-                        P->stream));
+    CU(launch_recombine(P->rc, P->d_grids, P->d_order, P->ntot, nb, u, P->rc_H.d(), P->rc_S.d(), out, P->stream));
     int kernels = 1;
     for (int c = 0; c < RECOMB_CLS; ++c) kernels += P->rc.cls_n[c] > 0 ? 2 : 0;
     count_kernels(P, 3, kernels);

@@ -363,9 +363,10 @@ struct RecombPlan {
 size_t recombine_smem_bytes(int n, int n_blocks, bool onchip);
 cudaError_t recombine_init(size_t max_smem);
 // out_b = Q u_b on every grid for nb consecutive states b (stride ntot; out
-// may alias u); H: nb x n_total, S: nb x n_sparse doubles of scratch, T: nb x
-// n_total doubles when class 0 is not empty; order: the grids by decreasing size.
+// may be u); H: nb x n_total, S: nb x n_sparse doubles of scratch (the grids of
+// class 0 also use out, which is complete only at the end); order: the grids by
+// decreasing size.
 cudaError_t launch_recombine(const RecombPlan &R, const GridInfo *grids, const int *order, long long ntot, int nb,
-                             const double *u, double *H, double *S, double *T, double *out, cudaStream_t s);
+                             const double *u, double *H, double *S, double *out, cudaStream_t s);
 
 }  // namespace pit

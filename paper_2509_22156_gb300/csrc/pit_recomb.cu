@@ -157,7 +157,8 @@ __device__ __forceinline__ void block_of(const Axes &A, int j, bool small, int &
 }
 
 // One CTA per (grid, state).  T: natural-order scratch of a state for grids
-// whose values do not fit on chip (NULL: on chip, dynamic shared memory).
+// whose values do not fit on chip, may be u (NULL: on chip, dynamic shared
+// memory).
 __global__ void __launch_bounds__(256, 4) hier_kernel(RecombPlan R, const GridInfo *grids, const int *order, int n_order,
                                                    long long ntot, const double *u, double *H, double *T)
 {
@@ -272,7 +273,7 @@ cudaError_t recombine_init(size_t max_smem)
 }
 
 cudaError_t launch_recombine(const RecombPlan &R, const GridInfo *grids, const int *order, long long ntot, int nb,
-                             const double *u, double *H, double *S, double *T, double *out, cudaStream_t s)
+                             const double *u, double *H, double *S, double *out, cudaStream_t s)
 {
     if (nb <= 0) return cudaSuccess;
     if ((long long)R.n_pieces * nb > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -281,7 +282,7 @@ cudaError_t launch_recombine(const RecombPlan &R, const GridInfo *grids, const i
     for (int c = 0; c < RECOMB_CLS; ++c)
         if (R.cls_n[c] > 0)
             hier_kernel<<<(unsigned)(R.cls_n[c] * nb), 256, R.cls_smem[c], s>>>(
-                R, grids, order + R.cls_first[c], R.cls_n[c], ntot, u, H, c == 0 ? T : nullptr);
+                R, grids, order + R.cls_first[c], R.cls_n[c], ntot, u, H, c == 0 ? out : nullptr);
     gather_kernel<<<(unsigned)(R.n_pieces * nb), 256, 0, s>>>(R, ntot, H, S);
     for (int c = 0; c < RECOMB_CLS; ++c)
         if (R.cls_n[c] > 0)

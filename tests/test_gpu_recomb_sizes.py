@@ -37,3 +37,20 @@ def test_recombination_matches_oracle(d, n, L0):
     assert np.linalg.norm(out.cpu().numpy() - ref) <= 1e-12 * np.linalg.norm(ref)
     P.recombine(ud, ud)  # in place: the same kernels, the same sums
     assert torch.equal(ud, out)
+
+
+def test_grids_in_global_memory_take_no_further_state():
+    # the surpluses of every grid and of the sparse grid, and the plan; a grid too large for the chip is worked on in
+    # the result's own place
+    P = B.Problem(2, 17, 1, W.OP_HEAT)
+    u = torch.from_numpy(W.random_vector(5, P.n_total)).cuda()
+    out = torch.empty_like(u)
+    n_sparse = 16 * 2 ** 17 + 1  # increments lam with |lam| <= n + 1: 2^(|lam| - 2) nodes each
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    P.recombine(u, out)
+    torch.cuda.synchronize()
+    taken = before - torch.cuda.mem_get_info()[0]
+    assert taken <= 8 * (P.n_total + n_sparse) + (8 << 20)
+    P.recombine(u, u)
+    assert torch.equal(u, out)
