@@ -1423,6 +1423,8 @@ pit_status recomb_plan(pit_problem *P)
         }
     }
     auto up = [&](auto *&dst, const auto &v) -> cudaError_t {
+        cudaFree(dst);  // (of an earlier call that ran out of memory)
+        dst = nullptr;
         cudaError_t e = dev_malloc(&dst, sizeof(v[0]) * v.size());
         if (e != cudaSuccess) return e;
         return cudaMemcpy(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice);
