@@ -438,6 +438,11 @@ __device__ __forceinline__ void net_weight_grad(const NetItem<D> &I, int k, cons
         }
         __syncthreads();
         if (active) {
+            // (a tile's sum by itself: the rounding errors of the whole grow with
+            // the tiles, not with the nodes)
+            float part[8];
+#pragma unroll
+            for (int o = 0; o < 8; ++o) part[o] = 0.0f;
             const float4 *z4 = reinterpret_cast<const float4 *>(I.zt + row * NET_TLD + split * (NET_TILE / 2));
 #pragma unroll 2
             for (int q = 0; q < NET_TILE / 8; ++q) {
@@ -445,12 +450,14 @@ __device__ __forceinline__ void net_weight_grad(const NetItem<D> &I, int k, cons
 #pragma unroll
                 for (int o = 0; o < 8; ++o) {
                     const float4 d = reinterpret_cast<const float4 *>(I.dt + (grp * 8 + o) * NET_TLD + split * (NET_TILE / 2))[q];
-                    acc[o] = fmaf(d.x, z.x, acc[o]);
-                    acc[o] = fmaf(d.y, z.y, acc[o]);
-                    acc[o] = fmaf(d.z, z.z, acc[o]);
-                    acc[o] = fmaf(d.w, z.w, acc[o]);
+                    part[o] = fmaf(d.x, z.x, part[o]);
+                    part[o] = fmaf(d.y, z.y, part[o]);
+                    part[o] = fmaf(d.z, z.z, part[o]);
+                    part[o] = fmaf(d.w, z.w, part[o]);
                 }
             }
+#pragma unroll
+            for (int o = 0; o < 8; ++o) acc[o] += part[o];
         }
     }
     __syncthreads();
