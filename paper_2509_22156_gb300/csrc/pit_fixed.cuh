@@ -163,8 +163,19 @@ __global__ void __launch_bounds__(512, 1) fixed_kernel(const __grid_constant__ S
     }
     R64.template sum<1>(ss);
     const bool bad = !(ss[0] <= 1.7976931348623157e308);  // (infinite or NaN)
+    int up0 = 0;
+    if (ss[0] < 0x1p-900) {
+        // (squares at the double range's other end: the norm of the state times 2^500)
+        up0 = 500;
+        ss[0] = 0.0;
+        for (int j = tid; j < n; j += nt) {
+            const double v = in[j] * 0x1p500;
+            ss[0] += v * v;
+        }
+        R64.template sum<1>(ss);
+    }
     const int E = FC.E;
-    int k = min(max(scale_exp(ss[0]) + 56, -900), 900);  // the state is held times 2^k
+    int k = min(max(scale_exp(ss[0]) + 56 + up0, -900), 900);  // the state is held times 2^k
     {
         const double up = pow2d(k);
         for (int j = tid; j < n; j += nt) x[j] = bad ? 0 : __double2ll_rn(in[j] * up);

@@ -168,3 +168,14 @@ def test_states_near_the_end_of_the_double_range():
     with pytest.raises(B.PitError) as err:
         solve(P, np.ldexp(u, e + 3), 1e-3, 12, opts())
     assert err.value.status == B.PIT_ERR_NONFINITE
+
+
+def test_states_whose_squares_leave_the_double_range():
+    # norms from 2^-500 to 2^-750: the squared norm is subnormal or zero from about 2^-511 on
+    P = B.Problem(3, 5, 1, W.OP_HEAT)
+    u = W.random_vector(9, P.n_total)
+    a, _ = solve(P, u, 1e-3, 12, opts())
+    for e in (-500, -512, -520, -535, -545, -750):
+        b, st = solve(P, np.ldexp(u, e), 1e-3, 12, opts())
+        assert st.n_failed == 0
+        np.testing.assert_array_equal(b, np.ldexp(a, e))
