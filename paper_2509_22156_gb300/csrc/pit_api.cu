@@ -446,7 +446,7 @@ int form_of(const pit_problem *P, const pit_solve_opts &o, const StepCall &c)
         return f;
     const bool carries = !c.f && !c.g && !c.guess && !c.sdirk && !c.ext;
     const double from = c.nsteps == 1 ? 1.5 : f == PAIR ? 5.0 : carries ? 0.0 : 0.5;
-    if (c.dt * P->finest < from) return f;
+    if (!(c.dt > 0.0) || c.dt * P->finest < from) return f;  // (dt = 0: the state as it is, bit by bit)
     return f == MIXED ? MIXED_D : f == PAIR ? PAIR_D : f;
 }
 

@@ -179,3 +179,13 @@ def test_states_whose_squares_leave_the_double_range():
         b, st = solve(P, np.ldexp(u, e), 1e-3, 12, opts())
         assert st.n_failed == 0
         np.testing.assert_array_equal(b, np.ldexp(a, e))
+
+
+@pytest.mark.parametrize("prec", [B.PIT_PREC_MIXED, B.PIT_PREC_FP64])
+def test_steps_of_length_zero_return_the_state(prec):
+    P = B.Problem(3, 5, 1, W.OP_HEAT)
+    u = W.random_vector(9, P.n_total) * 10.0 ** W.random_vector(10, P.n_total, -40, 0)
+    for steps in (1, 5):
+        got, st = solve(P, u, 0.0, steps, B.solve_opts(prec, rtol=1e-11, maxit=4000, inner_rtol=1e-6, ir_maxit=12))
+        assert st.n_failed == 0
+        np.testing.assert_array_equal(got, u)
