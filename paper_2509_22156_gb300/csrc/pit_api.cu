@@ -122,7 +122,7 @@ struct pit_problem {
     bool direct_ok = false;  // heat operator whose grids all take the direct solve
     double direct_dt = 0.0;  // largest step it is used for
     double finest = 0.0;     // largest 1 / h^2
-    int de_max = 1;            // most listed axes of a grid
+    int de_max = 1, n_max = 0; // most listed axes and nodes of a grid
     double fix_n = 0.0, fix_h = 0.0;  // largest n^{1/2}, n^{1/2} sum 1 / h^2 of a grid (error of the integer residual)
     int G = 0;
     long long ntot = 0;
@@ -458,7 +458,8 @@ StepArgs make_args(pit_problem *P, const pit_solve_opts &o, const StepCall &c, c
     a.masks = P->d_masks;
     a.order = P->d_order;
     a.n_order = P->G;
-    a.de = P->de_max;
+    // (see steps_kernel)
+    a.de = P->desc.op == PIT_OP_VARHEAT && (long long)c.nb * P->G <= P->n_sm && P->n_max >= 256 ? 0 : P->de_max;
     a.n_grids = P->G;
     a.n_total = P->ntot;
     a.xg = nullptr;
@@ -933,6 +934,7 @@ pit_status pit_problem_create(const pit_problem_desc *desc, void *stream, pit_pr
     for (const GridInfo &I : P->info) {
         P->direct_ok = P->direct_ok && direct_grid(I);
         P->de_max = std::max(P->de_max, I.de);
+        P->n_max = std::max(P->n_max, I.n);
         for (int i = 0; i < d; ++i) P->finest = std::max(P->finest, I.ih2[i]);
         P->fix_n = std::max(P->fix_n, sqrt((double)I.n));
         P->fix_h = std::max(P->fix_h, sqrt((double)I.n) * I.sum2);

@@ -121,7 +121,7 @@ struct StepArgs {
     const uint16_t *masks;  // neighbour mask of every node over its grid's listed axes, packed like a state
     const int *order;       // the launch's grids, by decreasing size
     int n_order;            // grids in order
-    int de;                 // most listed axes of any grid of the problem
+    int de;                 // most listed axes of any grid of the problem (0: steps_kernel's bodies are each grid's own)
     int n_grids;            // all grids of the problem (row length of norms)
     int n_batch;
     int nsteps;
@@ -176,14 +176,10 @@ inline int base_form(int prec) { return prec == MIXED_D ? MIXED : prec == PAIR_D
 // Whether a launch of form prec runs the integer-state kernel (pit_fixed.cuh):
 // steps without forcing or a caller's guess carry their residual.
 bool takes_fixed(int prec, const StepArgs &a);
-// Whether steps_kernel runs a body of the grid's own listed axes: the FP64 form
-// (every coefficient that is left out saves the FP64 unit), and the variable-
-// coefficient operator (whose tables are the longer for it) and the
-// mixed-derivative one (whose pairs of axes are counted by it) in any form.
-__host__ __device__ constexpr bool own_body(int op, int prec)
-{
-    return prec == PLAIN || op == PIT_OP_VARHEAT || op == PIT_OP_LSDE;
-}
+// Whether steps_kernel always runs a body of the grid's own listed axes: the FP64
+// form (every coefficient that is left out saves the FP64 unit) and the
+// mixed-derivative operator (whose pairs of axes are counted by it).
+__host__ __device__ constexpr bool own_body(int op, int prec) { return prec == PLAIN || op == PIT_OP_LSDE; }
 // Launch parts of one multi-step call: NBKT shared-memory buckets of the
 // grids whose state fits on chip, then the grids with global-memory state.
 constexpr int NBKT = 4;

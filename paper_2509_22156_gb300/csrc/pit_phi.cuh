@@ -1201,13 +1201,17 @@ __device__ __forceinline__ void steps_item(const StepArgs &a, const GridInfo &GI
             });
             if constexpr (!own_body(OP, PREC))
                 for (int q = GI.de; q < D; ++q) {
-                    if constexpr (PREC != SINGLE) tab64[(1 + 2 * q) * tld + j] = tab64[(2 + 2 * q) * tld + j] = 0.0;
+                    if constexpr (PREC == PAIR)
+                        reinterpret_cast<float2 *>(tab64)[2 * q * ld + j] =
+                            reinterpret_cast<float2 *>(tab64)[(2 * q + 1) * ld + j] = make_float2(0.0f, 0.0f);
+                    else if constexpr (PREC != SINGLE)
+                        tab64[(1 + 2 * q) * tld + j] = tab64[(2 + 2 * q) * tld + j] = 0.0;
                     tab32[(1 + 2 * q) * ld + j] = tab32[(2 + 2 * q) * ld + j] = 0.0f;
                 }
             if constexpr (PREC != SINGLE && PREC != PAIR) tab64[j] = diag;
             if constexpr (PREC == PAIR) {
                 // faces of the axes that are not listed (on one node, of all but axis 0)
-                if (D < a.op.d) {
+                if (GI.de < a.op.d) {
                     double rest = 0.0;
                     for (int i = 0; i < a.op.d; ++i)
                         if (GI.N[i] == 1 && i != GI.ax[0])
@@ -1278,7 +1282,7 @@ __device__ __forceinline__ void steps_item(const StepArgs &a, const GridInfo &GI
         PT.mask = mask;
         PT.c = reinterpret_cast<const float2 *>(tab64);
         PT.ld = ld;
-        PT.rest = D < a.op.d;
+        PT.rest = GI.de < a.op.d;
 #pragma unroll
         for (int i = 0; i < D; ++i) PT.S[i] = GI.S[GI.ax[i]];
     }
@@ -2085,7 +2089,10 @@ __device__ __forceinline__ void steps_item(const StepArgs &a, const GridInfo &GI
 // grids then has one body in the instruction caches instead of up to six (d =
 // 6, level 7, 40 steps on FP32 pairs: 1,229 us with a body per number of axes,
 // 672 with one; four-dimensional OU, level 5, 60 steps in refinement: 499 and
-// 379).
+// 379; MGRIT of the variable-coefficient problem, d = 3, level 8: 55.6 and 50.6
+// ms).  The variable-coefficient operator keeps the grids' own (a.de = 0) where
+// every CTA has an SM to itself and the largest grid at least 256 nodes: 256
+// steps at d = 3, level 8, 2,045 us, 2,114 with one.
 template <int OP, int PREC, bool XG>
 __global__ void __launch_bounds__(512, 1) steps_kernel(const __grid_constant__ StepArgs a)
 {
@@ -2107,7 +2114,7 @@ __global__ void __launch_bounds__(512, 1) steps_kernel(const __grid_constant__ S
     __syncthreads();
     item_const(a, GI, IC);
     __syncthreads();
-    switch (own_body(OP, PREC) ? GI.de : a.de) {
+    switch (own_body(OP, PREC) || (OP == PIT_OP_VARHEAT && a.de == 0) ? GI.de : a.de) {
     case 1: steps_item<OP, PREC, 1, XG>(a, GI, IC, g, b, red64, red32); break;
     case 2: steps_item<OP, PREC, 2, XG>(a, GI, IC, g, b, red64, red32); break;
     case 3: steps_item<OP, PREC, 3, XG>(a, GI, IC, g, b, red64, red32); break;
