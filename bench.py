@@ -51,8 +51,8 @@ SM_COUNT = 152
 FP32_FMA_TFLOPS = 73.1      # (nominal 152 SMs x 128 lanes x 2 x 2.07 GHz = 80.5)
 FP64_FMA_TFLOPS = 1.195     # (nominal 1.25)
 SMEM_LOAD_GBS = 39315.0     # (nominal 152 SMs x 128 B/clk x 2.07 GHz = 40,274)
-PREC_NAMES = ["fp64", "mixed (FP32 Krylov in FP64 refinement)", "fp32",
-              "pair (FP32 Krylov in a refinement on FP32 pairs)"]
+PREC_NAMES = ["fp64", "mixed (FP32 corrections in FP64 refinement)", "fp32",
+              "pair (FP32 corrections in a refinement on FP32 pairs)"]
 # Algorithmic HBM bytes per node (the minimum schedule of the solves, counted
 # in units of one scalar per node): an FP32 CG iteration moves 10 FP32 vectors
 # (40 B: the stencil pass reads r, p and writes p, q; the update pass reads x,
@@ -166,6 +166,7 @@ def measured_peaks():
 
 
 HBM_FALLBACK_GBS = 6800.0
+ISSUE_GLANE = 152 * 4 * 32 * 2.07  # lane instructions a nanosecond at the maximum clock
 
 
 def phi_source_hash() -> str:
@@ -194,12 +195,13 @@ def phi_source_hash() -> str:
 NCU_SUMMARY = {5: "fixed_kernel_heat6d.txt", 2: "steps_kernel_heat_mixed_heat3d_n9.txt"}
 
 
-def ncu_traffic(wl_k):
-    """DRAM bytes per node-step of the relaxation kernel from the committed ncu
-    summary, or None when there is none or the kernel source changed since."""
+def ncu_figures(wl_k):
+    """(DRAM bytes, lane instructions) per node-step of the relaxation kernel from
+    the committed ncu summary; None where there is none or the kernel source
+    changed since."""
     name = NCU_SUMMARY.get(wl_k)
     if name is None:
-        return None
+        return None, None
     try:
         kv = {}
         for line in open(os.path.join(ROOT, "profiles", name)):
@@ -207,10 +209,11 @@ def ncu_traffic(wl_k):
                 k, v = line.split(":", 1)
                 kv[k.strip()] = v.strip()
         if kv.get("source_sha256_16") != phi_source_hash():
-            return None
-        return float(kv["dram_bytes_per_node_step"])
+            return None, None
+        lane = kv.get("lane_instructions_per_node_step")
+        return float(kv["dram_bytes_per_node_step"]), None if lane is None else float(lane)
     except Exception:
-        return None
+        return None, None
 
 
 # ---------------------------------------------------------------------------
@@ -288,7 +291,7 @@ def inner_rtol(B, prec):
 
 
 def solver_setup(wl, B, tol=None, rtol=None, coarse=None, relax=None, coarse_prec=None, init=True, fine_prec=None):
-    """Options of the chosen form (FP32 Krylov inside FP64 iterative
+    """Options of the chosen form (FP32 corrections inside iterative
     refinement for every fine solve, learned coarse propagator or the
     implicit one solved for the correction with a loose tolerance) and of the
     plain FP64 form (the paper's algorithm: FAS form of Alg. 2, FP64 Krylov,
@@ -367,11 +370,15 @@ def train_network(P, wl, B, mixed, epochs, seed=0):
 
 
 def roofline_block(B, wl, prof, chosen, k):
-    """Roofline of the dominant kernel, the relaxation launches (family 0:
-    many entries per grid) of the timed region: algorithmic HBM bytes from the
-    kernel's own work counters (node x Krylov iterations, node x refinement
-    passes) over those launches' CUDA-event time, against the measured copy
-    bandwidth; the FP64-pipe, FP32 and shared-memory views beside it."""
+    """Roofline of the dominant kernel, the relaxation launches (family 0: many
+    entries per grid) of the timed region, over those launches' CUDA-event time.
+    Krylov forms: algorithmic HBM bytes from the kernel's own work counters
+    (node x Krylov iterations, node x refinement passes) against the measured
+    copy bandwidth, with the FP64-pipe, FP32 and shared-memory views.  Heat
+    refinements (direct solves and integer residuals on chip, about one byte of
+    DRAM traffic a node-step): the instructions issued, from the committed
+    profile's count per node-step, against the issue rate, with the DRAM traffic
+    beside it."""
     d = wl.d
     relax_ms = prof.ms[0]
     iters, passes, steps = prof.point_iters_f[0], prof.point_passes_f[0], prof.point_steps_f[0]
@@ -398,14 +405,12 @@ def roofline_block(B, wl, prof, chosen, k):
         f_pass = (39 * d + 31) if wl.op == B.PIT_OP_HEAT else (46 * d + 31)
     fp32_flops = iters * f_it + passes * f_pass
     smem_b = 2 + 4 * (2 * d + 1) + 4 + 16 + 8 + 8 + 4  # shared-memory bytes per node and FP32 CG iteration
-    trf = ncu_traffic(k)
+    trf, lane = ncu_figures(k)
     views = {
         "fp64_pipe": {"achieved": fp64_flops / t / 1e12 if t else None, "peak": FP64_FMA_TFLOPS, "unit": "TFLOP/s",
                       "frac": (fp64_flops / t / 1e12 / FP64_FMA_TFLOPS) if t else None,
                       "flops_per_node_pass": 3 * d + 4,
                       "op_mix_limit_frac": (3 * d + 4) / (2.0 * (2 * d + 3)),
-                      "note": "checks without forcing run on integer pipes and are counted as the FP64 passes "
-                              "that they replace" if wl.op == B.PIT_OP_HEAT else "",
                       "peak_source": "measured FP64 FMA probe on this pool"},
         "fp32": {"achieved": fp32_flops / t / 1e12 if t else None, "peak": FP32_FMA_TFLOPS, "unit": "TFLOP/s",
                  "frac": (fp32_flops / t / 1e12 / FP32_FMA_TFLOPS) if t else None,
@@ -415,28 +420,36 @@ def roofline_block(B, wl, prof, chosen, k):
                  "frac": (iters * smem_b / t / 1e9 / SMEM_LOAD_GBS) if t else None,
                  "bytes_per_node_iter": smem_b, "peak_source": "measured shared-memory load probe on this pool"},
     }
-    # heat refinements: direct FP32 solves, and without forcing integer checks;
-    # a solve counts as the iteration and a check as the pass that it replaces
-    direct = wl.op == B.PIT_OP_HEAT and prec != B.PIT_PREC_FP64
-    kern = {B.PIT_PREC_MIXED: "fixed_kernel and direct_kernel", B.PIT_PREC_MIXED_PAIR: "direct_kernel"}.get(prec) \
-        if direct else f"steps_kernel<{opname},{form}>"
-    how = "direct FP32 solves" if direct else "FP32 Krylov" if prec != B.PIT_PREC_FP64 else "FP64 Krylov"
-    return {"bound": "hbm", "kernel": f"{kern} (d = {d}, grid-resident multi-step backward Euler, {how}"
+    common = {"traffic": (trf * steps / max(1, int(prof.launches[0]))) if trf is not None else None,
+              "traffic_note": "DRAM bytes per relaxation launch: the committed ncu summary's DRAM bytes per "
+                              "node-step times the node-steps of an average relaxation launch of the timed "
+                              "region; null when the kernel changed since the capture",
+              "time_basis_ms": relax_ms, "relax_launches": int(prof.launches[0]),
+              "relax_kernels": int(prof.kernels[0]), "sweep_ms": prof.ms[1], "sweep_launches": int(prof.launches[1]),
+              "relax_node_steps": steps, "relax_passes_per_node_step": passes / max(1, steps),
+              "relax_share_of_kernel_time": relax_ms / max(1e-9, sum(prof.ms))}
+    if wl.op == B.PIT_OP_HEAT and prec != B.PIT_PREC_FP64:
+        # (dt / h^2 of these workloads is far above the line where CG is taken)
+        kern = "fixed_kernel and direct_kernel" if prec == B.PIT_PREC_MIXED else "direct_kernel"
+        rate = lane * steps / t / 1e9 if t and lane else None
+        dram = trf * steps / t / 1e9 if t and trf else None
+        return {"bound": "issue", "kernel": f"{kern} (d = {d}, grid-resident multi-step backward Euler, direct FP32 "
+                                            "solves in iterative refinement, integer residuals without forcing)",
+                "achieved": rate, "peak": ISSUE_GLANE, "unit": "G lane instructions/s",
+                "frac": rate / ISSUE_GLANE if rate else None,
+                "lane_instructions_per_node_step": lane,
+                "peak_source": "152 SMs x 4 warp instructions a clock x 32 lanes x 2,070 MHz",
+                "direct_solves_per_node_step": iters / max(1, steps),
+                "dram": {"achieved": dram, "peak": hbm, "unit": "GB/s", "frac": dram / hbm if dram else None,
+                         "bytes_per_node_step": trf, "peak_source": hbm_src},
+                **common}
+    how = "FP32 Krylov" if prec != B.PIT_PREC_FP64 else "FP64 Krylov"
+    return {"bound": "hbm", "kernel": f"steps_kernel<{opname},{form}> (d = {d}, grid-resident multi-step backward Euler, {how}"
                                       + (")" if prec == B.PIT_PREC_FP64 else " in iterative refinement)"),
             "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": (achieved / hbm) if achieved else None,
-            "traffic": (trf * steps / max(1, int(prof.launches[0]))) if trf is not None else None,
-            "traffic_note": "DRAM bytes per relaxation launch: the committed ncu summary's DRAM bytes per "
-                            "node-step times the node-steps of an average relaxation launch of the timed "
-                            "region; null when the kernel changed since the capture",
-            "algorithmic_bytes": "40 B per node and FP32 CG iteration + 40 B per node and FP64 refinement pass"
-                                 + (" (a direct solve and an integer check count as one of each)" if direct else ""),
-            "peak_source": hbm_src,
-            "time_basis_ms": relax_ms, "relax_launches": int(prof.launches[0]),
-            "relax_kernels": int(prof.kernels[0]), "sweep_ms": prof.ms[1], "sweep_launches": int(prof.launches[1]),
-            "relax_node_steps": steps, "relax_krylov_iters_per_node_step": iters / max(1, steps),
-            "relax_passes_per_node_step": passes / max(1, steps),
-            "relax_share_of_kernel_time": relax_ms / max(1e-9, sum(prof.ms)),
-            "alu_views": views}
+            "algorithmic_bytes": "40 B per node and FP32 CG iteration + 40 B per node and FP64 refinement pass",
+            "peak_source": hbm_src, "relax_krylov_iters_per_node_step": iters / max(1, steps),
+            "alu_views": views, **common}
 
 
 def run_pit(args, rank, world, local):
@@ -540,8 +553,10 @@ def run_pit(args, rank, world, local):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "f64 (FP32 inner Krylov inside FP64 iterative refinement; FP64 residuals, MGRIT norms and "
-                 "combination; BF16-weight coarse network, rejected by its judge)",
+        "dtype": "f64 (" + ("direct FP32 correction solves inside iterative refinement, residuals in 64-bit integers "
+                            "(FP64 with forcing)" if wl.op == B.PIT_OP_HEAT else
+                            "FP32 inner Krylov inside FP64 iterative refinement, FP64 residuals") +
+                 "; FP64 MGRIT norms and combination; BF16-weight coarse network, rejected by its judge)",
         "data": "synthetic (analytic initial value, seeded evaluation points)",
         "config": {"workload": wl.name, "d": wl.d, "level": wl.n, "grids": P.G, "n_total": P.n_total,
                    "accuracy_target": "relative L2 error <= 1e-6 of the combined solution vs the oracle's "

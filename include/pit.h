@@ -166,11 +166,13 @@ typedef struct {
  *                          FP32 Krylov on A e = r to relative
  *                          max(inner_rtol, 0.5 rtol ||b|| / ||r||) (at most maxit
  *                          iterations), x += e in FP64; at most ir_maxit
- *                          passes; the same FP64 stopping rule.  (Heat operator
- *                          without forcing: the state and b - A x as 64-bit
- *                          integers of the state's scale, where the error of
- *                          that, about 2^-50 n^{1/2} max(1, sum_i dt / h_i^2),
- *                          is below a quarter of rtol.)
+ *                          passes; the same FP64 stopping rule.  (Heat operator,
+ *                          where the correction is solved directly, see
+ *                          pit_precond, without inner_rtol: without forcing
+ *                          the state and b - A x as 64-bit integers of the
+ *                          state's scale, a unit of at most 2^-52 of a grid's
+ *                          norm, where the error of that, about 2^-50 n^{1/2}
+ *                          max(1, sum_i dt / h_i^2), is below a quarter of rtol.)
  *   prec = PIT_PREC_FP32:  Krylov in FP32 on a copy of the state scaled by a
  *                          power of two (inputs and outputs stay FP64) until
  *                          the FP32 recurrence residual meets rtol; for solves
