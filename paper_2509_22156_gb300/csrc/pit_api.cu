@@ -587,8 +587,9 @@ pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_op
         slot = P->forced_threads[wide ? 1 : 0];
         return PIT_OK;
     }
-    // (one warp: grids of a few dozen nodes, whose steps are a chain of reductions
-    // that then wait for no other warp; a trial that larger grids need not pay)
+    // (below 4 KB, grids of at most 136 nodes: one warp, whose reductions wait for
+    // no other, in place of 512 threads; four trials either way, since the first
+    // call pays for them)
     const int cand[5] = {32, 64, 128, 256, 512};
     const int first = v.smem < 4096 ? 0 : 1;
     CU(P->w_tune.ensure(sizeof(double) * P->ntot * c.nb));
@@ -629,7 +630,7 @@ pit_status tune(pit_problem *P, int prec, bool wide, int cls, const pit_solve_op
     CU(cudaEventCreate(&e1));
     float best = 1e30f;
     int best_t = 128;
-    for (int k = first; k < 5; ++k) {
+    for (int k = first; k < first + 4; ++k) {
         for (int rep = 0; rep < 3; ++rep) {  // first repetition warms up; the last is timed
             CU(cudaEventRecord(e0, P->stream));
             CU(launch_steps(prec, a, cand[k], v.smem, P->stream, v.xg));
