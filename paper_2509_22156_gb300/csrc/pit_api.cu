@@ -368,7 +368,9 @@ pit_status plan(pit_problem *P, int prec)
         P->split[prec][0] = 0;
         for (int q = 0; q < NBKT; ++q) {
             P->smem_bkt[prec][q] = k < n0 ? grid_smem_bytes(P, prec, cls[0][k]) : 0;
-            if (q == NBKT - 1) k = n0;
+            // (from 2.3 KB down no CTA size or occupancy changes that a launch of its
+            // own would pay for: sixteen one-warp CTAs fill an SM's registers)
+            if (q == NBKT - 1 || P->smem_bkt[prec][q] <= P->max_smem / 96) k = n0;
             else
                 while (k < n0 && (grid_smem_bytes(P, prec, cls[0][k]) << (q + 1)) > need[0]) ++k;
             P->split[prec][q + 1] = k;
